@@ -31,6 +31,7 @@ struct sdf_net {
     uint32_t bf16_layer_bytes = 0;
     int rows_pad = 0;
     float q_w[kMaxHidden] = {}, q_g[kMaxHidden + 1] = {}, q_o = 1.0f;  // SDF_FP8 scales
+    float* d_s32 = nullptr;       // SDF_FP32 on the tensor cores: the scales of NetView::s32
 };
 
 namespace {
@@ -269,6 +270,10 @@ NetView view_of(const sdf_net* n) {
     v.wbf_layer_bytes = n->bf16_layer_bytes;
     v.rows_pad = n->rows_pad;
     v.op_f16 = n->precision == SDF_FP16 ? 1 : 0;
+    if (n->precision == SDF_FP32) {
+        v.wbf_lo = nullptr;
+        v.s32 = n->d_s32;
+    }
     if (n->precision == SDF_FP8) {
         v.op_fp8 = 1;
         v.wbf_lo = nullptr;
@@ -285,6 +290,7 @@ void free_net(sdf_net* n) {
     DeviceGuard g(n->device);
     if (n->d_f32) cudaFree(n->d_f32);
     if (n->d_bf16) cudaFree(n->d_bf16);
+    if (n->d_s32) cudaFree(n->d_s32);
     delete n;
 }
 
@@ -297,6 +303,67 @@ struct ParsedImage {
     std::vector<double> wout;
     float bout = 0.0f;
 };
+
+// FP32 operands as half-precision heads and remainders (grad32_tc.cuh), per
+// hidden layer and K block the heads and then the remainders, and the scales
+// of NetView::s32.  All scales are powers of two, so that only the operands'
+// own rounding remains: a layer's weights are scaled to a largest magnitude in
+// [2^13, 2^14); the tangents after layer l are scaled so that their bound
+// max|W_0| * prod ||W_i||_inf lies there too (the bound exceeds the tangents of
+// real networks by a few bits per layer, of the 28 that a half has below 2^14).
+// Returns false (nothing usable) when a scale would leave the range of a float:
+// such a network runs on the SIMT kernels.
+bool split_image32(const std::vector<std::vector<double>>& Wl, int IN, int W, int KH, int rows_pad,
+                   std::vector<uint8_t>* img, float* s32) {
+    auto exponent = [](double x) {  // x < 2^e
+        int e = 0;
+        if (x > 0.0) std::frexp(x, &e);
+        return e;
+    };
+    double bound = 0.0;
+    for (int i = 0; i < W; ++i)
+        for (int c = 0; c < 3; ++c)
+            bound = std::max(bound, std::fabs(static_cast<double>(static_cast<float>(Wl[0][static_cast<size_t>(i) * IN + c]))));
+    int ge = 14 - exponent(bound);
+    bool ok = std::abs(ge) <= 60;
+    s32[4 * kMaxHidden] = std::ldexp(1.0f, ge);
+    const size_t plane = static_cast<size_t>(rows_pad) * 128u, layer = 2 * plane * (W / 64);
+    img->assign(KH * layer, 0);
+    const double comp = 1.0 + kAccComp * (W / 16);
+    for (int l = 1; l <= KH; ++l) {
+        double amax = 0.0, rmax = 0.0;
+        for (int r = 0; r < W; ++r) {
+            double sum = 0.0;
+            for (int k = 0; k < W; ++k) {
+                const double x = std::fabs(static_cast<double>(static_cast<float>(Wl[l][static_cast<size_t>(r) * W + k])));
+                amax = std::max(amax, x);
+                sum += x;
+            }
+            rmax = std::max(rmax, sum);
+        }
+        const int we = 14 - exponent(amax);
+        bound *= rmax;
+        const int gn = 14 - exponent(bound);
+        ok = ok && std::isfinite(bound) && std::abs(we) <= 60 && std::abs(gn) <= 60;
+        if (!ok) return false;
+        s32[4 * (l - 1)] = static_cast<float>(std::ldexp(comp, -we));
+        s32[4 * (l - 1) + 1] = static_cast<float>(std::ldexp(comp, gn - we - ge));
+        s32[4 * (l - 1) + 2] = static_cast<float>(std::ldexp(comp, -we - ge));
+        s32[4 * (l - 1) + 3] = 0.0f;
+        ge = gn;
+        uint8_t* dst = img->data() + static_cast<size_t>(l - 1) * layer;
+        for (int r = 0; r < W; ++r)
+            for (int k = 0; k < W; ++k) {
+                const float x = std::ldexp(static_cast<float>(Wl[l][static_cast<size_t>(r) * W + k]), we);
+                const __half hi = __float2half_rn(x), lo = __float2half_rn(x - __half2float(hi));
+                const uint16_t hb = __half_as_ushort(hi), lb = __half_as_ushort(lo);
+                uint8_t* at = dst + static_cast<size_t>(k / 64) * 2 * plane + sw128_offset(r, k & 63, rows_pad);
+                std::memcpy(at, &hb, 2);
+                std::memcpy(at + plane, &lb, 2);
+            }
+    }
+    return ok;
+}
 
 // Parses and folds an SDFN image; checks the header, the size and that every
 // parameter is finite (shape support is the caller's business).
@@ -456,6 +523,15 @@ int load_from_memory(const uint8_t* buf, size_t len, int precision, int device, 
         for (int l = 0; l <= KH; ++l) n->q_g[l] = static_cast<float>(gmax[l] > 0.0 ? 64.0 / gmax[l] : 1.0);
     }
 
+    float s32[kScales32] = {};
+    bool tc32 = false;
+    if (precision == SDF_FP32) {
+        n->rows_pad = W < 128 ? 128 : W;
+        n->bf16_layer_bytes = static_cast<uint32_t>(n->rows_pad) * W * 4u;
+        tc32 = split_image32(Wl, IN, W, KH, n->rows_pad, &bf, s32);
+        if (!tc32) bf.clear();
+    }
+
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) {
         cudaGetLastError();
@@ -473,6 +549,10 @@ int load_from_memory(const uint8_t* buf, size_t len, int precision, int device, 
     if (e == cudaSuccess && !bf.empty()) {
         e = cudaMalloc(&n->d_bf16, bf.size());
         if (e == cudaSuccess) e = cudaMemcpy(n->d_bf16, bf.data(), bf.size(), cudaMemcpyHostToDevice);
+    }
+    if (e == cudaSuccess && tc32) {
+        e = cudaMalloc(&n->d_s32, sizeof(s32));
+        if (e == cudaSuccess) e = cudaMemcpy(n->d_s32, s32, sizeof(s32), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
         free_net(n);
@@ -703,7 +783,9 @@ int launch_gradients(sdf_net_t net, const float* pts, const float* pt_time, cons
     ga.normalize = normalize;
     ga.grab = &counters[0];
     ga.status = status;
-    e = (net->precision != SDF_FP32) ? launch_grad_tc(ga, num_sms, s) : launch_grad_simt(ga, num_sms, s);
+    e = net->precision != SDF_FP32 ? launch_grad_tc(ga, num_sms, s)
+        : ga.net.s32 != nullptr    ? launch_grad32_tc(ga, num_sms, s)
+                                   : launch_grad_simt(ga, num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "launching gradient kernel");
     return SDF_OK;
 }

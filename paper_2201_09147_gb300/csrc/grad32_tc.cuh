@@ -1,0 +1,407 @@
+// Analytic-gradient kernel (Alg. 2) of the FP32 path on the tensor cores,
+// shared by normal mapping and the FP32 training forward.
+//
+// Every FP32 operand is held as two half-precision values, the rounding h and
+// the rounding l of the remainder x - h: 2 x 11 significand bits and the
+// remainder's sign, so the pair misses x by at most 2^-24 of its binade, the
+// half unit of a float.  A product is h h' + l h' + h l' (l l' is below
+// 2^-24), accumulated in FP32 by three tcgen05.mma per K step.
+//
+// What decides the accuracy is the accumulation: the tensor core truncates
+// the running sum to 24 bits once per K step of 16 (measured with random
+// operands: the mean error has the sign opposite to the sum).  So h h' has its own accumulator (the
+// two small products would otherwise truncate the large sum two more times
+// per step), and the known mean of the truncation is multiplied back in
+// (kAccComp: the sums stay rounded by less than the FMA chain they replace).
+// Contractions of 128 x K sines with K x 64 uniform weights on GB300, root
+// mean square error against FP64 in units of 1e-7, for K = 64 / 128 / 256: a
+// chain of FP32 FMAs 1.8 / 3.7 / 7.2, one accumulator for all three products
+// 3.9 / 9.7 / 24.9, two accumulators 1.6 / 3.5 / 8.7, with kAccComp 1.4 / 2.4 /
+// 5.2.
+#pragma once
+
+#include "tc_common.cuh"
+
+namespace sdfnn {
+namespace {
+
+template <int W>
+struct G32 {
+    static constexpr int MT = (W + 127) / 128;      // TMEM tiles of 128 feature rows
+    static constexpr int KB = W / 64;               // 64-wide K blocks of the contraction
+    static constexpr int ROWS_PAD = MT * 128;
+    static constexpr int NH = 2 / MT;               // independent tiles of 32 points ("halves") per CTA
+    static constexpr int CS = 2;                    // threads per feature and half: each takes 32 / CS points
+    static constexpr int HPTS = 32;
+    static constexpr int CPTS = HPTS / CS;
+    static constexpr int HROWS = 4 * HPTS;          // point-streams of a half = MMA N
+    static constexpr uint32_t PLANE = W * 256u;     // bytes of one operand plane of a half (h or l)
+    // A ring unit is one plane of a K block for one TMEM tile (16 KB, consecutive in the weight image).
+    static constexpr uint32_t UNIT = 16384u;
+    static constexpr int UNITS = KB * 2 * MT;       // units per layer
+    static constexpr int NS = 6;
+    static constexpr int GROUP_WARPS = 4 * MT * CS;
+    static constexpr int GROUP_THREADS = GROUP_WARPS * 32;
+    static constexpr int EPI_WARPS = NH * GROUP_WARPS;
+    static constexpr int PRODUCER_WARP = EPI_WARPS;
+    static constexpr int MMA_WARP = EPI_WARPS + 1;
+    static constexpr int THREADS = (EPI_WARPS + 2) * 32;
+    static constexpr int TMEM_COLS = 512;           // (half or TMEM tile) * 256 + {0: h h', 128: l h' + h l'}
+};
+
+struct G32Layout {
+    uint32_t x, ring, pts, bars, misc, total;
+};
+
+template <int W>
+__host__ __device__ inline G32Layout g32_layout() {
+    using C = G32<W>;
+    G32Layout L;
+    uint32_t o = 0;
+    L.x = o;
+    o += C::NH * 2u * C::PLANE;
+    L.ring = o;
+    o += C::NS * C::UNIT;
+    L.pts = o;
+    o += C::NH * C::HPTS * 16u;
+    L.bars = o;
+    o += (2 * C::NS + 2 * C::NH) * 8u;
+    o = (o + 15u) & ~15u;
+    L.misc = o;
+    o += 32u;
+    L.total = o;
+    return L;
+}
+
+// Two points (four streams each) of one feature as 16-byte chunks of the two planes.
+__device__ __forceinline__ void store_split8(uint32_t x_s, uint32_t plane, uint32_t off, const float (&v)[8]) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) pack_split<true>(v[2 * e], v[2 * e + 1], h[e], l[e]);
+    st_shared_v4(x_s + off, h[0], h[1], h[2], h[3]);
+    st_shared_v4(x_s + plane + off, l[0], l[1], l[2], l[3]);
+}
+
+// Byte offset in a half's MN-major plane of the chunk holding points 2c, 2c + 1 for feature m.
+template <int W>
+__device__ __forceinline__ uint32_t xoff32(int m, int c) {
+    return static_cast<uint32_t>(c >> 3) * (W * 128u) + static_cast<uint32_t>(m >> 3) * 1024u +
+           static_cast<uint32_t>(m & 7) * 128u + (static_cast<uint32_t>((c & 7) ^ (m & 7)) << 4);
+}
+
+// Sum over the 32 lanes of a warp of each of v[0..15]: afterwards lane L holds,
+// in v[0], the sum of entry L / 2 (recursive halving, 16 shuffles).
+__device__ __forceinline__ void warp_sum16(float (&v)[16], int lane) {
+#pragma unroll
+    for (int s = 8; s >= 1; s >>= 1) {
+        const bool upper = (lane & (2 * s)) != 0;
+#pragma unroll
+        for (int i = 0; i < s; ++i) {
+            const float send = upper ? v[i] : v[i + s];
+            const float keep = upper ? v[i + s] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * s);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// Index of point j (j < 0: none) of half h of this CTA's set i (-1 past the work).
+template <int NH, int HPTS>
+__device__ __forceinline__ int g32_index(const GradArgs& a, long long n_work, int h, int j, int i) {
+    const long long k = ((static_cast<long long>(i) * gridDim.x + blockIdx.x) * NH + h) * HPTS + j;
+    if (j < 0 || k >= n_work) return -1;
+    return a.list ? __ldg(a.list + k) : static_cast<int>(k);
+}
+
+// Copies (x, y, z, t) of point idx into the float4 at shared address dst
+// (zeros for idx < 0); complete after cp_async_wait_all in the same thread.
+__device__ __forceinline__ void g32_point_async(uint32_t dst, const GradArgs& a, bool timed, int idx) {
+    if (idx < 0) {
+        st_shared_v4(dst, 0u, 0u, 0u, 0u);
+        return;
+    }
+    cp_async4(dst, a.pts + idx);
+    cp_async4(dst + 4u, a.pts + a.n + idx);
+    cp_async4(dst + 8u, a.pts + 2 * a.n + idx);
+    if (timed)
+        cp_async4(dst + 12u, a.pt_time + idx);
+    else
+        st_shared_u32(dst + 12u, 0u);
+}
+
+// Same skeleton as grad_tc_kernel (features as MMA rows, N = 32 points x 4
+// streams, a producer warp streaming the weights, an MMA warp, epilogue groups
+// that own a feature per thread), with these differences: operands in two
+// planes and two accumulators; at width 256 the two planes of one half fill
+// the activation memory, so the CTA runs one half of 32 points (its MMAs, 6.1 k
+// clocks a layer, and epilogue, ~2 k, take turns; two halves of 16 points
+// would stream the weights twice and read them at N = 64, where shared-memory
+// bandwidth and not the tensor pipe bounds the MMAs); two threads share a
+// feature, so 16 epilogue warps hide the sines' latency; the output layer
+// runs in FP32 on the CUDA cores (w_out times the last tangents, summed over
+// the features by a warp butterfly and, in a fixed order, over the warps).
+// The FP32 FMA units did the same products before (grad_simt_kernel, now for
+// networks beyond the scales only): a call of 20,011 points of a (256,3) 0.73
+// -> 0.14 ms, of a (128,2) 0.168 -> 0.043, of a (64,2) 0.074 -> 0.042 (the
+// last two bound by the host), the error against FP64 5 to 15 % lower on each
+// of six networks.  What bounds the (256,3) now is the alternation of MMAs
+// (6.1 k clocks a layer) and epilogue.
+template <int W>
+__global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const GradArgs a) {
+    using C = G32<W>;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t raw_s = smem_u32(smem_raw);
+    const uint32_t base_s = (raw_s + 1023u) & ~1023u;
+    uint8_t* base = smem_raw + (base_s - raw_s);
+    const NetView& net = a.net;
+    const int KH = net.n_hidden;
+    const G32Layout L = g32_layout<W>();
+    const float4* pts = reinterpret_cast<const float4*>(base + L.pts);
+    const uint32_t bar_full = base_s + L.bars;
+    const uint32_t bar_empty = bar_full + 8u * C::NS;
+    const uint32_t bar_xready = bar_empty + 8u * C::NS;
+    const uint32_t bar_dfull = bar_xready + 8u * C::NH;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + L.misc);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(base + L.misc + 4);
+    const uint32_t x_s = base_s + L.x, ring_s = base_s + L.ring;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    if (tid == 0) {
+        for (int s = 0; s < C::NS; ++s) {
+            mbar_init(bar_full + 8u * s, 1);
+            mbar_init(bar_empty + 8u * s, 1);
+        }
+        for (int h = 0; h < C::NH; ++h) {
+            mbar_init(bar_xready + 8u * h, C::GROUP_THREADS);
+            mbar_init(bar_dfull + 8u * h, 1);
+        }
+        *abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    // Static schedule: half h of CTA b takes the tiles of 32 points b * NH + h, + G * NH, ...; all halves
+    // of a CTA run the same number of tiles (one beyond the work has no valid point).
+    const long long n_work = a.list ? static_cast<long long>(*a.count) : a.n;
+    const long long n_sets = (n_work + C::NH * C::HPTS - 1) / (C::NH * C::HPTS);
+    const long long G = gridDim.x;
+    const int my_sets = static_cast<int>(n_sets > blockIdx.x ? (n_sets - blockIdx.x + G - 1) / G : 0);
+    const int n_groups = my_sets * KH;  // (tile, hidden layer) pairs of each half, in order
+    bool ok = true;
+
+    if (warp == C::PRODUCER_WARP) {
+        if (lane == 0) {
+            uint32_t g = 0;
+            int l = 0;
+            for (int k = 0; k < n_groups && ok; ++k) {
+                const uint8_t* src = net.wbf + static_cast<size_t>(l) * net.wbf_layer_bytes;
+                for (int h = 0; h < C::NH && ok; ++h)
+                    for (int u = 0; u < C::UNITS && ok; ++u, ++g) {
+                        const uint32_t stage = g % C::NS, use = g / C::NS;
+                        if (use > 0) ok = mbar_wait_bounded(bar_empty + 8u * stage, (use - 1) & 1u, a.status, abort_flag);
+                        if (!ok) break;
+                        mbar_arrive_expect_tx(bar_full + 8u * stage, C::UNIT);
+                        bulk_g2s(ring_s + stage * C::UNIT, src + u * C::UNIT, C::UNIT, bar_full + 8u * stage);
+                    }
+                l = l + 1 == KH ? 0 : l + 1;
+            }
+            // every copy issued must land before the block exits
+            for (uint32_t gg = g > C::NS ? g - C::NS : 0; gg < g; ++gg)
+                mbar_drain(bar_full + 8u * (gg % C::NS), (gg / C::NS) & 1u);
+        }
+    } else if (warp == C::MMA_WARP) {
+        if (lane == 0) {
+            constexpr uint32_t idesc_l = idesc_f32acc(128, C::HROWS, true) | kIdescMajorMnB;
+            constexpr uint32_t idesc_h = idesc_f32acc(128, 2 * C::HROWS, true) | kIdescMajorMnB;
+            uint32_t g = 0;
+            for (int k = 0; k < n_groups && ok; ++k)
+                for (int h = 0; h < C::NH && ok; ++h) {
+                    ok = mbar_wait_bounded(bar_xready + 8u * h, k & 1, a.status, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t xd0 = desc_mnmajor_sw128(x_s + h * 2u * C::PLANE, W * 128u);
+                    for (int u = 0; u < C::UNITS && ok; ++u, ++g) {
+                        const uint32_t stage = g % C::NS, use = g / C::NS;
+                        ok = mbar_wait_bounded(bar_full + 8u * stage, use & 1u, a.status, abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const int mt = C::MT == 2 ? u & 1 : 0, kb = u / (2 * C::MT);
+                        const bool rem = ((u / C::MT) & 1) != 0;
+                        const uint64_t wd0 = desc_kmajor_sw128(ring_s + stage * C::UNIT);
+                        const uint32_t d = tmem + (mt + h) * 256u;
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            const uint64_t wd = desc_add(wd0, kk * 32u);
+                            const uint64_t xd = desc_add(xd0, static_cast<uint32_t>(kb * 8 + kk * 2) * 1024u);
+                            // the heads of W times both planes of X (h h' and h l', N = 256: the planes are
+                            // adjacent, as are the accumulators); the remainders of W times the heads of X
+                            if (!rem)
+                                mma_f16kind(d, wd, xd, idesc_h, (kb | kk) != 0);
+                            else
+                                mma_f16kind(d + 128u, wd, xd, idesc_l, 1u);
+                        }
+                        mma_commit(bar_empty + 8u * stage);
+                    }
+                    if (ok) mma_commit(bar_dfull + 8u * h);
+                }
+        }
+    } else {
+        // epilogue group h: thread <-> feature m, points cs * CPTS .. of half h
+        const int h = warp / C::GROUP_WARPS, ge = warp % C::GROUP_WARPS;
+        const int mt = (ge >> 2) % C::MT, cs = (ge >> 2) / C::MT, quad = ge & 3;
+        const int m = mt * 128 + quad * 32 + lane;
+        const bool live = mt * 128 + quad * 32 < W;  // warp-uniform
+        const int gt = ge * 32 + lane;
+        const uint32_t d_s = tmem + (static_cast<uint32_t>(quad * 32) << 16) + (mt + h) * 256u + cs * (C::CPTS * 4u);
+        const uint32_t xh = x_s + h * 2u * C::PLANE;
+        const int p0 = h * C::HPTS, q0 = p0 + cs * C::CPTS;
+        // output sums of the half: one row of HROWS floats per 32 features, in the half's activation
+        // memory (free between the last MMA of a tile and the next tile's input layer)
+        float* red = reinterpret_cast<float*>(base + L.x + h * 2u * C::PLANE);
+        const bool timed = a.pt_time != nullptr && net.in_dim == 4;
+        float4 u0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float ut = 0.0f, wo = 0.0f;
+        if (live) {
+            const float* w0 = net.w0 + m * net.in_dim;
+            u0 = make_float4(__ldg(w0), __ldg(w0 + 1), __ldg(w0 + 2), __ldg(net.b0 + m));
+            const float wt = net.in_dim == 4 ? __ldg(w0 + 3) : 0.0f;
+            if (timed)
+                ut = wt;
+            else
+                u0.w = fmaf(wt, a.time, u0.w);
+            wo = __ldg(net.wout + m);
+        }
+        const float g0 = __ldg(net.s32 + 4 * kMaxHidden);
+        // Thread gt < HPTS holds the index of point gt; the next tile's index is loaded a tile ahead and its
+        // coordinates are copied during this tile's layers, so no global load sits between two tiles.
+        int idx = -1, nidx = -1;
+        if (gt < C::HPTS) {
+            nidx = g32_index<C::NH, C::HPTS>(a, n_work, h, my_sets > 0 ? gt : -1, 0);
+            g32_point_async(base_s + L.pts + static_cast<uint32_t>(p0 + gt) * 16u, a, timed, nidx);
+        }
+        uint32_t df_phase = 0;
+        for (int i = 0; i < my_sets; ++i) {
+            if (gt < C::HPTS) {
+                cp_async_wait_all();
+                idx = nidx;
+                nidx = g32_index<C::NH, C::HPTS>(a, n_work, h, i + 1 < my_sets ? gt : -1, i + 1);
+            }
+            bar_named(1 + h, C::GROUP_THREADS);
+            // input layer: P_0 = sin(A_0), G_0^c = W_0[:, c] (.) cos(A_0), the tangents at scale g0
+            if (live) {
+#pragma unroll 2
+                for (int c = 0; c < C::CPTS / 2; ++c) {
+                    float v[8];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float4 q = pts[q0 + 2 * c + e];
+                        const float z = fmaf(u0.x, q.x, fmaf(u0.y, q.y, fmaf(u0.z, q.z, fmaf(ut, q.w, u0.w))));
+                        float sn, cn;
+                        sincos_r(z, &sn, &cn);
+                        cn *= g0;
+                        v[4 * e] = sn;
+                        v[4 * e + 1] = u0.x * cn;
+                        v[4 * e + 2] = u0.y * cn;
+                        v[4 * e + 3] = u0.z * cn;
+                    }
+                    store_split8(xh, C::PLANE, xoff32<W>(m, cs * (C::CPTS / 2) + c), v);
+                }
+            }
+            fence_proxy_async_smem();
+            tc_fence_before();
+            mbar_arrive(bar_xready + 8u * h);
+
+            for (int l = 0; l < KH && ok; ++l) {
+                ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_dfull + 8u * h, df_phase, a.status, abort_flag));
+                df_phase ^= 1u;
+                if (!ok) break;
+                if (l == 0 && gt < C::HPTS)
+                    g32_point_async(base_s + L.pts + static_cast<uint32_t>(p0 + gt) * 16u, a, timed, nidx);
+                tc_fence_after();
+                if (!live) {
+                    fence_proxy_async_smem();
+                    tc_fence_before();
+                    if (l + 1 < KH) mbar_arrive(bar_xready + 8u * h);
+                    continue;
+                }
+                const bool last = l + 1 == KH;
+                const float bb = __ldg(net.bh[l] + m), mf = __ldg(net.s32 + 4 * l);
+                // the tangents' multiplier: to the scale of the next operand, or to values times w_out
+                const float mg = last ? wo * __ldg(net.s32 + 4 * l + 2) : __ldg(net.s32 + 4 * l + 1);
+#pragma unroll 1
+                for (int q = 0; q < C::CPTS / 4; ++q) {
+                    // four points: 16 columns of each accumulator
+                    float v[16], c[16];
+                    tmem_ld16(d_s + q * 16u, v);
+                    tmem_ld16(d_s + 128u + q * 16u, c);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int j = 4 * e;
+                        float sn, cn;
+                        sincos_r(fmaf(v[j] + c[j], mf, bb), &sn, &cn);
+                        cn *= mg;
+                        v[j] = sn;
+#pragma unroll
+                        for (int s = 1; s < 4; ++s) v[j + s] = cn * (v[j + s] + c[j + s]);
+                    }
+                    if (last) {
+                        warp_sum16(v, lane);
+                        if ((lane & 1) == 0) red[(mt * 4 + quad) * C::HROWS + cs * (C::CPTS * 4) + q * 16 + (lane >> 1)] = v[0];
+                    } else {
+                        const float(&lo8)[8] = *reinterpret_cast<const float(*)[8]>(&v[0]);
+                        const float(&hi8)[8] = *reinterpret_cast<const float(*)[8]>(&v[8]);
+                        store_split8(xh, C::PLANE, xoff32<W>(m, cs * (C::CPTS / 2) + 2 * q), lo8);
+                        store_split8(xh, C::PLANE, xoff32<W>(m, cs * (C::CPTS / 2) + 2 * q + 1), hi8);
+                    }
+                }
+                fence_proxy_async_smem();
+                tc_fence_before();
+                if (!last) mbar_arrive(bar_xready + 8u * h);
+            }
+            // one decision for the group; the output rows of red are complete
+            if (bar_or(1 + h, C::GROUP_THREADS, !ok || *abort_flag != 0)) break;
+            if (gt < C::HPTS) {
+                if (idx >= 0) {
+                    float gx = 0.0f, gy = 0.0f, gz = 0.0f;
+#pragma unroll
+                    for (int r = 0; r < W / 32; ++r) {
+                        const float4 t = *reinterpret_cast<const float4*>(red + r * C::HROWS + gt * 4);
+                        gx += t.y;
+                        gy += t.z;
+                        gz += t.w;
+                    }
+                    if (a.normalize) {
+                        const float len = sqrtf(gx * gx + gy * gy + gz * gz);
+                        const float inv = len >= 1e-12f ? 1.0f / len : 0.0f;
+                        gx *= inv;
+                        gy *= inv;
+                        gz *= inv;
+                    }
+                    a.out[idx] = gx;
+                    a.out[a.n + idx] = gy;
+                    a.out[2 * a.n + idx] = gz;
+                }
+            }
+            // the barrier at the top of the next tile orders these reads of red before its input layer
+        }
+        if (gt < C::HPTS) cp_async_wait_all();
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc(tmem, C::TMEM_COLS);
+    }
+}
+
+}  // namespace
+}  // namespace sdfnn

@@ -8,6 +8,11 @@ namespace sdfnn {
 
 constexpr int kMaxHidden = 4;
 constexpr int kMaxLevels = 8;
+constexpr int kScales32 = 4 * kMaxHidden + 1;  // floats at NetView::s32
+
+// Mean relative truncation of the tensor core's FP32 accumulation (see
+// grad32_tc.cuh): each K step of 16 takes about kAccComp of the final sum.
+constexpr double kAccComp = 0.14 * 0x1p-23;
 
 // Device view of one prepared network (all pointers are device memory).
 struct NetView {
@@ -32,6 +37,12 @@ struct NetView {
     float q_g[kMaxHidden + 1];
     float q_o;
     const uint8_t* wout_q;
+    // FP32 networks on the tensor cores (s32 != NULL): wbf holds, per hidden layer and 64-wide K block, the
+    // half-precision heads and then the remainders of W_l * 2^w_l (each rows_pad x 128 bytes, 128-byte
+    // swizzle).  s32, device memory: [4 l] the multiplier from a layer-l accumulator to A, [4 l + 1] from a
+    // tangent accumulator to the tangent operand of layer l + 1, [4 l + 2] to W_l G_{l-1}; [4 kMaxHidden] the
+    // scale of the input layer's tangents.
+    const float* s32;
 };
 
 // The per-unit FP32 parameters of a width-64 network that the trace kernel
@@ -108,6 +119,7 @@ cudaError_t launch_trace_level_simt(const LevelArgs& a, int num_sms, cudaStream_
 cudaError_t launch_grad_simt(const GradArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_trace_level_tc(const LevelArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_grad_tc(const GradArgs& a, int num_sms, cudaStream_t s);
+cudaError_t launch_grad32_tc(const GradArgs& a, int num_sms, cudaStream_t s);  // FP32 networks with s32
 int trace_tiles_max(const NetView& net);  // largest `tiles` the tensor-core trace kernel accepts for net
 bool tc_trace_supported(int width, int n_hidden);
 // Measured throughput of the tensor-core kernels' sine on all SMs (sines per second).

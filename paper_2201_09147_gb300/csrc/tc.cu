@@ -102,20 +102,7 @@ __host__ __device__ inline uint32_t tmem_cols_for(int cols) {
     return n;
 }
 
-// 16-bit head and remainder of two floats, packed as pairs (the two
-// remainders in one packed FP32 operation: a - head(a) by an FMA with -1,
-// which is exact in the product, so each lane is the rounded difference).
-template <bool F16>
-__device__ __forceinline__ void pack_split(float a, float b, uint32_t& hi, uint32_t& lo) {
-    hi = pack16x2<F16>(a, b);
-    const float2 h = make_float2(from16<F16>(static_cast<uint16_t>(hi & 0xFFFFu)),
-                                 from16<F16>(static_cast<uint16_t>(hi >> 16)));
-    const float2 r = __ffma2_rn(h, make_float2(-1.0f, -1.0f), make_float2(a, b));
-    lo = pack16x2<F16>(r.x, r.y);
-}
-
-
-// The same parameters laid out for packed FP32 arithmetic on unit pairs
+// Layer-0 parameters laid out for packed FP32 arithmetic on unit pairs
 // (trace kernels): pair p = units 2p, 2p+1 as two float4s,
 // (w_x0, w_x1, w_y0, w_y1) and (w_z0, w_z1, b0, b1); w_t per unit as before.
 __device__ __forceinline__ void stage_layer0_pairs(const NetView& net, float time, bool timed, int i, float* w0s,

@@ -17,6 +17,18 @@ namespace {
 enum : int { kOpBF16 = 0, kOpF16 = 1, kOpE4M3 = 2 };
 constexpr float kFp8ActScale = 256.0f;
 
+// 16-bit head and remainder of two floats, packed as pairs (the two
+// remainders in one packed FP32 operation: a - head(a) by an FMA with -1,
+// which is exact in the product, so each lane is the rounded difference).
+template <bool F16>
+__device__ __forceinline__ void pack_split(float a, float b, uint32_t& hi, uint32_t& lo) {
+    hi = pack16x2<F16>(a, b);
+    const float2 h = make_float2(from16<F16>(static_cast<uint16_t>(hi & 0xFFFFu)),
+                                 from16<F16>(static_cast<uint16_t>(hi >> 16)));
+    const float2 r = __ffma2_rn(h, make_float2(-1.0f, -1.0f), make_float2(a, b));
+    lo = pack16x2<F16>(r.x, r.y);
+}
+
 // Layer-0 parameters in shared memory: (w_x, w_y, w_z, b) per unit as a
 // float4, and the time column w_t apart.  With per-ray times (TIMED) b is
 // the plain bias and each ray adds w_t * t_ray; otherwise the launch's
