@@ -752,6 +752,13 @@ int validate_grad(sdf_net_t net, const float* pts, const float* pt_time, const u
     return SDF_OK;
 }
 
+// The counters and the list are only used with a mask (the compaction) and by the SIMT kernel (its work
+// counter): other calls need no scratch and no memset before the kernel (of a call on a few points, a
+// tenth of its time).
+bool grad_needs_scratch(const sdf_net* net, bool mask) {
+    return mask || (net->precision == SDF_FP32 && net->d_s32 == nullptr);
+}
+
 // Bytes of gradient scratch: 4 counters, then a list of n indices with a mask.
 size_t grad_scratch_bytes(int64_t n, bool mask) {
     return 4 * sizeof(unsigned long long) + (mask ? static_cast<size_t>(n) * sizeof(int32_t) : 0);
@@ -763,7 +770,8 @@ int launch_gradients(sdf_net_t net, const float* pts, const float* pt_time, cons
                      int normalize, void* scratch, int* status, int num_sms, cudaStream_t s,
                      bool zero_unmasked = true) {
     const size_t counter_bytes = 4 * sizeof(unsigned long long);
-    cudaError_t e = cudaMemsetAsync(scratch, 0, counter_bytes, s);
+    cudaError_t e = cudaSuccess;
+    if (grad_needs_scratch(net, mask != nullptr)) e = cudaMemsetAsync(scratch, 0, counter_bytes, s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(counters)");
     auto* counters = static_cast<unsigned long long*>(scratch);
     int32_t* list = mask ? reinterpret_cast<int32_t*>(static_cast<uint8_t*>(scratch) + counter_bytes) : nullptr;
@@ -801,8 +809,10 @@ int grad_impl(sdf_net_t net, const float* pts, const float* pt_time, const uint8
     if ((rc = device_info(net->device, &di))) return rc;
     Scratch sc;
     sc.s = s;
-    cudaError_t e = cudaMallocFromPoolAsync(&sc.ptr, grad_scratch_bytes(n, mask != nullptr) + 256, di.pool, s);
-    if (e != cudaSuccess) return cuda_fail(e, "allocating scratch");
+    if (grad_needs_scratch(net, mask != nullptr)) {
+        const cudaError_t e = cudaMallocFromPoolAsync(&sc.ptr, grad_scratch_bytes(n, mask != nullptr) + 256, di.pool, s);
+        if (e != cudaSuccess) return cuda_fail(e, "allocating scratch");
+    }
     return launch_gradients(net, pts, pt_time, mask, n, out, normalize, sc.ptr, di.d_status, di.num_sms, s);
 }
 

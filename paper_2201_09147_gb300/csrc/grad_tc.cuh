@@ -168,12 +168,12 @@ __device__ __forceinline__ void mma_op(uint32_t d, uint64_t a, uint64_t b, uint3
         mma_f16kind(d, a, b, idesc, acc);
 }
 
-// Index of point j (j < 0: none) of half h of pair i of this CTA (-1 past the
-// work), and its coordinates (zero for -1).
-template <int HPTS>
-__device__ __forceinline__ int grad_point_index(const GradArgs& a, long long n_work, int cta, int h, int j,
+// Index of point j (j < 0: none) of half h of this CTA's pair i, or with ONE
+// (halves = 1) of its i-th half-tile (-1 past the work).
+template <int HPTS, bool ONE>
+__device__ __forceinline__ int grad_point_index(const GradArgs& a, long long n_work, int halves, int cta, int h, int j,
                                                 long long i) {
-    const long long k = ((i * gridDim.x + cta) * 2 + h) * HPTS + j;
+    const long long k = ((i * gridDim.x + cta) * (ONE ? halves : 2) + h) * HPTS + j;
     if (j < 0 || k >= n_work) return -1;
     return a.list ? a.list[k] : static_cast<int>(k);
 }
@@ -181,10 +181,10 @@ __device__ __forceinline__ int grad_point_index(const GradArgs& a, long long n_w
 // The same index written to the int at shared address dst: copied there
 // asynchronously when it comes from the list (complete after
 // cp_async_wait_all in the same thread).
-template <int HPTS>
-__device__ __forceinline__ void grad_point_index_async(uint32_t dst, const GradArgs& a, long long n_work, int cta,
-                                                       int h, int j, long long i) {
-    const long long k = ((i * gridDim.x + cta) * 2 + h) * HPTS + j;
+template <int HPTS, bool ONE>
+__device__ __forceinline__ void grad_point_index_async(uint32_t dst, const GradArgs& a, long long n_work, int halves,
+                                                       int cta, int h, int j, long long i) {
+    const long long k = ((i * gridDim.x + cta) * (ONE ? halves : 2) + h) * HPTS + j;
     if (j < 0 || k >= n_work)
         st_shared_u32(dst, 0xFFFFFFFFu);
     else if (a.list)
@@ -314,10 +314,16 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
     // b + 2G, ... (G = grid size) and half h of each pair is half-tile
     // 2 * pair + h.  Both halves run the same number of pairs, so the MMA warp
     // and the producer can follow the fixed schedule of grad_slot; a half-tile
-    // beyond the work is computed with no valid points.
+    // beyond the work is computed with no valid points.  Work of at most one
+    // half-tile per CTA is spread instead, a half-tile for each CTA's half 0:
+    // half 1 would take turns with it for the weights and the tensor core.  A
+    // call of 300 points of a (256,3), FP16: 22.8 us (5 CTAs streaming 768 KB of
+    // weights each) -> 14.4 us (10 CTAs, 384 KB, and no memset before the kernel).
     const long long n_work = a.list ? static_cast<long long>(*a.count) : a.n;
-    const long long n_pairs = (n_work + 2 * C::HPTS - 1) / (2 * C::HPTS);
     const long long G = gridDim.x;
+    constexpr bool kOne = !FP8;  // E4M3: the choice cost a large call 2.5 %
+    const int halves = kOne && n_work <= G * C::HPTS ? 1 : 2;
+    const long long n_pairs = (n_work + halves * C::HPTS - 1) / (halves * C::HPTS);
     const long long my_pairs = n_pairs > blockIdx.x ? (n_pairs - blockIdx.x + G - 1) / G : 0;
     // MMA schedule: each half runs n_groups groups in order (per pair: the KH
     // hidden layers, then the output layer).  With 16-bit operands half 1 runs
@@ -332,6 +338,7 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
     // groups per pair: the hidden layers, and the output layer unless TRAIN computes it in FP32
     const int GPP = TRAIN ? KH : KH + 1;
     const int n_groups = static_cast<int>(my_pairs) * GPP;
+    const int n_groups1 = halves == 2 ? n_groups : 0;  // of half 1
     bool ok = true;
 
     if (warp == C::PRODUCER_WARP) {
@@ -344,7 +351,7 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int grp = k - h * LAG;
-                    if (grp < 0 || grp >= n_groups) continue;
+                    if (grp < 0 || grp >= (kOne && h == 1 ? n_groups1 : n_groups)) continue;
                     const int l = lh[h];
                     lh[h] = l + 1 == GPP ? 0 : l + 1;
                     for (int sg = 0; sg < C::STAGES_PER_LAYER && l < KH && ok; ++sg, ++g) {
@@ -374,7 +381,7 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
 #pragma unroll
                 for (int h = 0; h < 2 && ok; ++h) {
                     const int grp = k - h * LAG;
-                    if (grp < 0 || grp >= n_groups) continue;
+                    if (grp < 0 || grp >= (kOne && h == 1 ? n_groups1 : n_groups)) continue;
                     const int l = lh[h];
                     lh[h] = l + 1 == GPP ? 0 : l + 1;
                     ok = mbar_wait_bounded(bar_xready + 8u * h, xr_phase[h], a.status, abort_flag);
@@ -437,24 +444,22 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
         const float g0s = FP8 ? net.q_g[0] : 1.0f;
         const float wo = TRAIN && live ? __ldg(net.wout + m) : 0.0f;  // w_out of this feature (TRAIN)
         uint32_t df_phase = 0;
-        // Point gt of this half in pair i (threads gt < HPTS): its index is
-        // loaded a pair ahead and its coordinates during the pair before, so
-        // neither global load sits between two pairs.
+        const long long pairs_h = kOne && h >= halves ? 0 : my_pairs;
         // Point gt < HPTS of this half: its index is copied into shared memory
         // at the start of the pair before, its coordinates once that pair's
         // input layer has read the current ones, so no global load sits
         // between two pairs.
         if (gt < C::HPTS) {
-            const int idx = grad_point_index<C::HPTS>(a, n_work, blockIdx.x, h, my_pairs > 0 ? gt : -1, 0);
+            const int idx = grad_point_index<C::HPTS, kOne>(a, n_work, halves, blockIdx.x, h, pairs_h > 0 ? gt : -1, 0);
             nidxs[p0 + gt] = idx;
             grad_point_async(base_s + L.pts + static_cast<uint32_t>(p0 + gt) * 16u, a, timed, idx);
         }
-        for (long long i = 0; i < my_pairs; ++i) {
+        for (long long i = 0; i < pairs_h; ++i) {
             if (gt < C::HPTS) {
                 cp_async_wait_all();
                 idxs[p0 + gt] = nidxs[p0 + gt];
-                grad_point_index_async<C::HPTS>(base_s + L.nidx + static_cast<uint32_t>(p0 + gt) * 4u, a, n_work,
-                                                blockIdx.x, h, i + 1 < my_pairs ? gt : -1, i + 1);
+                grad_point_index_async<C::HPTS, kOne>(base_s + L.nidx + static_cast<uint32_t>(p0 + gt) * 4u, a, n_work,
+                                                halves, blockIdx.x, h, i + 1 < pairs_h ? gt : -1, i + 1);
             }
             bar_named(1 + h, C::GROUP_THREADS);
             // input layer: P_0 = sin(A_0), G_0^c = W_0[:, c] (.) cos(A_0); the time
