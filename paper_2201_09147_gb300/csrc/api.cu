@@ -753,8 +753,7 @@ int validate_grad(sdf_net_t net, const float* pts, const float* pt_time, const u
 }
 
 // The counters and the list are only used with a mask (the compaction) and by the SIMT kernel (its work
-// counter): other calls need no scratch and no memset before the kernel (of a call on a few points, a
-// tenth of its time).
+// counter): other calls need no scratch and no memset before the kernel.
 bool grad_needs_scratch(const sdf_net* net, bool mask) {
     return mask || (net->precision == SDF_FP32 && net->d_s32 == nullptr);
 }
@@ -948,7 +947,10 @@ int plan_autotune(sdf_plan* p, int* status, int num_sms, cudaStream_t s) {
     for (int j = 0; j < p->n_levels && rc == SDF_OK; ++j) {
         const sdf_net* net = p->nets[j];
         const int tmax = net->precision == SDF_FP32 ? 0 : trace_tiles_max(view_of(net));
-        if (tmax <= 1) continue;
+        if (tmax <= 1) {
+            p->tiles[j] = tmax;  // one launch shape (0: FP32)
+            continue;
+        }
         float best = INFINITY;
         int best_t = tmax;
         for (int t = 1; t <= tmax && rc == SDF_OK; ++t) {

@@ -118,6 +118,7 @@ struct GradArgs {
 cudaError_t launch_trace_level_simt(const LevelArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_grad_simt(const GradArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_trace_level_tc(const LevelArgs& a, int num_sms, cudaStream_t s);
+cudaError_t launch_trace_wide(const LevelArgs& a, int num_sms, cudaStream_t s);  // trace_wide.cuh
 cudaError_t launch_grad_tc(const GradArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_grad32_tc(const GradArgs& a, int num_sms, cudaStream_t s);  // FP32 networks with s32
 int trace_tiles_max(const NetView& net);  // largest `tiles` the tensor-core trace kernel accepts for net

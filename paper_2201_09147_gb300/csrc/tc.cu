@@ -15,8 +15,8 @@
 //   output layer is an FP32 dot product of the last sine layer straight from
 //   TMEM, so the step t = f - d is never rounded to 16 bits.  Once the work
 //   list is empty the CTA regroups its remaining rays into its first tiles
-//   every few iterations.  Width 256 (trace_level_tc_stream): two tiles share
-//   hidden weights streamed through a ring of bulk-copied stages.
+//   every few iterations.  Widths 128 (head + remainder) and 256, and small
+//   calls of width 64, run trace_wide_kernel (trace_wide.cuh).
 //
 // grad_tc : analytic gradients (Alg. 2).  Tiles of 64 points in two halves;
 //   the MMA runs with the features as rows (M = 128 per TMEM tile,
@@ -87,6 +87,11 @@ __host__ __device__ inline TraceLayout trace_layout(int W, int KH, bool split, i
 constexpr uint32_t kSplitSmemLimit = 200u * 1024u;
 constexpr int kTailRound = 4;  // trace iterations between two regroupings of the tail's rays
 constexpr int kMaxTraceTiles = 6;
+// Width 64: calls of at most this many rays per SM run trace_wide_kernel (two
+// rounds of its 128 slots).  The two kernels' times at 139^2 / 196^2 / 240^2 rays
+// on 152 SMs, in us: (64,1) Lipschitz steps 82 / 156 / 227 against 196 / 211 /
+// 211, (64,1) coarse trace 99 / 120 / 139 against 119 / 122 / 124.
+constexpr int kWideRays = 256;
 constexpr int kTraceMaxThreads = 128 * kMaxTraceTiles;
 
 // The trace kernel's tensor pipe is mostly idle (its time goes to the sines),
@@ -100,22 +105,6 @@ __host__ __device__ inline uint32_t tmem_cols_for(int cols) {
     uint32_t n = 32;
     while (n < static_cast<uint32_t>(cols)) n <<= 1;
     return n;
-}
-
-// Layer-0 parameters laid out for packed FP32 arithmetic on unit pairs
-// (trace kernels): pair p = units 2p, 2p+1 as two float4s,
-// (w_x0, w_x1, w_y0, w_y1) and (w_z0, w_z1, b0, b1); w_t per unit as before.
-__device__ __forceinline__ void stage_layer0_pairs(const NetView& net, float time, bool timed, int i, float* w0s,
-                                                   float* wts) {
-    const int p = i >> 1, e = i & 1;
-    float bb = net.b0[i];
-    const float wt = net.in_dim == 4 ? net.w0[i * 4 + 3] : 0.0f;
-    if (!timed) bb = fmaf(wt, time, bb);
-    w0s[p * 8 + e] = net.w0[i * net.in_dim + 0];
-    w0s[p * 8 + 2 + e] = net.w0[i * net.in_dim + 1];
-    w0s[p * 8 + 4 + e] = net.w0[i * net.in_dim + 2];
-    w0s[p * 8 + 6 + e] = bb;
-    wts[i] = timed ? wt : 0.0f;
 }
 
 // Layer 0 (FP32) of one ray row: X[row] = 16-bit sin(W_0 (p, t) + b_0),
@@ -156,27 +145,19 @@ __device__ __forceinline__ void trace_layer0(const LevelArgs& a, const float4* w
 // Output layer of one ray row from N of its TMEM accumulator columns:
 // acc += w_out . sin(D + b), the bias additions and the products on unit
 // pairs (two packed accumulators, for units 4j, 4j+1 and 4j+2, 4j+3).
-template <int N, bool SCALED = false>
+template <int N>
 __device__ __forceinline__ void output_dot(const float (&v)[N], const float* bl, const float* wo, float2& acc01,
-                                           float2& acc23, float sc = 1.0f) {
-    const float2 sc2 = make_float2(sc, sc);
+                                           float2& acc23) {
 #pragma unroll
     for (int j4 = 0; j4 < N / 4; ++j4) {
         const float4 b4 = reinterpret_cast<const float4*>(bl)[j4];
         const float4 w4 = reinterpret_cast<const float4*>(wo)[j4];
         const float2 v01 = make_float2(v[4 * j4 + 0], v[4 * j4 + 1]), v23 = make_float2(v[4 * j4 + 2], v[4 * j4 + 3]);
-        // SCALED (E4M3 operands): the accumulator times the inverse of the operand scales
-        const float2 x01 = SCALED ? __ffma2_rn(v01, sc2, make_float2(b4.x, b4.y)) : __fadd2_rn(v01, make_float2(b4.x, b4.y));
-        const float2 x23 = SCALED ? __ffma2_rn(v23, sc2, make_float2(b4.z, b4.w)) : __fadd2_rn(v23, make_float2(b4.z, b4.w));
+        const float2 x01 = __fadd2_rn(v01, make_float2(b4.x, b4.y));
+        const float2 x23 = __fadd2_rn(v23, make_float2(b4.z, b4.w));
         acc01 = __ffma2_rn(make_float2(w4.x, w4.y), make_float2(sin_fast(x01.x), sin_fast(x01.y)), acc01);
         acc23 = __ffma2_rn(make_float2(w4.z, w4.w), make_float2(sin_fast(x23.x), sin_fast(x23.y)), acc23);
     }
-}
-
-template <bool SCALED = false>
-__device__ __forceinline__ void output_dot32(const float (&v)[32], const float* bl, const float* wo, float2& acc01,
-                                             float2& acc23, float sc = 1.0f) {
-    output_dot<32, SCALED>(v, bl, wo, acc01, acc23, sc);
 }
 
 // Hidden epilogue of one ray row for N columns from c0 (N a multiple of 8):
@@ -206,12 +187,6 @@ __device__ __forceinline__ void hidden_epilogue(const float (&v)[N], const float
         st_shared_v4(x_s + off, pk[0], pk[1], pk[2], pk[3]);
         if (SPLIT) st_shared_v4(xlo_s + off, pl[0], pl[1], pl[2], pl[3]);
     }
-}
-
-template <bool F16, bool SPLIT>
-__device__ __forceinline__ void hidden_epilogue32(const float (&v)[32], const float* bl, int row, int c0,
-                                                  uint32_t x_s, uint32_t xlo_s) {
-    hidden_epilogue<32, F16, SPLIT>(v, bl, row, c0, x_s, xlo_s);
 }
 
 // T = blockDim.x / 128 independent ray tiles per CTA.  Tile t owns warps
@@ -462,322 +437,6 @@ __global__ void __launch_bounds__(kTraceMaxThreads, 1) trace_level_tc_kernel(con
     }
 }
 
-// Layer 0 of one ray row as E4M3 bytes of 256 sin(W_0 (p, t) + b_0): K-major
-// rows of 128-element blocks with the 128-byte swizzle, one 16-byte chunk
-// (16 units) per vector store; the units in pairs as in trace_layer0.
-template <int W, bool TIMED>
-__device__ __forceinline__ void trace_layer0_e4m3(const LevelArgs& a, const float* w0s, const float* wts,
-                                                  const Ray& ray, int row, uint32_t x_s) {
-    const float tm = (TIMED && ray.state == kSlotActive) ? __ldg(a.ray_time + ray.idx) : 0.0f;
-    const float2 px = make_float2(ray.px, ray.px), py = make_float2(ray.py, ray.py), pz = make_float2(ray.pz, ray.pz);
-    const float2 t2 = make_float2(tm, tm);
-    for (int j16 = 0; j16 < W / 16; ++j16) {
-        float sv[16];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int pr = j16 * 8 + q;
-            const float4 A = reinterpret_cast<const float4*>(w0s)[2 * pr];
-            const float4 B = reinterpret_cast<const float4*>(w0s)[2 * pr + 1];
-            float2 c = make_float2(B.z, B.w);
-            if (TIMED) c = __ffma2_rn(reinterpret_cast<const float2*>(wts)[pr], t2, c);
-            const float2 z = __ffma2_rn(make_float2(A.x, A.y), px,
-                                        __ffma2_rn(make_float2(A.z, A.w), py, __ffma2_rn(make_float2(B.x, B.y), pz, c)));
-            sv[2 * q] = kFp8ActScale * sin_fast(z.x);
-            sv[2 * q + 1] = kFp8ActScale * sin_fast(z.y);
-        }
-        st_shared_v4(x_s + sw128_chunk_offset(row, j16, 128), pack_e4m3x4(sv[0], sv[1], sv[2], sv[3]),
-                     pack_e4m3x4(sv[4], sv[5], sv[6], sv[7]), pack_e4m3x4(sv[8], sv[9], sv[10], sv[11]),
-                     pack_e4m3x4(sv[12], sv[13], sv[14], sv[15]));
-    }
-}
-
-// Hidden epilogue of one ray row for accumulator columns c0 .. c0+31 with
-// E4M3 operands: X = E4M3(256 sin(D * mf + b)), two 16-byte chunks.
-__device__ __forceinline__ void hidden_epilogue32_e4m3(const float (&v)[32], const float* bl, float mf, int row,
-                                                       int c0, uint32_t x_s) {
-    const float2 mf2 = make_float2(mf, mf);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        float sv[16];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int j = h * 16 + 2 * e;
-            const float2 x = __ffma2_rn(make_float2(v[j], v[j + 1]), mf2, make_float2(bl[c0 + j], bl[c0 + j + 1]));
-            sv[2 * e] = kFp8ActScale * sin_fast(x.x);
-            sv[2 * e + 1] = kFp8ActScale * sin_fast(x.y);
-        }
-        st_shared_v4(x_s + sw128_chunk_offset(row, (c0 >> 4) + h, 128), pack_e4m3x4(sv[0], sv[1], sv[2], sv[3]),
-                     pack_e4m3x4(sv[4], sv[5], sv[6], sv[7]), pack_e4m3x4(sv[8], sv[9], sv[10], sv[11]),
-                     pack_e4m3x4(sv[12], sv[13], sv[14], sv[15]));
-    }
-}
-
-// ---------------------------------------------------------------------------
-// trace kernel, width 256 with streamed weights
-// ---------------------------------------------------------------------------
-// Same per-ray structure as trace_level_tc_kernel, for width 256, whose
-// hidden weights (128 KB per layer) leave no room for a second tile of
-// activations when held in shared memory.  A producer warp streams the 64-wide K blocks of every
-// hidden layer (256 rows x 128 bytes = 32 KB) from L2 through a ring in the
-// order the MMAs consume them, cycling over the layers for as long as rays
-// remain; thread 0 issues the MMAs as stages arrive.  ST ray tiles of 128
-// (TMEM columns [t*256, (t+1)*256), 64 KB of activations each) share every
-// weight stage: with two tiles each streamed byte serves twice the rays and
-// eight warps instead of four overlap their layer-0 and epilogue work.
-constexpr int kStreamW = 256;
-constexpr uint32_t kStreamStageBytes = kStreamW * 128u;
-__host__ __device__ constexpr int stream_stages(int ST) { return ST == 1 ? 3 : 2; }
-__host__ __device__ constexpr int stream_threads(int ST) { return 128 * ST + 32; }  // ray threads + producer warp
-
-struct StreamLayout {
-    uint32_t x, ring, w0, wt, bh, wout, bars, misc, total;
-};
-
-__host__ __device__ inline StreamLayout stream_layout(int KH, int ST, int EB) {
-    StreamLayout L;
-    uint32_t o = 0;
-    L.x = o;
-    o += static_cast<uint32_t>(ST) * 128u * kStreamW * static_cast<uint32_t>(EB);
-    L.ring = o;
-    o += stream_stages(ST) * kStreamStageBytes;
-    L.w0 = o;
-    o += kStreamW * 4u * 4u;
-    L.wt = o;
-    o += kStreamW * 4u;
-    L.bh = o;
-    o += static_cast<uint32_t>(KH) * kStreamW * 4u;
-    L.wout = o;
-    o += kStreamW * 4u;
-    L.bars = o;
-    o += (2 * stream_stages(ST) + 1) * 8u;
-    o = (o + 15u) & ~15u;
-    L.misc = o;
-    o += 32u;
-    L.total = o;
-    return L;
-}
-
-template <int OP, int ST>
-__global__ void __launch_bounds__(stream_threads(ST)) trace_level_tc_stream_kernel(const LevelArgs a) {
-    constexpr bool F16 = OP == kOpF16, FP8 = OP == kOpE4M3;
-    constexpr int EB = FP8 ? 1 : 2;  // operand bytes per element
-    // 128-byte K blocks per layer; a stage is one K block of all 256 rows (32 KB)
-    constexpr int W = kStreamW, KB = W * EB / 128, NS = stream_stages(ST), NRAY = 128 * ST;
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
-    const uint32_t raw_s = smem_u32(smem_raw);
-    const uint32_t base_s = (raw_s + 1023u) & ~1023u;
-    uint8_t* base = smem_raw + (base_s - raw_s);
-    const NetView& net = a.net;
-    const int KH = net.n_hidden;
-    const StreamLayout L = stream_layout(KH, ST, EB);
-    float* w0s = reinterpret_cast<float*>(base + L.w0);
-    float* wts = reinterpret_cast<float*>(base + L.wt);
-    float* bhs = reinterpret_cast<float*>(base + L.bh);
-    float* wos = reinterpret_cast<float*>(base + L.wout);
-    const uint32_t bar_full = base_s + L.bars, bar_empty = bar_full + 8u * NS, bar_mma = bar_empty + 8u * NS;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + L.misc);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(base + L.misc + 4);
-    volatile int* done_flag = reinterpret_cast<volatile int*>(base + L.misc + 8);
-    volatile uint32_t* consumed = reinterpret_cast<volatile uint32_t*>(base + L.misc + 12);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tile = tid >> 7, ttid = tid & 127;
-    constexpr uint32_t xbytes = 128u * W * EB;
-    const uint32_t x_s = base_s + L.x + static_cast<uint32_t>(tile < ST ? tile : 0) * xbytes;
-    const uint32_t ring_s = base_s + L.ring;
-
-    if (tid == 0) {
-        for (int s = 0; s < NS; ++s) {
-            mbar_init(bar_full + 8u * s, 1);
-            mbar_init(bar_empty + 8u * s, 1);
-        }
-        mbar_init(bar_mma, 1);
-        *abort_flag = 0;
-        *done_flag = 0;
-        *consumed = 0;
-        fence_mbar_init();
-    }
-    if (warp == 0) {
-        tmem_alloc(smem_u32(tmem_slot), W * ST);
-        tmem_relinquish();
-    }
-    const bool timed = a.ray_time != nullptr && net.in_dim == 4;
-    for (int i = tid; i < W; i += stream_threads(ST)) {
-        stage_layer0_pairs(net, a.time, timed, i, w0s, wts);
-        wos[i] = net.wout[i];
-        for (int l = 0; l < KH; ++l) bhs[l * W + i] = net.bh[l][i];
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem0 = *tmem_slot;
-
-    if (warp == 4 * ST) {
-        // producer: K blocks of layer 0..KH-1 in consumption order, cyclically
-        if (lane == 0) {
-            uint32_t g = 0;
-            bool ok = true;
-            while (ok) {
-                const uint32_t stage = g % NS, use = g / NS;
-                if (use > 0) {
-                    const uint32_t bar = bar_empty + 8u * stage, par = (use - 1) & 1u;
-                    const uint64_t t0 = globaltimer_ns();
-                    bool got = false;
-                    while (!(got = mbar_try_wait(bar, par))) {
-                        if (*done_flag || *abort_flag) break;
-                        if (globaltimer_ns() - t0 > kWaitBudgetNs) {
-                            raise_status(a.status, kStatusTimeout);
-                            *abort_flag = 1;
-                            break;
-                        }
-                    }
-                    if (!got) break;
-                }
-                const uint32_t l = (g / KB) % KH, kb = g % KB;
-                mbar_arrive_expect_tx(bar_full + 8u * stage, kStreamStageBytes);
-                bulk_g2s(ring_s + stage * kStreamStageBytes,
-                         net.wbf + static_cast<size_t>(l) * net.wbf_layer_bytes +
-                             static_cast<size_t>(kb) * net.rows_pad * 128u,
-                         kStreamStageBytes, bar_full + 8u * stage);
-                ++g;
-            }
-            // every copy issued must land before the block exits
-            for (uint32_t gg = *consumed; gg < g; ++gg) mbar_drain(bar_full + 8u * (gg % NS), (gg / NS) & 1u);
-        }
-    } else {
-        const long long n_work = a.in_list ? static_cast<long long>(*a.in_count) : a.n;
-        const uint32_t lane_base = static_cast<uint32_t>((ttid >> 5) * 32) << 16;
-        const uint32_t tmem = tmem0 + static_cast<uint32_t>(tile * W);
-        // E4M3: the format fields 0 of this descriptor select E4M3 under kind::f8f6f4
-        constexpr uint32_t idesc = idesc_f32acc(128, W, F16 || FP8);
-        const uint64_t rd0 = desc_kmajor_sw128(ring_s);
-        uint32_t mma_phase = 0, g = 0;
-        bool issue_ok = true;  // thread 0: every weight stage so far arrived in time
-        Ray ray;
-        // Stop decisions go through the ray threads' barrier: a timed-out wait
-        // drops the ray (the status word reports it) instead of leaving the loop.
-        while (true) {
-            refill_ray(a, ray, n_work);
-            if (a.cap <= 0) {
-                if (!bar_or(1, NRAY, ray.state == kSlotActive)) break;
-                pass_ray(a, ray);
-                continue;
-            }
-            // a warp with no active slot skips its rows (as in trace_level_tc_kernel)
-            const bool wact = __any_sync(0xffffffffu, ray.state == kSlotActive);
-            if (wact) {
-                if (FP8) {
-                    if (timed)
-                        trace_layer0_e4m3<W, true>(a, w0s, wts, ray, ttid, x_s);
-                    else
-                        trace_layer0_e4m3<W, false>(a, w0s, wts, ray, ttid, x_s);
-                } else if (timed) {
-                    trace_layer0<W, F16, false, true>(a, reinterpret_cast<const float4*>(w0s), wts, ray, ttid, x_s, x_s);
-                } else {
-                    trace_layer0<W, F16, false, false>(a, reinterpret_cast<const float4*>(w0s), wts, ray, ttid, x_s, x_s);
-                }
-            }
-            fence_proxy_async_smem();
-            tc_fence_before();
-            if (!bar_or(1, NRAY, ray.state == kSlotActive)) break;
-
-            float f = 0.0f;
-            bool good = true;
-            for (int l = 0; l < KH; ++l) {
-                if (tid == 0) {
-                    tc_fence_after();
-                    for (int kb = 0; kb < KB && issue_ok; ++kb, ++g) {
-                        const uint32_t stage = g % NS;
-                        issue_ok = mbar_wait_bounded(bar_full + 8u * stage, (g / NS) & 1u, a.status, abort_flag);
-                        if (!issue_ok) break;
-                        tc_fence_after();
-#pragma unroll
-                        for (int t = 0; t < ST; ++t) {
-                            const uint64_t xd0 = desc_kmajor_sw128(base_s + L.x + t * xbytes);
-#pragma unroll
-                            for (int kk = 0; kk < 4; ++kk) {
-                                const uint64_t xd = desc_add(xd0, kb * 128u * 128u + kk * 32u);
-                                const uint64_t wd = desc_add(rd0, stage * kStreamStageBytes + kk * 32u);
-                                if (FP8)
-                                    mma_f8kind(tmem0 + t * W, xd, wd, idesc, (kb | kk) != 0);
-                                else
-                                    mma_f16kind(tmem0 + t * W, xd, wd, idesc, (kb | kk) != 0);
-                            }
-                        }
-                        mma_commit(bar_empty + 8u * stage);
-                    }
-                    if (issue_ok) mma_commit(bar_mma);
-                }
-                // a warp either reads the accumulator whole or not at all
-                good = __all_sync(0xffffffffu, mbar_wait_bounded(bar_mma, mma_phase, a.status, abort_flag) && good);
-                mma_phase ^= 1u;
-                tc_fence_after();
-                const float* bl = bhs + l * W;
-                const bool rd = good && wact;
-                // E4M3: accumulator -> value (the operand scales q_w and 256 divided out)
-                const float mf = FP8 ? 1.0f / (net.q_w[l] * kFp8ActScale) : 1.0f;
-                // 32-column chunks, the next one loading from TMEM while the current
-                // one is processed
-                float va[32], vb[32];
-                if (rd) {
-                    tmem_ld32(tmem + lane_base, va);
-                    tmem_wait_ld();
-                }
-                if (l + 1 < KH) {
-                    if (rd) {
-#pragma unroll
-                        for (int q = 0; q < W / 32; ++q) {
-                            float(&v)[32] = (q & 1) ? vb : va;
-                            float(&vn)[32] = (q & 1) ? va : vb;
-                            if (q + 1 < W / 32) tmem_ld32(tmem + lane_base + (q + 1) * 32u, vn);
-                            if (FP8)
-                                hidden_epilogue32_e4m3(v, bl, mf, ttid, q * 32, x_s);
-                            else
-                                hidden_epilogue32<F16, false>(v, bl, ttid, q * 32, x_s, x_s);
-                            tmem_wait_ld();
-                        }
-                    }
-                    fence_proxy_async_smem();
-                    tc_fence_before();
-                    bar_named(1, NRAY);
-                } else {
-                    float2 acc01 = make_float2(0.0f, 0.0f), acc23 = make_float2(0.0f, 0.0f);
-                    if (rd) {
-#pragma unroll
-                        for (int q = 0; q < W / 32; ++q) {
-                            float(&v)[32] = (q & 1) ? vb : va;
-                            float(&vn)[32] = (q & 1) ? va : vb;
-                            if (q + 1 < W / 32) tmem_ld32(tmem + lane_base + (q + 1) * 32u, vn);
-                            output_dot32<FP8>(v, bl + q * 32, wos + q * 32, acc01, acc23, mf);
-                            tmem_wait_ld();
-                        }
-                    }
-                    f = ((acc01.x + acc01.y) + (acc23.x + acc23.y)) + net.bout;
-                }
-            }
-            tc_fence_before();
-            if (good)
-                step_ray(a, ray, f);
-            else
-                ray.state = kSlotDone;
-        }
-        if (tid == 0) *consumed = g;
-        bar_named(1, NRAY);
-        if (tid == 0) {
-            __threadfence_block();
-            *done_flag = 1;
-        }
-    }
-
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        tc_fence_after();
-        tmem_dealloc(tmem0, W * ST);
-    }
-}
-
-
-
 }  // namespace
 
 bool tc_trace_supported(int width, int n_hidden) {
@@ -819,66 +478,41 @@ static int trace_tiles(Kernel k, int W, int KH, bool split) {
 }
 
 // The launch takes min(a.tiles, maximum) tiles per CTA when a.tiles > 0.
-template <int W, bool F16>
+template <int W, bool F16, bool SPLIT>
 static cudaError_t launch_trace_resident(const LevelArgs& a, int num_sms, cudaStream_t s) {
     const int KH = a.net.n_hidden;
-    const bool split = a.net.wbf_lo != nullptr && trace_split(W, KH);
-    if (split) {
-        auto k = trace_level_tc_kernel<W, F16, true>;
-        int T = trace_tiles(k, W, KH, true);
-        if (a.tiles > 0) T = std::min(T, a.tiles);
-        return launch_tc(k, 128 * T, trace_layout(W, KH, true, T).total + 1024, tmem_cols_for(T * W), num_sms, s, &a);
-    }
-    auto k = trace_level_tc_kernel<W, F16, false>;
-    int T = trace_tiles(k, W, KH, false);
+    auto k = trace_level_tc_kernel<W, F16, SPLIT>;
+    int T = trace_tiles(k, W, KH, SPLIT);
     if (a.tiles > 0) T = std::min(T, a.tiles);
-    return launch_tc(k, 128 * T, trace_layout(W, KH, false, T).total + 1024, tmem_cols_for(T * W), num_sms, s, &a);
+    return launch_tc(k, 128 * T, trace_layout(W, KH, SPLIT, T).total + 1024, tmem_cols_for(T * W), num_sms, s, &a);
 }
 
-template <int W, bool F16>
-static int trace_tiles_resident(const NetView& net) {
-    const int KH = net.n_hidden;
-    if (net.wbf_lo != nullptr && trace_split(W, KH)) return trace_tiles(trace_level_tc_kernel<W, F16, true>, W, KH, true);
-    return trace_tiles(trace_level_tc_kernel<W, F16, false>, W, KH, false);
-}
+// Networks of width 64 always fit with head and remainder operands; width 128 does up to k = 2.
+static bool split_of(const NetView& net) { return net.wbf_lo != nullptr && trace_split(net.width, net.n_hidden); }
 
 int trace_tiles_max(const NetView& net) {
     if (!tc_trace_supported(net.width, net.n_hidden)) return 0;
-    const bool f16 = net.op_f16 != 0;
-    switch (net.width) {
-    case 64:
-        return f16 ? trace_tiles_resident<64, true>(net) : trace_tiles_resident<64, false>(net);
-    case 128:
-        return f16 ? trace_tiles_resident<128, true>(net) : trace_tiles_resident<128, false>(net);
-    case 256:
-        return 2;  // the streamed-weight kernel: one or two tiles
-    }
-    return 0;
-}
-
-// Streamed-weight trace: two ray tiles per CTA unless a.tiles asks for one.
-template <int OP>
-static cudaError_t launch_trace_stream(const LevelArgs& a, int num_sms, cudaStream_t s) {
-    const int KH = a.net.n_hidden, EB = OP == kOpE4M3 ? 1 : 2;
-    if (a.tiles == 1)
-        return launch_tc(trace_level_tc_stream_kernel<OP, 1>, stream_threads(1),
-                         stream_layout(KH, 1, EB).total + 1024, kStreamW, num_sms, s, &a);
-    return launch_tc(trace_level_tc_stream_kernel<OP, 2>, stream_threads(2), stream_layout(KH, 2, EB).total + 1024,
-                     2 * kStreamW, num_sms, s, &a);
+    const int KH = net.n_hidden;
+    if (net.width == 64)
+        return net.op_f16 ? trace_tiles(trace_level_tc_kernel<64, true, true>, 64, KH, true)
+                          : trace_tiles(trace_level_tc_kernel<64, false, true>, 64, KH, true);
+    if (net.width == 128 && !split_of(net))
+        return net.op_f16 ? trace_tiles(trace_level_tc_kernel<128, true, false>, 128, KH, false)
+                          : trace_tiles(trace_level_tc_kernel<128, false, false>, 128, KH, false);
+    return 1;  // trace_wide_kernel: one launch shape
 }
 
 cudaError_t launch_trace_level_tc(const LevelArgs& a, int num_sms, cudaStream_t s) {
     const bool f16 = a.net.op_f16 != 0;
-    switch (a.net.width) {
-    case 64:
-        return f16 ? launch_trace_resident<64, true>(a, num_sms, s) : launch_trace_resident<64, false>(a, num_sms, s);
-    case 128:
-        return f16 ? launch_trace_resident<128, true>(a, num_sms, s) : launch_trace_resident<128, false>(a, num_sms, s);
-    case 256:
-        if (a.net.op_fp8) return launch_trace_stream<kOpE4M3>(a, num_sms, s);
-        return f16 ? launch_trace_stream<kOpF16>(a, num_sms, s) : launch_trace_stream<kOpBF16>(a, num_sms, s);
+    if (a.net.width == 64) {
+        if (a.n <= static_cast<int64_t>(num_sms) * kWideRays) return launch_trace_wide(a, num_sms, s);
+        return f16 ? launch_trace_resident<64, true, true>(a, num_sms, s)
+                   : launch_trace_resident<64, false, true>(a, num_sms, s);
     }
-    return cudaErrorInvalidValue;
+    if (a.net.width == 128 && !split_of(a.net))
+        return f16 ? launch_trace_resident<128, true, false>(a, num_sms, s)
+                   : launch_trace_resident<128, false, false>(a, num_sms, s);
+    return launch_trace_wide(a, num_sms, s);
 }
 
 bool tc_trace_split(int width, int n_hidden) { return width <= 128 && trace_split(width, n_hidden); }

@@ -44,6 +44,22 @@ __device__ __forceinline__ void stage_layer0(const NetView& net, float time, boo
     wts[i] = timed ? wt : 0.0f;
 }
 
+// Layer-0 parameters laid out for packed FP32 arithmetic on unit pairs
+// (trace kernels): pair p = units 2p, 2p+1 as two float4s,
+// (w_x0, w_x1, w_y0, w_y1) and (w_z0, w_z1, b0, b1); w_t per unit as before.
+__device__ __forceinline__ void stage_layer0_pairs(const NetView& net, float time, bool timed, int i, float* w0s,
+                                                   float* wts) {
+    const int p = i >> 1, e = i & 1;
+    float bb = net.b0[i];
+    const float wt = net.in_dim == 4 ? net.w0[i * 4 + 3] : 0.0f;
+    if (!timed) bb = fmaf(wt, time, bb);
+    w0s[p * 8 + e] = net.w0[i * net.in_dim + 0];
+    w0s[p * 8 + 2 + e] = net.w0[i * net.in_dim + 1];
+    w0s[p * 8 + 4 + e] = net.w0[i * net.in_dim + 2];
+    w0s[p * 8 + 6 + e] = bb;
+    wts[i] = timed ? wt : 0.0f;
+}
+
 // CTAs of `k` that fit on one SM, from its registers, shared memory, threads
 // and TMEM columns (the runtime's occupancy query reports 1 for kernels that
 // use tcgen05, whatever their footprint).
