@@ -35,9 +35,10 @@ RAYS = 300 * 152
 
 @pytest.mark.parametrize("width,hidden,in_dim,precision", [
     (64, 1, 3, "SDF_BF16"), (64, 3, 4, "SDF_FP16"), (128, 2, 3, "SDF_FP16"), (128, 1, 4, "SDF_BF16"),
-    (256, 2, 3, "SDF_BF16"), (256, 1, 4, "SDF_FP16"), (256, 2, 3, "SDF_FP8")])
+    (256, 2, 3, "SDF_BF16"), (256, 1, 4, "SDF_FP16"), (256, 2, 3, "SDF_FP8"), (64, 2, 4, "SDF_FP32"),
+    (128, 2, 3, "SDF_FP32"), (256, 1, 4, "SDF_FP32")])
 def test_few_rays_match_a_larger_call(sdf, width, hidden, in_dim, precision):
-    b = inputs.net_to_bytes(inputs.siren_init(5, width, hidden, in_dim=in_dim, out_shift=0.15))
+    b = inputs.net_to_bytes(inputs.siren_init(5, width, hidden, in_dim=in_dim, out_scale=30.0, out_shift=0.1))
     net = sdf.Net(b, getattr(sdf, precision))
     u = inputs.uniform01(31, 5 * RAYS).reshape(5, RAYS)
     orig = np.stack([3.0 * u[0] - 1.5, 3.0 * u[1] - 1.5, np.full(RAYS, 2.5)])
