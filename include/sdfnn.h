@@ -63,7 +63,8 @@ enum {
  * sine/cosine epilogues, the ray state and the step update are FP32 in all
  * modes. */
 enum {
-    SDF_FP32 = 0, /* SIMT FP32 contractions (the plain comparison path) */
+    SDF_FP32 = 0, /* FP32 results: traces on the FP32 units; gradients and training on
+                   * the tensor cores with operands split to FP32 accuracy */
     SDF_BF16 = 1, /* tcgen05 tensor-core contractions, bfloat16 operands, FP32 accumulation */
     SDF_FP8 = 2,  /* tcgen05 kind::f8f6f4 contractions with E4M3 operands, FP32 accumulation, for
                      sdf_normals / sdf_normal_map(_timed) of width 128 or 256 networks and
@@ -349,12 +350,17 @@ void sdf_frame_queue_free(sdf_frame_queue_t queue);
  *
  * sdf_train_shape_info: the length of theta and the workspace bytes the
  *   forward / backward pair needs for n points at that precision (either
- *   pointer may be NULL).  FP32: (1 + 8k) w floats per point; 16-bit:
- *   (1 + 5k) w floats per point plus two 16-bit copies of the hidden weights.
+ *   pointer may be NULL).  FP32: (1 + 8k) w floats per point plus copies of the hidden
+ *   weights (14 bytes each); 16-bit: (1 + 5k) w floats per point
+ *   plus two.
  * sdf_train_forward: f (n) and the unnormalised grad f (3, n) at pts (3, n)
  *   (pt_time (n) for 4-input networks, else NULL); saves the layers'
  *   pre-activations in `workspace` (device, 256-byte aligned, of the size
  *   above) for the backward.
+ * sdf_fit_forward: the same call for a fitting step.  At SDF_FP32 it forms
+ *   f and grad f by chains of FP32 FMAs in a fixed order, so that the
+ *   objective (FP64 sums over them) does not depend on how the tensor core
+ *   accumulates; elsewhere it is sdf_train_forward.
  * sdf_train_backward: ADDS dL/dtheta to d_theta (16-byte aligned, like theta) given d_f = dL/df (n) and
  *   d_grad = dL/d(grad f) (3, n), from the workspace of the forward call made
  *   with the same theta, points and n (zero d_theta first for a fresh
@@ -374,6 +380,9 @@ void sdf_frame_queue_free(sdf_frame_queue_t queue);
 int sdf_train_shape_info(int precision, int in_dim, int width, int n_hidden, int64_t n, int64_t *param_count,
                          int64_t *workspace_bytes);
 int sdf_train_forward(int precision, int in_dim, int width, int n_hidden, const float *theta, const float *pts,
+                      const float *pt_time, int64_t n, float *out_f, float *out_grad, void *workspace,
+                      void *cuda_stream);
+int sdf_fit_forward(int precision, int in_dim, int width, int n_hidden, const float *theta, const float *pts,
                       const float *pt_time, int64_t n, float *out_f, float *out_grad, void *workspace,
                       void *cuda_stream);
 int sdf_train_backward(int precision, int in_dim, int width, int n_hidden, const float *theta, const float *pts,

@@ -16,7 +16,7 @@ PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 INCLUDE = PKG.parent / "include"
 BUILD = PKG / "_build"
-SOURCES = ["api.cu", "simt.cu", "tc.cu", "trace_wide.cu", "f32_tc.cu", "train.cu", "train_tc.cu"]
+SOURCES = ["api.cu", "simt.cu", "tc.cu", "trace_wide.cu", "f32_tc.cu", "train.cu", "train_tc.cu", "train32_tc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
               "-Xptxas", "-warn-spills"]

@@ -1658,9 +1658,10 @@ static int train_prepare(int precision, int in_dim, int width, int n_hidden, con
     return SDF_OK;
 }
 
-int sdf_train_forward(int precision, int in_dim, int width, int n_hidden, const float* theta, const float* pts,
-                      const float* pt_time, int64_t n, float* out_f, float* out_grad, void* workspace,
-                      void* cuda_stream) {
+// fit: FP32 by FMA chains (the forward of a fitting step).
+static int train_forward(bool fit, int precision, int in_dim, int width, int n_hidden, const float* theta,
+                         const float* pts, const float* pt_time, int64_t n, float* out_f, float* out_grad,
+                         void* workspace, void* cuda_stream) {
     TrainArgs a;
     int dev = -1;
     int rc = train_prepare(precision, in_dim, width, n_hidden, theta, pts, pt_time, n, workspace, &a, &dev);
@@ -1674,10 +1675,25 @@ int sdf_train_forward(int precision, int in_dim, int width, int n_hidden, const 
     a.out_grad = out_grad;
     a.status = di.d_status;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    cudaError_t e = precision == SDF_FP32 ? launch_train_forward(a, di.num_sms, s)
-                                          : launch_train_forward_tc(a, precision == SDF_FP16, di.num_sms, s);
+    cudaError_t e = precision != SDF_FP32 ? launch_train_forward_tc(a, precision == SDF_FP16, di.num_sms, s)
+                    : fit                 ? launch_fit_forward(a, di.num_sms, s)
+                                          : launch_train_forward(a, di.num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "launching the training forward");
     return SDF_OK;
+}
+
+int sdf_train_forward(int precision, int in_dim, int width, int n_hidden, const float* theta, const float* pts,
+                      const float* pt_time, int64_t n, float* out_f, float* out_grad, void* workspace,
+                      void* cuda_stream) {
+    return train_forward(false, precision, in_dim, width, n_hidden, theta, pts, pt_time, n, out_f, out_grad, workspace,
+                         cuda_stream);
+}
+
+int sdf_fit_forward(int precision, int in_dim, int width, int n_hidden, const float* theta, const float* pts,
+                    const float* pt_time, int64_t n, float* out_f, float* out_grad, void* workspace,
+                    void* cuda_stream) {
+    return train_forward(true, precision, in_dim, width, n_hidden, theta, pts, pt_time, n, out_f, out_grad, workspace,
+                         cuda_stream);
 }
 
 int sdf_train_backward(int precision, int in_dim, int width, int n_hidden, const float* theta, const float* pts,

@@ -146,7 +146,11 @@ __device__ __forceinline__ void g32_point_async(uint32_t dst, const GradArgs& a,
 // last two bound by the host), the error against FP64 5 to 15 % lower on each
 // of six networks.  What bounds the (256,3) now is the alternation of MMAs
 // (6.1 k clocks a layer) and epilogue.
-template <int W>
+//
+// TRAIN: the training forward.  It saves A_0 ([n][W]) and (A_l, H_l^x, H_l^y,
+// H_l^z) ([k][n][W] float4: a warp's store is 512 consecutive bytes) and also
+// writes f (no list, no normalisation).
+template <int W, bool TRAIN = false>
 __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const GradArgs a) {
     using C = G32<W>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -294,6 +298,9 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
                 nidx = g32_index<C::NH, C::HPTS>(a, n_work, h, i + 1 < my_sets ? gt : -1, i + 1);
             }
             bar_named(1 + h, C::GROUP_THREADS);
+            // TRAIN: this thread's first point, and how many of its points are in the batch
+            const long long pb = ((static_cast<long long>(i) * G + blockIdx.x) * C::NH + h) * C::HPTS + cs * C::CPTS;
+            const int nv = TRAIN ? static_cast<int>(min(max(a.n - pb, 0ll), static_cast<long long>(C::CPTS))) : 0;
             // input layer: P_0 = sin(A_0), G_0^c = W_0[:, c] (.) cos(A_0), the tangents at scale g0
             if (live) {
 #pragma unroll 2
@@ -303,6 +310,7 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
                     for (int e = 0; e < 2; ++e) {
                         const float4 q = pts[q0 + 2 * c + e];
                         const float z = fmaf(u0.x, q.x, fmaf(u0.y, q.y, fmaf(u0.z, q.z, fmaf(ut, q.w, u0.w))));
+                        if (TRAIN && 2 * c + e < nv) a.save_a0[(pb + 2 * c + e) * W + m] = z;
                         float sn, cn;
                         sincos_r(z, &sn, &cn);
                         cn *= g0;
@@ -334,7 +342,9 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
                 const bool last = l + 1 == KH;
                 const float bb = __ldg(net.bh[l] + m), mf = __ldg(net.s32 + 4 * l);
                 // the tangents' multiplier: to the scale of the next operand, or to values times w_out
-                const float mg = last ? wo * __ldg(net.s32 + 4 * l + 2) : __ldg(net.s32 + 4 * l + 1);
+                const float mo = __ldg(net.s32 + 4 * l + 2);
+                const float mg = last ? wo * mo : __ldg(net.s32 + 4 * l + 1);
+                float4* save = TRAIN ? reinterpret_cast<float4*>(a.save_a) + (static_cast<size_t>(l) * a.n + pb) * W + m : nullptr;
 #pragma unroll 1
                 for (int q = 0; q < C::CPTS / 4; ++q) {
                     // four points: 16 columns of each accumulator
@@ -345,12 +355,17 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const int j = 4 * e;
-                        float sn, cn;
-                        sincos_r(fmaf(v[j] + c[j], mf, bb), &sn, &cn);
-                        cn *= mg;
-                        v[j] = sn;
+                        const float A = fmaf(v[j] + c[j], mf, bb);
 #pragma unroll
-                        for (int s = 1; s < 4; ++s) v[j + s] = cn * (v[j + s] + c[j + s]);
+                        for (int s = 1; s < 4; ++s) v[j + s] += c[j + s];
+                        if (TRAIN && 4 * q + e < nv)
+                            save[(4 * q + e) * W] = make_float4(A, v[j + 1] * mo, v[j + 2] * mo, v[j + 3] * mo);
+                        float sn, cn;
+                        sincos_r(A, &sn, &cn);
+                        cn *= mg;
+                        v[j] = TRAIN && last ? wo * sn : sn;
+#pragma unroll
+                        for (int s = 1; s < 4; ++s) v[j + s] *= cn;
                     }
                     if (last) {
                         warp_sum16(v, lane);
@@ -370,14 +385,16 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
             if (bar_or(1 + h, C::GROUP_THREADS, !ok || *abort_flag != 0)) break;
             if (gt < C::HPTS) {
                 if (idx >= 0) {
-                    float gx = 0.0f, gy = 0.0f, gz = 0.0f;
+                    float f = 0.0f, gx = 0.0f, gy = 0.0f, gz = 0.0f;
 #pragma unroll
                     for (int r = 0; r < W / 32; ++r) {
                         const float4 t = *reinterpret_cast<const float4*>(red + r * C::HROWS + gt * 4);
+                        f += t.x;
                         gx += t.y;
                         gy += t.z;
                         gz += t.w;
                     }
+                    if (TRAIN) a.out_f[idx] = f + __ldg(a.out_bias);
                     if (a.normalize) {
                         const float len = sqrtf(gx * gx + gy * gy + gz * gz);
                         const float inv = len >= 1e-12f ? 1.0f / len : 0.0f;

@@ -104,11 +104,12 @@ struct GradArgs {
     int normalize;                  // 1: unit normal (0 where |g| < 1e-12)
     unsigned long long* grab;       // tile counter, zero at launch
     int* status;
-    // training forward of the tensor-core path (the kernel's TRAIN variant): the
-    // pre-activations saved for the backward, f written beside grad f
+    // training forward (the kernels' TRAIN variants): the pre-activations saved
+    // for the backward, f written beside grad f
     float* save_a0;                 // [n][width] A_0
-    float* save_a;                  // A_l, hidden layers 1..k (layout: rec_a in grad_tc.cuh)
-    uint2* save_h;                  // (H_l^x, H_l^y | H_l^z, 0) in the operand type (layout: rec_h)
+    float* save_a;                  // 16-bit path: A_l, hidden layers 1..k (layout: rec_a in grad_tc.cuh);
+                                    // FP32 path: (A_l, H_l) [k][n][width][4]
+    uint2* save_h;                  // 16-bit path: (H_l^x, H_l^y | H_l^z, 0) in the operand type (layout: rec_h)
     int64_t save_np;                // points of the record layout: n rounded up to 64
     float* out_f;                   // (n)
     const float* out_bias;          // device address of b_out
@@ -132,7 +133,7 @@ bool tc_trace_split(int width, int n_hidden);  // head+remainder operands in the
 bool tc_grad_supported(int width, int n_hidden);
 
 // ---------------------------------------------------------------------------
-// training path (FP32)
+// training path
 // ---------------------------------------------------------------------------
 // Parameter vector theta: the folded parameters of Eq. 2 in the order of the
 // SDFN file (W_0 [w][in], b_0, then per hidden layer W_i [w][w], b_i, then
@@ -145,15 +146,18 @@ TrainShape train_shape(int in_dim, int width, int n_hidden);
 
 // Workspace of one forward / backward pair over n points.
 struct TrainWork {
-    // FP32 SIMT path
-    float* wt;                     // [k][w][w] transposed hidden weights
-    float* z0;                     // [n][w] layer-0 pre-activations A_0 (both paths)
-    float* z;                      // [k][n][4][w] per hidden layer: A_i and the tangent pre-images W_i G_{i-1}
-    float* d;                      // [k][n][4][w] their adjoints (backward)
+    // both paths
+    float* z0;                     // [n][w] layer-0 pre-activations A_0
+    uint8_t* wbf;                  // [k] W_l images (K-major, 128-byte swizzle, rows padded to 128): 16-bit, or FP32
+                                   // as two half planes per K block
+    uint8_t* wbft;                 // [k] W_l^T images, same layout: 16-bit, or FP32 as three bfloat16 planes per K block
     unsigned long long* counters;  // [4] tile counters
-    // tensor-core path
-    uint8_t* wbf;                  // [k] 16-bit W_l images (K-major, 128-byte swizzle, rows padded to 128)
-    uint8_t* wbft;                 // [k] 16-bit W_l^T images, same layout
+    // FP32 path
+    float* wt;                     // [k][w][w] transposed hidden weights (fitting forward)
+    float* s32;                    // the scales of NetView::s32, and at + 64 the norms they come from
+    float* z;                      // [k][n][w][4] per hidden layer: A_i and the tangent pre-images W_i G_{i-1}
+    float* d;                      // [k][n][w][4] their adjoints (backward)
+    // 16-bit path
     float* qa;                     // A_l records (rec_a layout)
     uint2* qh;                     // H_l^x, H_l^y | H_l^z, 0 as 16-bit operand-type values (rec_h layout)
     uint8_t* dtile;                // [k][n_halves][w * 256] 16-bit (dA_l, dH_l) tiles
@@ -180,6 +184,8 @@ struct TrainArgs {
 };
 cudaError_t launch_train_forward(const TrainArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_train_backward(const TrainArgs& a, int num_sms, cudaStream_t s);
+cudaError_t launch_fit_forward(const TrainArgs& a, int num_sms, cudaStream_t s);      // FP32 FMA chains
+cudaError_t launch_pack32_backward(const TrainArgs& a, int num_sms, cudaStream_t s);  // the W_l^T images alone
 // Tensor-core training (16-bit operands: f16 = IEEE half, else bfloat16; FP32 accumulation).
 cudaError_t launch_train_forward_tc(const TrainArgs& a, bool f16, int num_sms, cudaStream_t s);
 cudaError_t launch_train_backward_tc(const TrainArgs& a, bool f16, int num_sms, cudaStream_t s);

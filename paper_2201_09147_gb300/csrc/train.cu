@@ -1,23 +1,7 @@
-// Training path of the sine MLPs (FP32 SIMT).
-//
-// The fitting objective (values, gradient directions near the surface and
-// the Eikonal term) depends on f and on grad f, so its parameter gradient
-// runs backwards through Eq. 2 and through the tangent recursion of Alg. 2:
-//
-//   forward (per layer i):  A_i = W_i P_{i-1} + b_i,  H_i^c = W_i G_{i-1}^c,
-//                           P_i = sin A_i,  G_i^c = cos A_i (.) H_i^c,
-//                           f = w . P_k + b,  (grad f)_c = w . G_k^c
-//   backward:               dA_i  = dP_i (.) cos A_i - sin A_i (.) sum_c dG_i^c (.) H_i^c
-//                           dH_i^c = dG_i^c (.) cos A_i
-//                           dP_{i-1} = W_i^T dA_i,  dG_{i-1}^c = W_i^T dH_i^c
-//                           dW_i = dA_i P_{i-1}^T + sum_c dH_i^c (G_{i-1}^c)^T,  db_i = dA_i
-//
-// with layer 0 fed by the point (G_0^c = cos A_0 (.) W_0[:, c]).  Tiles of 32
-// points x 4 streams (value, three tangents) run through the same
-// register-tiled GEMM as the FP32 inference kernels; the forward saves A_i
-// and H_i for every layer, the backward writes (dA_i, dH_i) and the weight
-// gradients dW_i are separate GEMMs over all points.  Biases, W_0 and w_out
-// are reduced per CTA in shared memory and added once at the end.
+// Training path: the parameter vector's layout, the FP32 forward of a fitting
+// step, the fitting objective with its adjoints, and Adam.  The other forward
+// and backward kernels are in train32_tc.cu (FP32) and train_tc.cu (16-bit
+// operands).
 #include <cstdint>
 
 #include "common.cuh"
@@ -52,34 +36,17 @@ TrainShape train_shape(int in_dim, int width, int n_hidden) {
 }
 
 namespace {
-size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
-}  // namespace
-
-size_t train_workspace_bytes(const TrainShape& sh, int64_t n) {
-    const size_t W = sh.width, k = sh.n_hidden, N = static_cast<size_t>(n);
-    return align256(k * W * W * 4) + align256(N * W * 4) + 2 * align256(k * N * 4 * W * 4) + 256;
-}
-
-TrainWork train_work(const TrainShape& sh, int64_t n, void* ws) {
-    const size_t W = sh.width, k = sh.n_hidden, N = static_cast<size_t>(n);
-    uint8_t* p = static_cast<uint8_t*>(ws);
-    TrainWork w{};
-    w.wt = reinterpret_cast<float*>(p);
-    p += align256(k * W * W * 4);
-    w.z0 = reinterpret_cast<float*>(p);
-    p += align256(N * W * 4);
-    w.z = reinterpret_cast<float*>(p);
-    p += align256(k * N * 4 * W * 4);
-    w.d = reinterpret_cast<float*>(p);
-    p += align256(k * N * 4 * W * 4);
-    w.counters = reinterpret_cast<unsigned long long*>(p);
-    return w;
-}
-
-namespace {
 
 using namespace simt;
 
+// ---------------------------------------------------------------------------
+// forward of a fitting step
+// ---------------------------------------------------------------------------
+// f and grad f as chains of FP32 FMAs in a fixed order.  A fitting step reports
+// its objective in double, summed over f and grad f: the last bits of their
+// contractions show there, so it keeps this forward, whose values do not
+// depend on the tensor core's accumulation (train32_tc.cu has the other one,
+// for gradients through autograd).
 constexpr int kTilePts = 32;  // 32 points x 4 streams = the 128 rows of a tile
 
 // W^T of every hidden layer (the forward GEMM streams W^T).
@@ -106,7 +73,7 @@ struct FwdSmem {
 };
 
 template <int W>
-__global__ void __launch_bounds__(kSimtThreads) train_fwd_kernel(const TrainArgs a) {
+__global__ void __launch_bounds__(kSimtThreads, W == 64 ? 3 : W == 128 ? 2 : 1) train_fwd_kernel(const TrainArgs a) {
     extern __shared__ float4 smem_f4[];
     FwdSmem<W>& S = *reinterpret_cast<FwdSmem<W>*>(smem_f4);
     constexpr int FPT = W / 16;
@@ -170,14 +137,13 @@ __global__ void __launch_bounds__(kSimtThreads) train_fwd_kernel(const TrainArgs
         for (int l = 0; l < KH; ++l) {
             simt_gemm<W>(S.xt, a.w.wt + static_cast<size_t>(l) * W * W, S.ws, acc, r0, fg);
             const float* bl = a.theta + sh.off_b[l];
-            float* zl = a.w.z + static_cast<size_t>(l) * n * 4 * W;
+            float4* zl = reinterpret_cast<float4*>(a.w.z) + static_cast<size_t>(l) * n * W;
             const bool last = l + 1 == KH;
             float dot[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) dot[i] = 0.0f;
 #pragma unroll
             for (int jg = 0; jg < FPT / 4; ++jg) {
-                float zs[2][4][4];  // [point][stream][feature]
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int j = jg * 4 + e, nn = feat_of(j, fg);
@@ -187,10 +153,8 @@ __global__ void __launch_bounds__(kSimtThreads) train_fwd_kernel(const TrainArgs
                     for (int pp = 0; pp < 2; ++pp) {
                         const float A = acc[pp * 4][j] + bb;
                         const float h0 = acc[pp * 4 + 1][j], h1 = acc[pp * 4 + 2][j], h2 = acc[pp * 4 + 3][j];
-                        zs[pp][0][e] = A;
-                        zs[pp][1][e] = h0;
-                        zs[pp][2][e] = h1;
-                        zs[pp][3][e] = h2;
+                        const int64_t i = base + p0 + pp;
+                        if (i < n) zl[i * W + nn] = make_float4(A, h0, h1, h2);
                         float sn, cs;
                         sincos_r(A, &sn, &cs);
                         if (!last) {
@@ -202,16 +166,6 @@ __global__ void __launch_bounds__(kSimtThreads) train_fwd_kernel(const TrainArgs
                             dot[pp * 4 + 2] = fmaf(wo, cs * h1, dot[pp * 4 + 2]);
                             dot[pp * 4 + 3] = fmaf(wo, cs * h2, dot[pp * 4 + 3]);
                         }
-                    }
-                }
-#pragma unroll
-                for (int pp = 0; pp < 2; ++pp) {
-                    const int64_t i = base + p0 + pp;
-                    if (i < n) {
-#pragma unroll
-                        for (int st = 0; st < 4; ++st)
-                            *reinterpret_cast<float4*>(zl + (i * 4 + st) * W + feat_of(jg * 4, fg)) =
-                                make_float4(zs[pp][st][0], zs[pp][st][1], zs[pp][st][2], zs[pp][st][3]);
                     }
                 }
             }
@@ -236,295 +190,6 @@ __global__ void __launch_bounds__(kSimtThreads) train_fwd_kernel(const TrainArgs
         }
         __syncthreads();
     }
-}
-
-// ---------------------------------------------------------------------------
-// backward through the forward and tangent passes
-// ---------------------------------------------------------------------------
-template <int W>
-struct BwdSmem {
-    float xt[W * 128];
-    float ws[2 * kChunkK * W];
-    float px[kTilePts], py[kTilePts], pz[kTilePts], pt[kTilePts];
-    float df[kTilePts], dg[3][kTilePts];
-    float gb[(kMaxHidden + 1) * W];  // db_0 .. db_k
-    float gw0[4 * W];                // dW_0 [unit][input]
-    float gwo[W];                    // dw_out
-    float gbo;                       // db_out
-    long long tile;
-};
-
-template <int W>
-__global__ void __launch_bounds__(kSimtThreads) train_bwd_kernel(const TrainArgs a) {
-    extern __shared__ float4 smem_f4[];
-    BwdSmem<W>& S = *reinterpret_cast<BwdSmem<W>*>(smem_f4);
-    constexpr int FPT = W / 16;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int rg = warp * 2 + (lane >> 4), fg = lane & 15, r0 = rg * 8, p0 = r0 >> 2;
-    const TrainShape& sh = a.sh;
-    const int IN = sh.in_dim, KH = sh.n_hidden;
-    const float* W0 = a.theta + sh.off_w0;
-    const float* WO = a.theta + sh.off_wout;
-    const int64_t n = a.n;
-
-    for (int i = tid; i < (KH + 1) * W; i += kSimtThreads) S.gb[i] = 0.0f;
-    for (int i = tid; i < 4 * W; i += kSimtThreads) S.gw0[i] = 0.0f;
-    for (int i = tid; i < W; i += kSimtThreads) S.gwo[i] = 0.0f;
-    if (tid == 0) S.gbo = 0.0f;
-
-    while (true) {
-        __syncthreads();
-        if (tid == 0) S.tile = static_cast<long long>(atomicAdd(&a.w.counters[1], 1ull));
-        __syncthreads();
-        const int64_t base = S.tile * kTilePts;
-        if (base >= n) break;
-        if (tid < kTilePts) {
-            const int64_t i = base + tid;
-            const bool v = i < n;
-            S.px[tid] = v ? a.pts[i] : 0.0f;
-            S.py[tid] = v ? a.pts[n + i] : 0.0f;
-            S.pz[tid] = v ? a.pts[2 * n + i] : 0.0f;
-            S.pt[tid] = (v && a.pt_time) ? a.pt_time[i] : 0.0f;
-            const float dfi = v ? a.d_f[i] : 0.0f;
-            S.df[tid] = dfi;
-            S.dg[0][tid] = v ? a.d_grad[i] : 0.0f;
-            S.dg[1][tid] = v ? a.d_grad[n + i] : 0.0f;
-            S.dg[2][tid] = v ? a.d_grad[2 * n + i] : 0.0f;
-            float sdf = dfi;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sdf += __shfl_xor_sync(0xffffffffu, sdf, o);
-            if (tid == 0) S.gbo += sdf;
-        }
-        __syncthreads();
-
-        // adjoints of the last layer's outputs: dP_k = df w_out, dG_k^c = dg_c w_out,
-        // and dw_out = sum_p (df P_k + sum_c dg_c G_k^c)
-        float Y[8][FPT];
-        {
-            const float* zl = a.w.z + static_cast<size_t>(KH - 1) * n * 4 * W;
-#pragma unroll
-            for (int jg = 0; jg < FPT / 4; ++jg) {
-                float4 z[2][4];
-#pragma unroll
-                for (int pp = 0; pp < 2; ++pp) {
-                    const int64_t i = base + p0 + pp;
-#pragma unroll
-                    for (int st = 0; st < 4; ++st)
-                        z[pp][st] = i < n ? *reinterpret_cast<const float4*>(zl + (i * 4 + st) * W + feat_of(jg * 4, fg))
-                                          : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int j = jg * 4 + e, nn = feat_of(j, fg);
-                    const float wo = WO[nn];
-                    float gsum = 0.0f;
-#pragma unroll
-                    for (int pp = 0; pp < 2; ++pp) {
-                        const int p = p0 + pp;
-                        const float A = reinterpret_cast<const float*>(&z[pp][0])[e];
-                        float sn, cs;
-                        sincos_r(A, &sn, &cs);
-                        const float h0 = reinterpret_cast<const float*>(&z[pp][1])[e];
-                        const float h1 = reinterpret_cast<const float*>(&z[pp][2])[e];
-                        const float h2 = reinterpret_cast<const float*>(&z[pp][3])[e];
-                        gsum += S.df[p] * sn + cs * (S.dg[0][p] * h0 + S.dg[1][p] * h1 + S.dg[2][p] * h2);
-                        Y[pp * 4 + 0][j] = S.df[p] * wo;
-                        Y[pp * 4 + 1][j] = S.dg[0][p] * wo;
-                        Y[pp * 4 + 2][j] = S.dg[1][p] * wo;
-                        Y[pp * 4 + 3][j] = S.dg[2][p] * wo;
-                    }
-                    atomicAdd(&S.gwo[nn], gsum);
-                }
-            }
-        }
-
-        // hidden layers, last to first: (dA_l, dH_l) from (dP_l, dG_l), then dP_{l-1}, dG_{l-1}
-        for (int l = KH - 1; l >= 0; --l) {
-            const float* zl = a.w.z + static_cast<size_t>(l) * n * 4 * W;
-            float* dl = a.w.d + static_cast<size_t>(l) * n * 4 * W;
-#pragma unroll
-            for (int jg = 0; jg < FPT / 4; ++jg) {
-                float4 z[2][4];
-#pragma unroll
-                for (int pp = 0; pp < 2; ++pp) {
-                    const int64_t i = base + p0 + pp;
-#pragma unroll
-                    for (int st = 0; st < 4; ++st)
-                        z[pp][st] = i < n ? *reinterpret_cast<const float4*>(zl + (i * 4 + st) * W + feat_of(jg * 4, fg))
-                                          : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                }
-                float dv[2][4][4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int j = jg * 4 + e, nn = feat_of(j, fg);
-                    float bsum = 0.0f;
-#pragma unroll
-                    for (int pp = 0; pp < 2; ++pp) {
-                        const float A = reinterpret_cast<const float*>(&z[pp][0])[e];
-                        const float h0 = reinterpret_cast<const float*>(&z[pp][1])[e];
-                        const float h1 = reinterpret_cast<const float*>(&z[pp][2])[e];
-                        const float h2 = reinterpret_cast<const float*>(&z[pp][3])[e];
-                        float sn, cs;
-                        sincos_r(A, &sn, &cs);
-                        const float dA = Y[pp * 4][j] * cs -
-                                         sn * (Y[pp * 4 + 1][j] * h0 + Y[pp * 4 + 2][j] * h1 + Y[pp * 4 + 3][j] * h2);
-                        const float d0 = Y[pp * 4 + 1][j] * cs, d1 = Y[pp * 4 + 2][j] * cs, d2 = Y[pp * 4 + 3][j] * cs;
-                        dv[pp][0][e] = dA;
-                        dv[pp][1][e] = d0;
-                        dv[pp][2][e] = d1;
-                        dv[pp][3][e] = d2;
-                        bsum += dA;
-                        *reinterpret_cast<float4*>(S.xt + xt_index(nn, r0 + pp * 4)) = make_float4(dA, d0, d1, d2);
-                    }
-                    atomicAdd(&S.gb[(l + 1) * W + nn], bsum);
-                }
-#pragma unroll
-                for (int pp = 0; pp < 2; ++pp) {
-                    const int64_t i = base + p0 + pp;
-                    if (i < n) {
-#pragma unroll
-                        for (int st = 0; st < 4; ++st)
-                            *reinterpret_cast<float4*>(dl + (i * 4 + st) * W + feat_of(jg * 4, fg)) =
-                                make_float4(dv[pp][st][0], dv[pp][st][1], dv[pp][st][2], dv[pp][st][3]);
-                    }
-                }
-            }
-            __syncthreads();
-            // rows x W_l (row-major [unit][input]): dP_{l-1} = W_l^T dA_l, dG_{l-1}^c = W_l^T dH_l^c
-            simt_gemm<W>(S.xt, a.theta + sh.off_w[l], S.ws, Y, r0, fg);
-        }
-
-        // layer 0: dA_0 = dP_0 cos A_0 - sin A_0 sum_c dG_0^c W_0[:, c];
-        // dW_0[:, c] = dA_0 x_c + dG_0^c cos A_0 (c < 3), dA_0 t (c = 3);  db_0 = dA_0
-#pragma unroll
-        for (int jg = 0; jg < FPT / 4; ++jg) {
-            float4 z[2];
-#pragma unroll
-            for (int pp = 0; pp < 2; ++pp) {
-                const int64_t i = base + p0 + pp;
-                z[pp] = i < n ? *reinterpret_cast<const float4*>(a.w.z0 + i * W + feat_of(jg * 4, fg))
-                              : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int j = jg * 4 + e, nn = feat_of(j, fg);
-                const float wx = W0[nn * IN], wy = W0[nn * IN + 1], wz = W0[nn * IN + 2];
-                float g0 = 0.0f, g1 = 0.0f, g2 = 0.0f, g3 = 0.0f, gbs = 0.0f;
-#pragma unroll
-                for (int pp = 0; pp < 2; ++pp) {
-                    const int p = p0 + pp;
-                    const float A = reinterpret_cast<const float*>(&z[pp])[e];
-                    float sn, cs;
-                    sincos_r(A, &sn, &cs);
-                    const float y1 = Y[pp * 4 + 1][j], y2 = Y[pp * 4 + 2][j], y3 = Y[pp * 4 + 3][j];
-                    const float dA = Y[pp * 4][j] * cs - sn * (y1 * wx + y2 * wy + y3 * wz);
-                    g0 += dA * S.px[p] + y1 * cs;
-                    g1 += dA * S.py[p] + y2 * cs;
-                    g2 += dA * S.pz[p] + y3 * cs;
-                    g3 += dA * S.pt[p];
-                    gbs += dA;
-                }
-                atomicAdd(&S.gw0[nn * 4 + 0], g0);
-                atomicAdd(&S.gw0[nn * 4 + 1], g1);
-                atomicAdd(&S.gw0[nn * 4 + 2], g2);
-                atomicAdd(&S.gw0[nn * 4 + 3], g3);
-                atomicAdd(&S.gb[nn], gbs);
-            }
-        }
-    }
-
-    // per-CTA partial sums into dL/dtheta
-    __syncthreads();
-    for (int i = tid; i < W; i += kSimtThreads) {
-        atomicAdd(a.d_theta + sh.off_b0 + i, S.gb[i]);
-        for (int l = 0; l < KH; ++l) atomicAdd(a.d_theta + sh.off_b[l] + i, S.gb[(l + 1) * W + i]);
-        for (int c = 0; c < IN; ++c) atomicAdd(a.d_theta + sh.off_w0 + i * IN + c, S.gw0[i * 4 + c]);
-        atomicAdd(a.d_theta + sh.off_wout + i, S.gwo[i]);
-    }
-    if (tid == 0) atomicAdd(a.d_theta + sh.off_bout, S.gbo);
-}
-
-// ---------------------------------------------------------------------------
-// dW_l = sum over rows (point, stream) of (dA_l, dH_l)[row] x (P_{l-1}, G_{l-1})[row]
-// ---------------------------------------------------------------------------
-// Block: all W units x 64 inputs of dW_l, over a contiguous range of rows
-// (split-K over blockIdx.y); the input activations are recomputed from the
-// saved pre-activations of the layer below (or layer 0).
-constexpr int kWgRows = 32;
-
-template <int W>
-__global__ void __launch_bounds__(256) wgrad_kernel(const TrainArgs a, int l, int64_t rows_per_split) {
-    constexpr int TM = W / 32;  // units per thread
-    __shared__ float Ds[kWgRows][W];
-    __shared__ float Xs[kWgRows][64 + 4];
-    const int tid = threadIdx.x, tm = tid >> 3, tn = tid & 7;
-    const int kb = blockIdx.x * 64;
-    const TrainShape& sh = a.sh;
-    const int IN = sh.in_dim;
-    const int64_t n = a.n, rows = 4 * n;
-    const int64_t r_begin = static_cast<int64_t>(blockIdx.y) * rows_per_split;
-    const int64_t r_end = r_begin + rows_per_split < rows ? r_begin + rows_per_split : rows;
-    const float* dl = a.w.d + static_cast<size_t>(l) * n * 4 * W;
-    const float* zb = l > 0 ? a.w.z + static_cast<size_t>(l - 1) * n * 4 * W : nullptr;
-    const float* W0 = a.theta + sh.off_w0;
-    float acc[TM][8];
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) acc[i][b] = 0.0f;
-
-    for (int64_t r0 = r_begin; r0 < r_end; r0 += kWgRows) {
-        // adjoint rows (all W units)
-        for (int q = tid; q < kWgRows * W / 4; q += 256) {
-            const int rr = q / (W / 4), c4 = q % (W / 4);
-            const int64_t r = r0 + rr;
-            const float4 v = r < r_end ? *reinterpret_cast<const float4*>(dl + r * W + c4 * 4)
-                                       : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            *reinterpret_cast<float4*>(&Ds[rr][c4 * 4]) = v;
-        }
-        // input activations of this block's 64 inputs: row tid / 8, inputs (tid % 8) * 8 .. + 7
-        {
-            const int rr = tid >> 3, c0 = (tid & 7) * 8;
-            const int64_t r = r0 + rr;
-            const int64_t p = r >> 2;
-            const int st = static_cast<int>(r & 3);
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                const int k = kb + c0 + b;
-                float x = 0.0f;
-                if (r < r_end) {
-                    float sn, cs;
-                    if (l > 0) {
-                        sincos_r(zb[(p * 4) * W + k], &sn, &cs);
-                        x = st == 0 ? sn : cs * zb[(p * 4 + st) * W + k];
-                    } else {
-                        sincos_r(a.w.z0[p * W + k], &sn, &cs);
-                        x = st == 0 ? sn : cs * W0[k * IN + st - 1];
-                    }
-                }
-                Xs[rr][c0 + b] = x;
-            }
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int rr = 0; rr < kWgRows; ++rr) {
-            float dv[TM], xv[8];
-#pragma unroll
-            for (int i = 0; i < TM; ++i) dv[i] = Ds[rr][tm * TM + i];
-#pragma unroll
-            for (int b = 0; b < 8; ++b) xv[b] = Xs[rr][tn * 8 + b];
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int b = 0; b < 8; ++b) acc[i][b] = fmaf(dv[i], xv[b], acc[i][b]);
-        }
-        __syncthreads();
-    }
-    float* gw = a.d_theta + sh.off_w[l];
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) atomicAdd(gw + (tm * TM + i) * W + kb + tn * 8 + b, acc[i][b]);
 }
 
 // ---------------------------------------------------------------------------
@@ -664,30 +329,11 @@ cudaError_t forward_w(const TrainArgs& a, int num_sms, cudaStream_t s) {
     return launch_simt_persistent(train_fwd_kernel<W>, sizeof(FwdSmem<W>), num_sms, s, &a);
 }
 
-template <int W>
-cudaError_t backward_w(const TrainArgs& a, int num_sms, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(a.w.counters, 0, 4 * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
-    e = launch_simt_persistent(train_bwd_kernel<W>, sizeof(BwdSmem<W>), num_sms, s, &a);
-    if (e != cudaSuccess) return e;
-    // split the rows of each weight-gradient GEMM over about two CTAs per SM
-    const int64_t rows = 4 * a.n;
-    const int kblocks = W / 64;
-    int64_t splits = (2 * num_sms + kblocks - 1) / kblocks;
-    int64_t per = (rows + splits - 1) / splits;
-    per = (per + kWgRows - 1) / kWgRows * kWgRows;
-    splits = (rows + per - 1) / per;
-    for (int l = 0; l < a.sh.n_hidden; ++l) {
-        wgrad_kernel<W><<<dim3(kblocks, static_cast<unsigned>(splits)), 256, 0, s>>>(a, l, per);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
 }  // namespace
 
-cudaError_t launch_train_forward(const TrainArgs& a, int num_sms, cudaStream_t s) {
+cudaError_t launch_fit_forward(const TrainArgs& a, int num_sms, cudaStream_t s) {
+    cudaError_t e = launch_pack32_backward(a, num_sms, s);
+    if (e != cudaSuccess) return e;
     switch (a.sh.width) {
     case 64:
         return forward_w<64>(a, num_sms, s);
@@ -695,18 +341,6 @@ cudaError_t launch_train_forward(const TrainArgs& a, int num_sms, cudaStream_t s
         return forward_w<128>(a, num_sms, s);
     case 256:
         return forward_w<256>(a, num_sms, s);
-    }
-    return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_train_backward(const TrainArgs& a, int num_sms, cudaStream_t s) {
-    switch (a.sh.width) {
-    case 64:
-        return backward_w<64>(a, num_sms, s);
-    case 128:
-        return backward_w<128>(a, num_sms, s);
-    case 256:
-        return backward_w<256>(a, num_sms, s);
     }
     return cudaErrorInvalidValue;
 }

@@ -23,7 +23,7 @@ ERRORS = {-1: "SDF_ERR_ARG", -2: "SDF_ERR_FILE", -3: "SDF_ERR_FORMAT", -4: "SDF_
 EXPORTS = ["sdf_net_load", "sdf_net_load_mem", "sdf_net_info", "sdf_net_set_time", "sdf_net_free",
            "sdf_trace_multiscale", "sdf_normals", "sdf_normal_map", "sdf_render_host", "sdf_sync_status",
            "sdf_last_error", "sdf_trace_multiscale_noalloc", "sdf_normal_map_timed", "sdf_plan_create",
-           "sdf_plan_launch", "sdf_plan_info", "sdf_plan_free", "sdf_train_shape_info", "sdf_train_forward",
+           "sdf_plan_launch", "sdf_plan_info", "sdf_plan_free", "sdf_train_shape_info", "sdf_train_forward", "sdf_fit_forward",
            "sdf_train_backward", "sdf_fit_loss", "sdf_adam_step", "sdf_selftest_wait_timeout",
            "sdf_measure_sine_rate", "sdf_frame_queue_create", "sdf_frame_queue_submit", "sdf_frame_queue_wait",
            "sdf_frame_queue_free", "sdf_selftest_noalloc_timeout", "sdf_theta_from_image",
@@ -86,7 +86,8 @@ def lib():
         L.sdf_frame_queue_free.restype = None
         i64p = C.POINTER(C.c_int64)
         L.sdf_train_shape_info.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int64, i64p, i64p]
-        L.sdf_train_forward.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, vp, vp, vp, C.c_int64, vp, vp, vp, vp]
+        for fwd in (L.sdf_train_forward, L.sdf_fit_forward):
+            fwd.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, vp, vp, vp, C.c_int64, vp, vp, vp, vp]
         L.sdf_train_backward.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, vp, vp, vp, C.c_int64, vp, vp, vp, vp,
                                          vp]
         L.sdf_fit_loss.argtypes = [vp, vp, vp, vp, vp, C.c_int64, C.c_float, C.c_float, vp, vp, vp, vp]
@@ -413,6 +414,10 @@ def sdfn_from_theta(shape, theta) -> bytes:
 def train_forward(shape, theta, pts, pt_time=None, workspace=None, stream=None, precision: int = SDF_FP32):
     """f (n) and grad f (3, n) at device points (3, n); returns (f, grad, workspace).  A given
     workspace is used if it is large enough, else a new one is made."""
+    return _forward(lib().sdf_train_forward, shape, theta, pts, pt_time, workspace, stream, precision)
+
+
+def _forward(entry, shape, theta, pts, pt_time, workspace, stream, precision):
     in_dim, width, n_hidden = shape
     n = pts.shape[1]
     _, wb = train_shape_info(in_dim, width, n_hidden, n, precision)
@@ -420,8 +425,8 @@ def train_forward(shape, theta, pts, pt_time=None, workspace=None, stream=None, 
         workspace = torch.empty(wb, dtype=torch.uint8, device=pts.device)
     f = torch.empty(n, dtype=torch.float32, device=pts.device)
     g = torch.empty((3, n), dtype=torch.float32, device=pts.device)
-    _check(lib().sdf_train_forward(precision, in_dim, width, n_hidden, _ptr(theta), _ptr(pts), _ptr(pt_time), n,
-                                   _ptr(f), _ptr(g), _ptr(workspace), C.c_void_p(_stream(stream))))
+    _check(entry(precision, in_dim, width, n_hidden, _ptr(theta), _ptr(pts), _ptr(pt_time), n, _ptr(f), _ptr(g),
+                 _ptr(workspace), C.c_void_p(_stream(stream))))
     return f, g, workspace
 
 
@@ -481,8 +486,7 @@ def fit_step(shape, theta, m, v, step, pts, target_f, target_grad, near, *, lam_
     loss is the device float64 vector (l_val, l_dir, l_eik, L) before the update.
     sine_lr_scale multiplies the learning rate of the sine layers' (folded) parameters: with the
     frequency omega it gives the steps Adam takes on the unfolded SIREN parameters."""
-    f, g, workspace = train_forward(shape, theta, pts, pt_time=pt_time, workspace=workspace, stream=stream,
-                                    precision=precision)
+    f, g, workspace = _forward(lib().sdf_fit_forward, shape, theta, pts, pt_time, workspace, stream, precision)
     d_f, d_g, loss = fit_loss(f, g, target_f, target_grad, near, lam_n, lam_e, stream=stream)
     d_theta = train_backward(shape, theta, pts, d_f, d_g, workspace, pt_time=pt_time, stream=stream,
                              precision=precision)

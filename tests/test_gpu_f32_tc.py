@@ -1,5 +1,5 @@
-"""Gradients of FP32 networks on the tensor cores (half-precision head and remainder operands) against the FP64
-oracle, at the sizes where the tiles can go wrong.
+"""Gradients and training of FP32 networks on the tensor cores (operands split into 16-bit parts)
+against FP64, at the sizes where the tiles can go wrong.
 
 Tolerance.  u = 2^-24.  A sine layer adds a sine error of at most 8u (5e-7) and a contraction whose
 rounding stays below 8u of its result's scale; the layers that follow may amplify both by the gain
@@ -93,3 +93,47 @@ def test_small_weights(sdf, log2):
     ref = oracle.Net(b).grad_batch(pts.astype(np.float64))
     s = 2.0 ** -log2
     assert rel_rms(g.astype(np.float64) * s, ref * s) <= 64 * U * 3
+
+
+def reference_training(shape, theta, pts, time, d_f, d_g):
+    """f, grad f and dL/dtheta of L = <d_f, f> + <d_g, grad f> in float64 (torch autograd)."""
+    d, w, k = shape
+    th = torch.from_numpy(theta).double().cuda().requires_grad_(True)
+    x = torch.from_numpy(pts).double().cuda()
+    if d == 4:
+        x = torch.cat([x, torch.from_numpy(time).double().cuda()[None]])
+    o, h, g = 0, x, None
+    for layer in range(k + 1):
+        fan = d if layer == 0 else w
+        W, b = th[o:o + w * fan].reshape(w, fan), th[o + w * fan:o + w * fan + w]
+        o += w * fan + w
+        z = W @ h + b[:, None]
+        c, h = torch.cos(z), torch.sin(z)
+        g = [W[:, i:i + 1] * c for i in range(3)] if layer == 0 else [(W @ t) * c for t in g]
+    f = th[o:o + w] @ h + th[o + w]
+    grad = torch.stack([th[o:o + w] @ t for t in g])
+    loss = (f * torch.from_numpy(d_f).double().cuda()).sum() + (grad * torch.from_numpy(d_g).double().cuda()).sum()
+    return f.detach(), grad.detach(), torch.autograd.grad(loss, th)[0]
+
+
+# one point, the edges of a K block (16 points), of a tile (32) and of a CTA's two tiles, and a batch whose
+# weight-gradient blocks do not divide evenly over the CTAs.  d_theta adds a third contraction (over the batch)
+# and the sums of the backward to the forward's errors: 128 u (k + 1).
+@pytest.mark.parametrize("n", [1, 15, 17, 33, 64, 65, 3001])
+@pytest.mark.parametrize("name", ["64x1", "64x3", "128x2_t", "256x1", "256x4"])
+def test_training_gradients(sdf, name, n):
+    w, k, d = NETS[name]
+    shape, theta = sdfnn_theta(net_bytes(name))
+    pts, time = points(n), inputs.uniform01(7, n).astype(np.float32)
+    z = (2.0 * inputs.uniform01(8, 4 * n) - 1.0).astype(np.float32) / n
+    d_f, d_g = z[:n].copy(), z[n:].reshape(3, n).copy()
+    dev = lambda a: torch.from_numpy(a).cuda()
+    th, tm = dev(theta), dev(time) if d == 4 else None
+    f, g, ws = sdf.train_forward(shape, th, dev(pts), pt_time=tm)
+    d_theta = sdf.train_backward(shape, th, dev(pts), dev(d_f), dev(d_g), ws, pt_time=tm)
+    sdf.sync_status()
+    rf, rg, rt = reference_training(shape, theta, pts, time, d_f, d_g)
+    host = lambda t: t.cpu().numpy().astype(np.float64)
+    assert rel_rms(host(f), host(rf)) <= 64 * U * (k + 1)
+    assert rel_rms(host(g), host(rg)) <= 64 * U * (k + 1)
+    assert rel_rms(host(d_theta), host(rt)) <= 128 * U * (k + 1)
