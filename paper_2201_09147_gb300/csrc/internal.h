@@ -109,7 +109,7 @@ struct GradArgs {
     float* save_a0;                 // [n][width] A_0
     float* save_a;                  // 16-bit path: A_l, hidden layers 1..k (layout: rec_a in grad_tc.cuh);
                                     // FP32 path: (A_l, H_l) [k][n][width][4]
-    uint2* save_h;                  // 16-bit path: (H_l^x, H_l^y | H_l^z, 0) in the operand type (layout: rec_h)
+    uint2* save_h;                  // 16-bit path: H_l in the operand type (layout: rec_h)
     int64_t save_np;                // points of the record layout: n rounded up to 64
     float* out_f;                   // (n)
     const float* out_bias;          // device address of b_out
@@ -159,7 +159,7 @@ struct TrainWork {
     float* d;                      // [k][n][w][4] their adjoints (backward)
     // 16-bit path
     float* qa;                     // A_l records (rec_a layout)
-    uint2* qh;                     // H_l^x, H_l^y | H_l^z, 0 as 16-bit operand-type values (rec_h layout)
+    uint2* qh;                     // H_l as 16-bit operand-type values (rec_h layout)
     uint8_t* dtile;                // [k][n_halves][w * 256] 16-bit (dA_l, dH_l) tiles
     int64_t n_halves;              // 2 ceil(n / 64): half-tiles of 32 points, in pairs
 };

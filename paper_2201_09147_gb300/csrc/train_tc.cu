@@ -117,8 +117,8 @@ struct TrainTcArgs {
     const float* d_f;            // (n)
     const float* d_grad;         // SoA (3, n)
     const float* a0;             // [n][W] A_0 (training forward)
-    const float* qa;             // A_l records (rec_a layout)
-    const uint2* qh;             // H_l records, 16-bit operand type (x, y | z, 0) (rec_h layout)
+    const float4* qa;            // A_l records (rec_a layout)
+    const uint4* qh;             // H_l records in the 16-bit operand type (rec_h layout)
     int64_t np;                  // points of the record layout (n rounded up to 64)
     uint8_t* dtile;              // [k][n_halves][W * 256]: D_l tiles, 16-bit, the swizzled operand image
     int64_t n_halves;
@@ -127,16 +127,23 @@ struct TrainTcArgs {
     const uint32_t* amax_bits;   // bits of max |d_f|, |d_grad| (a non-negative float)
 };
 
-// A saved (A_l, H_l) from its A and its 16-bit H image (x, y | z, 0).  The
-// kernels load the records of a chunk of consecutive points as 16-byte
-// vectors (4 points' A, 2 points' H per load), all in flight at once, and
-// decode each one where it is used.
-template <bool F16>
-__device__ __forceinline__ float4 decode_q(float a, uint32_t hxy, uint32_t hz) {
-    return make_float4(a, from16<F16>(static_cast<uint16_t>(hxy & 0xFFFFu)), from16<F16>(static_cast<uint16_t>(hxy >> 16)),
-                       from16<F16>(static_cast<uint16_t>(hz & 0xFFFFu)));
-}
 __device__ __forceinline__ float pick4(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+__device__ __forceinline__ uint32_t word4(const uint4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+
+// Point e of a chunk of consecutive points (the first a multiple of 8) from its
+// records: a4[u] the A of points 4u .. 4u+3, h4 the H words of 8 points per
+// three vectors.  The kernels load a chunk's records as 16-byte vectors, all in
+// flight at once, and decode each point where it is used.
+template <bool F16, int NA, int NH>
+__device__ __forceinline__ float4 decode_q(const float4 (&a4)[NA], const uint4 (&h4)[NH], int e) {
+    const int w = (e >> 1) * 3;  // the pair's first word
+    const uint32_t w0 = word4(h4[w >> 2], w & 3), w1 = word4(h4[(w + 1) >> 2], (w + 1) & 3),
+                   w2 = word4(h4[(w + 2) >> 2], (w + 2) & 3);
+    auto lo = [](uint32_t x) { return from16<F16>(static_cast<uint16_t>(x & 0xFFFFu)); };
+    auto hi = [](uint32_t x) { return from16<F16>(static_cast<uint16_t>(x >> 16)); };
+    const float A = pick4(a4[e >> 2], e & 3);
+    return (e & 1) ? make_float4(A, hi(w1), lo(w2), hi(w2)) : make_float4(A, lo(w0), hi(w0), lo(w1));
+}
 
 // Hint: bring the line holding p into L2 (no register, no completion to wait for).
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
@@ -340,16 +347,13 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
                         // the chunk's 8 saved (A, H): independent read-only loads, all in flight at once
                         // the chunk's 8 points are consecutive, the first a multiple of 8
                         float4 a4[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-                        uint4 h4[4] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u),
-                                       make_uint4(0u, 0u, 0u, 0u)};
+                        uint4 h4[3] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
                         const int idx8 = idxs[p0 + q * 8];
                         if (idx8 >= 0) {
 #pragma unroll
-                            for (int u = 0; u < 2; ++u)
-                                a4[u] = __ldg(reinterpret_cast<const float4*>(a.qa + rec_a(l, a.np, W, idx8 + 4 * u, m)));
+                            for (int u = 0; u < 2; ++u) a4[u] = __ldg(a.qa + rec_a(l, a.np, W, idx8, m) + u * W);
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                h4[u] = __ldg(reinterpret_cast<const uint4*>(a.qh + rec_h(l, a.np, W, idx8 + 2 * u, m)));
+                            for (int u = 0; u < 3; ++u) h4[u] = __ldg(a.qh + rec_h(l, a.np, W, idx8, m) + u * W);
                         }
                         // the next chunk's records (this layer's next chunk, or the first chunk of the
                         // layer below) towards L2 while this one is processed
@@ -358,9 +362,9 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
                             const int in8 = idxs[p0 + ((q + 1) % (C::HROWS / 32)) * 8];
                             if (ln >= 0 && in8 >= 0) {
 #pragma unroll
-                                for (int u = 0; u < 2; ++u) prefetch_l2(a.qa + rec_a(ln, a.np, W, in8 + 4 * u, m));
+                                for (int u = 0; u < 2; ++u) prefetch_l2(a.qa + rec_a(ln, a.np, W, in8, m) + u * W);
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) prefetch_l2(a.qh + rec_h(ln, a.np, W, in8 + 2 * u, m));
+                                for (int u = 0; u < 3; ++u) prefetch_l2(a.qh + rec_h(ln, a.np, W, in8, m) + u * W);
                             }
                         }
 #pragma unroll
@@ -369,10 +373,7 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
 #pragma unroll
                             for (int e = 0; e < 2; ++e) {
                                 const int p = p0 + q * 8 + 2 * c + e, j = (2 * c + e) * 4;
-                                const int ee = 2 * c + e;  // point of the chunk
-                                const uint4& hp = h4[ee >> 1];
-                                const float4 Q = idxs[p] >= 0 ? decode_q<F16>(pick4(a4[ee >> 2], ee & 3),
-                                                                              (ee & 1) ? hp.z : hp.x, (ee & 1) ? hp.w : hp.y)
+                                const float4 Q = idxs[p] >= 0 ? decode_q<F16>(a4, h4, 2 * c + e)
                                                               : make_float4(0.f, 0.f, 0.f, 0.f);
                                 float y0, y1, y2, y3;
                                 if (top) {
@@ -620,21 +621,19 @@ __global__ void __launch_bounds__(WgCfg<W>::THREADS) train_wgrad_tc_kernel(const
                     const int64_t pbase = (kb >> 1) * 32 + (kb & 1) * 16;
                     // the K block's 16 saved (A, H) (or A_0): independent read-only loads first
                     // the K block's 16 consecutive points (pbase a multiple of 16): layer l - 1's records
-                    // as 4 + 8 16-byte loads, or A_0 (layer 0, whose tangents are W_0's columns)
+                    // as 4 + 6 16-byte loads, or A_0 (layer 0, whose tangents are W_0's columns)
                     float4 a4[4];
-                    uint4 h4[8];
+                    uint4 h4[6];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) a4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) h4[u] = make_uint4(0u, 0u, 0u, 0u);
+                    for (int u = 0; u < 6; ++u) h4[u] = make_uint4(0u, 0u, 0u, 0u);
                     if (pbase < a.n) {
                         if (l > 0) {
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                a4[u] = __ldg(reinterpret_cast<const float4*>(a.qa + rec_a(l - 1, a.np, W, pbase + 4 * u, k)));
+                            for (int u = 0; u < 4; ++u) a4[u] = __ldg(a.qa + rec_a(l - 1, a.np, W, pbase, k) + u * W);
 #pragma unroll
-                            for (int u = 0; u < 8; ++u)
-                                h4[u] = __ldg(reinterpret_cast<const uint4*>(a.qh + rec_h(l - 1, a.np, W, pbase + 2 * u, k)));
+                            for (int u = 0; u < 6; ++u) h4[u] = __ldg(a.qh + rec_h(l - 1, a.np, W, pbase, k) + u * W);
                         } else {
 #pragma unroll
                             for (int u = 0; u < 16; ++u) {
@@ -653,12 +652,10 @@ __global__ void __launch_bounds__(WgCfg<W>::THREADS) train_wgrad_tc_kernel(const
                         for (int e = 0; e < 2; ++e) {
                             const int64_t p = pbase + 2 * c + e;
                             const int ee = 2 * c + e;
-                            const uint4& hp = h4[ee >> 1];
-                            const float A = pick4(a4[ee >> 2], ee & 3);
                             // layer 0's tangents are W_0's columns (FP32); above, the saved H_l;
                             // points past the batch (the padding is never written) are zero
-                            float4 Q = l > 0 ? decode_q<F16>(A, (ee & 1) ? hp.z : hp.x, (ee & 1) ? hp.w : hp.y)
-                                             : make_float4(A, w0k.x, w0k.y, w0k.z);
+                            float4 Q = l > 0 ? decode_q<F16>(a4, h4, ee)
+                                             : make_float4(pick4(a4[ee >> 2], ee & 3), w0k.x, w0k.y, w0k.z);
                             if (p >= a.n) Q = make_float4(0.f, 0.f, 0.f, 0.f);
                             float sn = 0.0f, cs = 0.0f;
                             if (p < a.n) sincos_fast(Q.x, &sn, &cs);
@@ -765,8 +762,8 @@ cudaError_t backward_tc_w(const TrainArgs& a, int num_sms, cudaStream_t s) {
     t.d_f = a.d_f;
     t.d_grad = a.d_grad;
     t.a0 = a.w.z0;
-    t.qa = a.w.qa;
-    t.qh = a.w.qh;
+    t.qa = reinterpret_cast<const float4*>(a.w.qa);
+    t.qh = reinterpret_cast<const uint4*>(a.w.qh);
     t.np = rec_points(a.n);
     t.dtile = a.w.dtile;
     t.n_halves = a.w.n_halves;
