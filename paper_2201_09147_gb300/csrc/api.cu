@@ -1742,12 +1742,10 @@ int sdf_fit_loss(const float* f, const float* grad, const float* target_f, const
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     Scratch sc;
     sc.s = s;
-    cudaError_t e = cudaMallocFromPoolAsync(&sc.ptr, 64, di.pool, s);
+    cudaError_t e = cudaMallocFromPoolAsync(&sc.ptr, sizeof(FitScratch), di.pool, s);
     if (e != cudaSuccess) return cuda_fail(e, "allocating scratch");
-    double* sums = static_cast<double*>(sc.ptr);
-    auto* cnt = reinterpret_cast<unsigned long long*>(sums + 4);
-    e = launch_fit_loss(f, grad, target_f, target_grad, near, n, lam_n, lam_e, d_f, d_grad, sums, cnt, loss, di.num_sms,
-                        s);
+    e = launch_fit_loss(f, grad, target_f, target_grad, near, n, lam_n, lam_e, d_f, d_grad,
+                        static_cast<FitScratch*>(sc.ptr), loss, di.num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "launching the fitting objective");
     return SDF_OK;
 }

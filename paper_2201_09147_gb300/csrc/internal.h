@@ -189,9 +189,15 @@ cudaError_t launch_pack32_backward(const TrainArgs& a, int num_sms, cudaStream_t
 // Tensor-core training (16-bit operands: f16 = IEEE half, else bfloat16; FP32 accumulation).
 cudaError_t launch_train_forward_tc(const TrainArgs& a, bool f16, int num_sms, cudaStream_t s);
 cudaError_t launch_train_backward_tc(const TrainArgs& a, bool f16, int num_sms, cudaStream_t s);
+// Device scratch of one fit_loss call (zeroed by the launcher).
+struct FitScratch {
+    double sums[3];
+    unsigned long long n_near;
+    unsigned int ticket;
+};
 cudaError_t launch_fit_loss(const float* f, const float* grad, const float* tf, const float* tgrad,
                             const uint8_t* near, int64_t n, float lam_n, float lam_e, float* d_f, float* d_grad,
-                            double* sums, unsigned long long* n_near, double* out, int num_sms, cudaStream_t s);
+                            FitScratch* sc, double* out, int num_sms, cudaStream_t s);
 cudaError_t launch_adam(float* theta, const float* grad, float* m, float* v, int64_t count, float lr, float beta1,
                         float beta2, float eps, int step, int num_sms, cudaStream_t s);
 

@@ -210,13 +210,16 @@ __device__ __forceinline__ float sign_of(float x) { return x > 0.0f ? 1.0f : (x 
 //   value:      |f - g|                       -> sign(f - g) / n
 //   direction:  1 - <a, b> / (|a| |b|)  (near) -> -(b / (|a| |b|) - cos a / |a|^2) * lam_n / n_near
 //   Eikonal:    | |a| - 1 |                    -> sign(|a| - 1) a / |a| * lam_e / n
-// (a = grad f, b = the target gradient).  Sums of the terms go to sums[0..2].
+// (a = grad f, b = the target gradient).  Sums of the terms go to sums[0..2];
+// the last block to finish (*ticket, zero at launch) writes out = (mean |f - g|,
+// mean over near points of (1 - cos), mean | |grad f| - 1 |, total).
 __global__ void fit_loss_kernel(const float* __restrict__ f, const float* __restrict__ grad,
                                 const float* __restrict__ tf, const float* __restrict__ tgrad,
                                 const uint8_t* __restrict__ near, int64_t n, float lam_n, float lam_e,
                                 const unsigned long long* n_near, float* __restrict__ df, float* __restrict__ dgrad,
-                                double* sums) {
+                                double* sums, unsigned int* ticket, double* out) {
     __shared__ double red[3][8];
+    __shared__ bool last;
     const unsigned long long nn = *n_near;
     const float inv_n = 1.0f / static_cast<float>(n);
     const float dir_w = nn ? lam_n / static_cast<float>(nn) : 0.0f;
@@ -267,19 +270,21 @@ __global__ void fit_loss_kernel(const float* __restrict__ f, const float* __rest
         double t = 0.0;
         for (int k = 0; k < (blockDim.x >> 5); ++k) t += red[threadIdx.x][k];
         atomicAdd(&sums[threadIdx.x], t);
+        __threadfence();
     }
-}
-
-// out = (mean |f - g|, mean over near points of (1 - cos), mean | |grad f| - 1 |, total)
-__global__ void fit_loss_finalize_kernel(const double* sums, int64_t n, const unsigned long long* n_near, float lam_n,
-                                         float lam_e, double* out) {
-    const double lv = sums[0] / static_cast<double>(n);
-    const double ld = *n_near ? sums[1] / static_cast<double>(*n_near) : 0.0;
-    const double le = sums[2] / static_cast<double>(n);
-    out[0] = lv;
-    out[1] = ld;
-    out[2] = le;
-    out[3] = lv + static_cast<double>(lam_n) * ld + static_cast<double>(lam_e) * le;
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) + 1u == gridDim.x;
+    __syncthreads();
+    if (last && threadIdx.x == 0) {
+        __threadfence();
+        const double lv = __ldcg(sums) / static_cast<double>(n);
+        const double ld = nn ? __ldcg(sums + 1) / static_cast<double>(nn) : 0.0;
+        const double le = __ldcg(sums + 2) / static_cast<double>(n);
+        out[0] = lv;
+        out[1] = ld;
+        out[2] = le;
+        out[3] = lv + static_cast<double>(lam_n) * ld + static_cast<double>(lam_e) * le;
+    }
 }
 
 // Adam (Kingma and Ba): m <- b1 m + (1 - b1) g;  v <- b2 v + (1 - b2) g^2;
@@ -347,16 +352,15 @@ cudaError_t launch_fit_forward(const TrainArgs& a, int num_sms, cudaStream_t s) 
 
 cudaError_t launch_fit_loss(const float* f, const float* grad, const float* tf, const float* tgrad,
                             const uint8_t* near, int64_t n, float lam_n, float lam_e, float* d_f, float* d_grad,
-                            double* sums, unsigned long long* n_near, double* out, int num_sms, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(sums, 0, 3 * sizeof(double), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(n_near, 0, sizeof(unsigned long long), s);
+                            FitScratch* sc, double* out, int num_sms, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(sc, 0, sizeof(FitScratch), s);
     if (e != cudaSuccess) return e;
     int blocks = static_cast<int>((n + 255) / 256);
     if (blocks > 4 * num_sms) blocks = 4 * num_sms;
     if (blocks < 1) blocks = 1;
-    count_near_kernel<<<blocks, 256, 0, s>>>(near, n, n_near);
-    fit_loss_kernel<<<blocks, 256, 0, s>>>(f, grad, tf, tgrad, near, n, lam_n, lam_e, n_near, d_f, d_grad, sums);
-    fit_loss_finalize_kernel<<<1, 1, 0, s>>>(sums, n, n_near, lam_n, lam_e, out);
+    count_near_kernel<<<blocks, 256, 0, s>>>(near, n, &sc->n_near);
+    fit_loss_kernel<<<blocks, 256, 0, s>>>(f, grad, tf, tgrad, near, n, lam_n, lam_e, &sc->n_near, d_f, d_grad, sc->sums,
+                                           &sc->ticket, out);
     return cudaGetLastError();
 }
 

@@ -227,11 +227,14 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
     const float S = (e_bits == 0u) ? 1.0f : __uint_as_float(static_cast<uint32_t>(min(max(253 - static_cast<int>(e_bits), 1), 254)) << 23);
     const float invS = 1.0f / S;  // exact: a power of two
 
-    const long long n_pairs = (a.n + 2 * C::HPTS - 1) / (2 * C::HPTS);
+    // at most one half-tile per CTA: spread over the CTAs' halves 0, as in grad_tc_kernel
     const long long G = gridDim.x;
+    const int halves = a.n_halves <= G ? 1 : 2;
+    const long long n_pairs = a.n_halves / halves;
     const long long my_pairs = n_pairs > blockIdx.x ? (n_pairs - blockIdx.x + G - 1) / G : 0;
     constexpr int LAG = 1;
     const int n_groups = static_cast<int>(my_pairs) * KH;
+    const int n_groups1 = halves == 2 ? n_groups : 0;  // of half 1
     bool ok = true;
 
     if (warp == C::PRODUCER_WARP) {
@@ -241,7 +244,7 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int grp = k - h * LAG;
-                    if (grp < 0 || grp >= n_groups) continue;
+                    if (grp < 0 || grp >= (h == 1 ? n_groups1 : n_groups)) continue;
                     const int l = KH - 1 - grp % KH;  // layers from the top
                     for (int sg = 0; sg < C::STAGES_PER_LAYER && ok; ++sg, ++g) {
                         const uint32_t stage = g % C::NS, use = g / C::NS;
@@ -265,7 +268,7 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
 #pragma unroll
                 for (int h = 0; h < 2 && ok; ++h) {
                     const int grp = k - h * LAG;
-                    if (grp < 0 || grp >= n_groups) continue;
+                    if (grp < 0 || grp >= (h == 1 ? n_groups1 : n_groups)) continue;
                     ok = mbar_wait_bounded(bar_xready + 8u * h, xr_phase[h], a.status, abort_flag);
                     xr_phase[h] ^= 1u;
                     if (!ok) break;
@@ -308,8 +311,9 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
         const float4 w0m = live ? reinterpret_cast<const float4*>(w0s)[m] : make_float4(0.f, 0.f, 0.f, 0.f);
         const bool timed = a.pt_time != nullptr && IN == 4;
         uint32_t df_phase = 0;
-        for (long long i = 0; i < my_pairs; ++i) {
-            const long long T = (i * G + blockIdx.x) * 2 + h;  // half-tile of the batch
+        const long long pairs_h = h < halves ? my_pairs : 0;
+        for (long long i = 0; i < pairs_h; ++i) {
+            const long long T = (i * G + blockIdx.x) * halves + h;  // half-tile of the batch
             if (gt < C::HPTS) {
                 const long long k = T * C::HPTS + gt;
                 const int idx = k < a.n ? static_cast<int>(k) : -1;
@@ -554,53 +558,66 @@ __global__ void __launch_bounds__(WgCfg<W>::THREADS) train_wgrad_tc_kernel(const
                            ? 1.0f
                            : 1.0f / __uint_as_float(static_cast<uint32_t>(min(max(253 - static_cast<int>(e_bits), 1), 254)) << 23);
 
-    // K blocks (64 point-streams = 16 points) of every layer, split over the CTAs
-    const int64_t total = 2 * a.n_halves;
-    const int64_t per = (total + gridDim.x - 1) / gridDim.x;
-    const int64_t kb_lo = static_cast<int64_t>(blockIdx.x) * per;
-    const int64_t kb_hi = std::min<int64_t>(total, kb_lo + per);
+    // The K blocks (64 point-streams = 16 points) of all layers in a row, split evenly over the CTAs, so that a
+    // CTA adds its accumulator to dL/dtheta about as often as there are layers for a large batch, and once or
+    // twice for a small one (a (256,3) at 2,000 points: 152 additions of 256 KB instead of 384).  An
+    // accumulator takes at most kb_acc blocks: no more than a layer's share of a CTA, or 32.
+    const int64_t nkb = 2 * a.n_halves, total = nkb * KH;
+    const int64_t lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
+    const int64_t share = (nkb + gridDim.x - 1) / gridDim.x;
+    const int kb_acc = static_cast<int>(share > 32 ? share : 32);
     bool ok = true;
 
-    if (kb_hi > kb_lo) {
+    if (hi > lo) {
+        int l = static_cast<int>(lo / nkb);
+        int64_t kb = lo - l * nkb;
         if (warp == C::PRODUCER_WARP) {
             if (lane == 0) {
                 uint32_t g = 0;
-                for (int l = 0; l < KH && ok; ++l)
-                    for (int64_t kb = kb_lo; kb < kb_hi && ok; ++kb, ++g) {
-                        const uint32_t stage = static_cast<uint32_t>(g % C::NS), use = static_cast<uint32_t>(g / C::NS);
-                        if (use > 0) ok = mbar_wait_bounded(bar_empty + 8u * stage, (use - 1) & 1u, a.status, abort_flag);
-                        if (!ok) break;
-                        mbar_arrive_expect_tx(bar_full + 8u * stage, W * 128u);
-                        bulk_g2s(st_s + stage * C::STAGE,
-                                 a.dtile + (static_cast<size_t>(l) * a.n_halves + kb / 2) * (W * 256u) +
-                                     static_cast<size_t>(kb & 1) * (W * 128u),
-                                 W * 128u, bar_full + 8u * stage);
+                for (int64_t t = lo; t < hi && ok; ++t, ++g) {
+                    const uint32_t stage = g % C::NS, use = g / C::NS;
+                    if (use > 0) ok = mbar_wait_bounded(bar_empty + 8u * stage, (use - 1) & 1u, a.status, abort_flag);
+                    if (!ok) break;
+                    mbar_arrive_expect_tx(bar_full + 8u * stage, W * 128u);
+                    bulk_g2s(st_s + stage * C::STAGE,
+                             a.dtile + (static_cast<size_t>(l) * a.n_halves + kb / 2) * (W * 256u) +
+                                 static_cast<size_t>(kb & 1) * (W * 128u),
+                             W * 128u, bar_full + 8u * stage);
+                    if (++kb == nkb) {
+                        kb = 0;
+                        ++l;
                     }
+                }
                 for (uint32_t gg = g > C::NS ? g - C::NS : 0; gg < g; ++gg)
                     mbar_drain(bar_full + 8u * (gg % C::NS), (gg / C::NS) & 1u);
             }
         } else if (warp == C::MMA_WARP) {
             if (lane == 0) {
                 constexpr uint32_t idesc = idesc_f32acc(128, W, F16);
-                uint32_t g = 0;
-                for (int l = 0; l < KH && ok; ++l) {
-                    if (l > 0) ok = mbar_wait_bounded(bar_flushed, (l - 1) & 1u, a.status, abort_flag);
-                    for (int64_t kb = kb_lo; kb < kb_hi && ok; ++kb, ++g) {
-                        const uint32_t stage = static_cast<uint32_t>(g % C::NS), use = static_cast<uint32_t>(g / C::NS);
-                        ok = mbar_wait_bounded(bar_full + 8u * stage, use & 1u, a.status, abort_flag) &&
-                             mbar_wait_bounded(bar_xfull + 8u * stage, use & 1u, a.status, abort_flag);
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t sa = st_s + stage * C::STAGE, sx = sa + C::A_BYTES;
+                uint32_t g = 0, flushes = 0;
+                int in_acc = 0;
+                for (int64_t t = lo; t < hi && ok; ++t, ++g) {
+                    const uint32_t stage = g % C::NS, use = g / C::NS;
+                    if (in_acc == 0 && flushes > 0)
+                        ok = mbar_wait_bounded(bar_flushed, (flushes - 1) & 1u, a.status, abort_flag);
+                    ok = ok && mbar_wait_bounded(bar_full + 8u * stage, use & 1u, a.status, abort_flag) &&
+                         mbar_wait_bounded(bar_xfull + 8u * stage, use & 1u, a.status, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t sa = st_s + stage * C::STAGE, sx = sa + C::A_BYTES;
 #pragma unroll
-                        for (int mt = 0; mt < C::MT; ++mt)
+                    for (int mt = 0; mt < C::MT; ++mt)
 #pragma unroll
-                            for (int kk = 0; kk < 4; ++kk)
-                                mma_f16kind(tmem + mt * W, desc_kmajor_sw128(sa + mt * 16384u + kk * 32u),
-                                            desc_kmajor_sw128(sx + kk * 32u), idesc, (kb != kb_lo || kk != 0) ? 1u : 0u);
-                        mma_commit(bar_empty + 8u * stage);
+                        for (int kk = 0; kk < 4; ++kk)
+                            mma_f16kind(tmem + mt * W, desc_kmajor_sw128(sa + mt * 16384u + kk * 32u),
+                                        desc_kmajor_sw128(sx + kk * 32u), idesc, (in_acc | kk) != 0 ? 1u : 0u);
+                    mma_commit(bar_empty + 8u * stage);
+                    if (++kb == nkb) kb = 0;
+                    if (++in_acc == kb_acc || kb == 0 || t + 1 == hi) {
+                        mma_commit(bar_done);
+                        ++flushes;
+                        in_acc = 0;
                     }
-                    if (ok) mma_commit(bar_done);
                 }
             }
         } else {
@@ -609,70 +626,76 @@ __global__ void __launch_bounds__(WgCfg<W>::THREADS) train_wgrad_tc_kernel(const
             const int mt = warp >> 2, quad = warp & 3;
             const int nrow = mt * 128 + quad * 32 + lane;  // output unit of the TMEM lane read below
             const float4 w0k = reinterpret_cast<const float4*>(w0s)[k];
-            uint32_t g = 0;
-            for (int l = 0; l < KH && ok; ++l) {
-                for (int64_t kb = kb_lo; kb < kb_hi && ok; ++kb, ++g) {
-                    const uint32_t stage = static_cast<uint32_t>(g % C::NS), use = static_cast<uint32_t>(g / C::NS);
-                    if (use > 0)
-                        ok = __all_sync(0xffffffffu,
-                                        mbar_wait_bounded(bar_empty + 8u * stage, (use - 1) & 1u, a.status, abort_flag));
-                    if (!ok) break;
-                    const uint32_t sx = st_s + stage * C::STAGE + C::A_BYTES;
-                    const int64_t pbase = (kb >> 1) * 32 + (kb & 1) * 16;
-                    // the K block's 16 saved (A, H) (or A_0): independent read-only loads first
-                    // the K block's 16 consecutive points (pbase a multiple of 16): layer l - 1's records
-                    // as 4 + 6 16-byte loads, or A_0 (layer 0, whose tangents are W_0's columns)
-                    float4 a4[4];
-                    uint4 h4[6];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) a4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                    for (int u = 0; u < 6; ++u) h4[u] = make_uint4(0u, 0u, 0u, 0u);
-                    if (pbase < a.n) {
-                        if (l > 0) {
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) a4[u] = __ldg(a.qa + rec_a(l - 1, a.np, W, pbase, k) + u * W);
-#pragma unroll
-                            for (int u = 0; u < 6; ++u) h4[u] = __ldg(a.qh + rec_h(l - 1, a.np, W, pbase, k) + u * W);
-                        } else {
-#pragma unroll
-                            for (int u = 0; u < 16; ++u) {
-                                const float v0 = pbase + u < a.n ? __ldg(a.a0 + static_cast<size_t>(pbase + u) * W + k) : 0.0f;
-                                if ((u & 3) == 0) a4[u >> 2].x = v0;
-                                else if ((u & 3) == 1) a4[u >> 2].y = v0;
-                                else if ((u & 3) == 2) a4[u >> 2].z = v0;
-                                else a4[u >> 2].w = v0;
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        uint32_t w[4];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int64_t p = pbase + 2 * c + e;
-                            const int ee = 2 * c + e;
-                            // layer 0's tangents are W_0's columns (FP32); above, the saved H_l;
-                            // points past the batch (the padding is never written) are zero
-                            float4 Q = l > 0 ? decode_q<F16>(a4, h4, ee)
-                                             : make_float4(pick4(a4[ee >> 2], ee & 3), w0k.x, w0k.y, w0k.z);
-                            if (p >= a.n) Q = make_float4(0.f, 0.f, 0.f, 0.f);
-                            float sn = 0.0f, cs = 0.0f;
-                            if (p < a.n) sincos_fast(Q.x, &sn, &cs);
-                            w[2 * e] = pack16x2<F16>(sn, cs * Q.y);
-                            w[2 * e + 1] = pack16x2<F16>(cs * Q.z, cs * Q.w);
-                        }
-                        st_shared_v4(sx + (k >> 3) * 1024u + (k & 7) * 128u + ((c ^ (k & 7)) << 4), w[0], w[1], w[2],
-                                     w[3]);
-                    }
-                    fence_proxy_async_smem();
-                    mbar_arrive(bar_xfull + 8u * stage);
-                }
+            uint32_t g = 0, flushes = 0;
+            int in_acc = 0;
+            for (int64_t t = lo; t < hi && ok; ++t, ++g) {
+                const uint32_t stage = g % C::NS, use = g / C::NS;
+                if (use > 0)
+                    ok = __all_sync(0xffffffffu,
+                                    mbar_wait_bounded(bar_empty + 8u * stage, (use - 1) & 1u, a.status, abort_flag));
                 if (!ok) break;
-                ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_done, l & 1u, a.status, abort_flag));
+                const uint32_t sx = st_s + stage * C::STAGE + C::A_BYTES;
+                const int64_t pbase = (kb >> 1) * 32 + (kb & 1) * 16;
+                // the K block's 16 saved (A, H) (or A_0): independent read-only loads first
+                // the K block's 16 consecutive points (pbase a multiple of 16): layer l - 1's records
+                // as 4 + 6 16-byte loads, or A_0 (layer 0, whose tangents are W_0's columns)
+                float4 a4[4];
+                uint4 h4[6];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) a4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 6; ++u) h4[u] = make_uint4(0u, 0u, 0u, 0u);
+                if (pbase < a.n) {
+                    if (l > 0) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) a4[u] = __ldg(a.qa + rec_a(l - 1, a.np, W, pbase, k) + u * W);
+#pragma unroll
+                        for (int u = 0; u < 6; ++u) h4[u] = __ldg(a.qh + rec_h(l - 1, a.np, W, pbase, k) + u * W);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) {
+                            const float v0 = pbase + u < a.n ? __ldg(a.a0 + static_cast<size_t>(pbase + u) * W + k) : 0.0f;
+                            if ((u & 3) == 0) a4[u >> 2].x = v0;
+                            else if ((u & 3) == 1) a4[u >> 2].y = v0;
+                            else if ((u & 3) == 2) a4[u >> 2].z = v0;
+                            else a4[u >> 2].w = v0;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int64_t p = pbase + 2 * c + e;
+                        const int ee = 2 * c + e;
+                        // layer 0's tangents are W_0's columns (FP32); above, the saved H_l;
+                        // points past the batch (the padding is never written) are zero
+                        float4 Q = l > 0 ? decode_q<F16>(a4, h4, ee)
+                                         : make_float4(pick4(a4[ee >> 2], ee & 3), w0k.x, w0k.y, w0k.z);
+                        if (p >= a.n) Q = make_float4(0.f, 0.f, 0.f, 0.f);
+                        float sn = 0.0f, cs = 0.0f;
+                        if (p < a.n) sincos_fast(Q.x, &sn, &cs);
+                        w[2 * e] = pack16x2<F16>(sn, cs * Q.y);
+                        w[2 * e + 1] = pack16x2<F16>(cs * Q.z, cs * Q.w);
+                    }
+                    st_shared_v4(sx + (k >> 3) * 1024u + (k & 7) * 128u + ((c ^ (k & 7)) << 4), w[0], w[1], w[2],
+                                 w[3]);
+                }
+                fence_proxy_async_smem();
+                mbar_arrive(bar_xfull + 8u * stage);
+                const int layer = l;
+                if (++kb == nkb) {
+                    kb = 0;
+                    ++l;
+                }
+                if (++in_acc < kb_acc && kb != 0 && t + 1 < hi) continue;
+                in_acc = 0;
+                ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_done, flushes & 1u, a.status, abort_flag));
+                ++flushes;
                 if (!ok) break;
                 tc_fence_after();
-                float* gw = a.d_theta + sh.off_w[l];
+                float* gw = a.d_theta + sh.off_w[layer];
                 for (int cc = 0; cc < W / 32; ++cc) {
                     float v[32];
                     tmem_ld32(tmem + (static_cast<uint32_t>(quad * 32) << 16) + mt * W + cc * 32u, v);

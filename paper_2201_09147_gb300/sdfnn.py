@@ -448,7 +448,7 @@ def fit_loss(f, grad, target_f, target_grad, near, lam_n: float, lam_e: float, s
     n = f.shape[0]
     d_f = torch.empty_like(f)
     d_g = torch.empty_like(grad)
-    loss = torch.zeros(4, dtype=torch.float64, device=f.device)
+    loss = (torch.empty if n else torch.zeros)(4, dtype=torch.float64, device=f.device)  # written whole unless n = 0
     _check(lib().sdf_fit_loss(_ptr(f), _ptr(grad), _ptr(target_f), _ptr(target_grad), _ptr(near), n, float(lam_n),
                               float(lam_e), _ptr(d_f), _ptr(d_g), _ptr(loss), C.c_void_p(_stream(stream))))
     return d_f, d_g, loss
