@@ -18,8 +18,8 @@
 //   - train_bwd_tc_kernel walks a tile of 64 points from the top layer down:
 //     the epilogue threads (one per feature) form D_l from Y_l and the saved
 //     (A_l, H_l), store it in the MN-major 16-bit layout as the B operand of
-//     the MMA Y_{l-1} = W_l^T D_l (W_l^T streamed from L2 by bulk copies), and
-//     copy the same 16-byte chunks to a global tile image; the input layer
+//     the MMA Y_{l-1} = W_l^T D_l (W_l^T streamed from L2 by bulk copies); the
+//     MMA warp copies the same image to a global tile; the input layer
 //     ends in FP32 reductions for W_0, b_0 (and w_out, b_out at the top);
 //   - train_wgrad_tc_kernel splits every layer's point-streams over the CTAs:
 //     per K block of 64 point-streams it bulk-copies the D tile (a K-major A
@@ -274,6 +274,12 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t xh = x_s + h * (W * 256u);
+                    // D_l of the half is complete: its operand image to global memory as one bulk store, beside the
+                    // MMAs that read it
+                    bulk_s2g(a.dtile + (static_cast<size_t>(KH - 1 - grp % KH) * a.n_halves +
+                                        (static_cast<size_t>(grp / KH) * G + blockIdx.x) * halves + h) * (W * 256u),
+                             xh, W * 256u);
+                    bulk_commit();
                     for (int sg = 0; sg < C::STAGES_PER_LAYER && ok; ++sg, ++g) {
                         const uint32_t stage = g % C::NS, use = g / C::NS;
                         ok = mbar_wait_bounded(bar_full + 8u * stage, use & 1u, a.status, abort_flag);
@@ -295,8 +301,11 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
                         }
                         mma_commit(bar_empty + 8u * stage);
                     }
+                    // the epilogue that waits for this commit overwrites the image
+                    bulk_wait_read();
                     if (ok) mma_commit(bar_dfull + 8u * h);
                 }
+            bulk_wait();
         }
     } else {
         // epilogue group h: thread <-> feature row m (of the layer below the MMA), points 32h .. 32h+31
@@ -337,7 +346,6 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
                     if (!ok) break;
                     tc_fence_after();
                 }
-                uint8_t* dt = l >= 0 ? a.dtile + (static_cast<size_t>(l) * a.n_halves + T) * (W * 256u) : nullptr;
                 float s_b = 0.0f, s_o = 0.0f, s_w[4] = {0.0f, 0.0f, 0.0f, 0.0f};
                 for (int q = 0; q < C::HROWS / 32; ++q) {
                     // 32 accumulator columns (8 points x 4 streams) of Y; single-buffered: the
@@ -407,7 +415,6 @@ __global__ void __launch_bounds__(GradCfg<W, kOpBF16>::THREADS) train_bwd_tc_ker
                                 w[2 * e + 1] = pack16x2<F16>(y2 * cs, y3 * cs);
                             }
                             st_shared_v4(x_s + xoff16<W>(h, m, q * 4 + c), w[0], w[1], w[2], w[3]);
-                            *reinterpret_cast<uint4*>(dt + xoff16<W>(0, m, q * 4 + c)) = make_uint4(w[0], w[1], w[2], w[3]);
                         }
                     }
                     if (live && l < 0) {
