@@ -454,7 +454,7 @@ def main():
     nm_peak = pk["bf16_tflops_sustained"]
     roofline_nm = {"kernel": "grad_tc_kernel<256> (neural normal mapping, (256,3))", "bound": "tensor",
                    "achieved": nm_achieved, "peak": nm_peak, "unit": "TFLOP/s", "frac": nm_achieved / nm_peak,
-                   "traffic": traffic_tbl.get("grad_tc_kernel<256, 0, 0>"),
+                   "traffic": traffic_tbl.get("grad_tc_kernel<256, 0, 0, 0>"),
                    "peak_source": f"{pk['source']} bf16 sustained",
                    "work": f"{n_hit} points x {normal_flops_per_point} hidden-layer MMA flops"}
     if nm_ms >= tr_ms:

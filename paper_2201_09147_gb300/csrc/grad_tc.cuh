@@ -244,7 +244,7 @@ __device__ __forceinline__ void warp_sum32(float (&v)[32], int lane) {
 // faster).  Without it otherwise: the width-256 variants then allocate 96
 // registers (the cap of 18 warps, five of which share one scheduler's 16 K
 // registers) and spill, and the width-128 normal map measured 1 % slower.
-template <int W, int OP, bool TRAIN = false>
+template <int W, int OP, bool TRAIN = false, bool FEW = TRAIN>
 __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN || OP == kOpE4M3)) ? 1 : 0)
     grad_tc_kernel(const GradArgs a) {
     using C = GradCfg<W, OP>;
@@ -317,15 +317,16 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
     // b + 2G, ... (G = grid size) and half h of each pair is half-tile
     // 2 * pair + h.  Both halves run the same number of pairs, so the MMA warp
     // and the producer can follow the fixed schedule of grad_slot; a half-tile
-    // beyond the work is computed with no valid points.  Work of at most one
-    // half-tile per CTA is spread instead, a half-tile for each CTA's half 0:
-    // half 1 would take turns with it for the weights and the tensor core.  A
-    // call of 300 points of a (256,3), FP16: 22.8 us (5 CTAs streaming 768 KB of
-    // weights each) -> 14.4 us (10 CTAs, 384 KB, and no memset before the kernel).
+    // beyond the work is computed with no valid points.  With FEW, work of at
+    // most one half-tile per CTA is spread instead, a half-tile for each CTA's
+    // half 0: half 1 would take turns with it for the weights and the tensor
+    // core.  A call of 300 points of a (256,3), FP16: 22.8 us (5 CTAs streaming
+    // 768 KB of weights each) -> 14.4 us (10 CTAs, 384 KB, and no memset before
+    // the kernel).  The choice itself costs a large call 0.3 % (E4M3: 2.5 %), so
+    // the inference kernels have it in an instance of their own.
     const long long n_work = a.list ? static_cast<long long>(*a.count) : a.n;
     const long long G = gridDim.x;
-    constexpr bool kOne = !FP8;  // E4M3: the choice cost a large call 2.5 %
-    const int halves = kOne && n_work <= G * C::HPTS ? 1 : 2;
+    const int halves = FEW && n_work <= G * C::HPTS ? 1 : 2;
     const long long n_pairs = (n_work + halves * C::HPTS - 1) / (halves * C::HPTS);
     const long long my_pairs = n_pairs > blockIdx.x ? (n_pairs - blockIdx.x + G - 1) / G : 0;
     // MMA schedule: each half runs n_groups groups in order (per pair: the KH
@@ -354,7 +355,7 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int grp = k - h * LAG;
-                    if (grp < 0 || grp >= (kOne && h == 1 ? n_groups1 : n_groups)) continue;
+                    if (grp < 0 || grp >= (FEW && h == 1 ? n_groups1 : n_groups)) continue;
                     const int l = lh[h];
                     lh[h] = l + 1 == GPP ? 0 : l + 1;
                     for (int sg = 0; sg < C::STAGES_PER_LAYER && l < KH && ok; ++sg, ++g) {
@@ -384,7 +385,7 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
 #pragma unroll
                 for (int h = 0; h < 2 && ok; ++h) {
                     const int grp = k - h * LAG;
-                    if (grp < 0 || grp >= (kOne && h == 1 ? n_groups1 : n_groups)) continue;
+                    if (grp < 0 || grp >= (FEW && h == 1 ? n_groups1 : n_groups)) continue;
                     const int l = lh[h];
                     lh[h] = l + 1 == GPP ? 0 : l + 1;
                     ok = mbar_wait_bounded(bar_xready + 8u * h, xr_phase[h], a.status, abort_flag);
@@ -447,13 +448,13 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
         const float g0s = FP8 ? net.q_g[0] : 1.0f;
         const float wo = TRAIN && live ? __ldg(net.wout + m) : 0.0f;  // w_out of this feature (TRAIN)
         uint32_t df_phase = 0;
-        const long long pairs_h = kOne && h >= halves ? 0 : my_pairs;
+        const long long pairs_h = FEW && h >= halves ? 0 : my_pairs;
         // Point gt < HPTS of this half: its index is copied into shared memory
         // at the start of the pair before, its coordinates once that pair's
         // input layer has read the current ones, so no global load sits
         // between two pairs.
         if (gt < C::HPTS) {
-            const int idx = grad_point_index<C::HPTS, kOne>(a, n_work, halves, blockIdx.x, h, pairs_h > 0 ? gt : -1, 0);
+            const int idx = grad_point_index<C::HPTS, FEW>(a, n_work, halves, blockIdx.x, h, pairs_h > 0 ? gt : -1, 0);
             nidxs[p0 + gt] = idx;
             grad_point_async(base_s + L.pts + static_cast<uint32_t>(p0 + gt) * 16u, a, timed, idx);
         }
@@ -461,7 +462,7 @@ __global__ void __launch_bounds__(GradCfg<W, OP>::THREADS, (W < 256 && (TRAIN ||
             if (gt < C::HPTS) {
                 cp_async_wait_all();
                 idxs[p0 + gt] = nidxs[p0 + gt];
-                grad_point_index_async<C::HPTS, kOne>(base_s + L.nidx + static_cast<uint32_t>(p0 + gt) * 4u, a, n_work,
+                grad_point_index_async<C::HPTS, FEW>(base_s + L.nidx + static_cast<uint32_t>(p0 + gt) * 4u, a, n_work,
                                                 halves, blockIdx.x, h, i + 1 < pairs_h ? gt : -1, i + 1);
             }
             bar_named(1 + h, C::GROUP_THREADS);

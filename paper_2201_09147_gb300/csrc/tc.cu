@@ -521,6 +521,9 @@ template <int W, int OP>
 static cudaError_t launch_grad_op(const GradArgs& a, int num_sms, cudaStream_t s) {
     using C = GradCfg<W, OP>;
     const size_t smem = grad_layout<W, OP>(a.net.n_hidden).total + 1024;
+    // at most one half-tile per SM (an upper bound when a mask selects among the n points): the kernel that spreads
+    if (a.n <= static_cast<int64_t>(num_sms) * C::HPTS)
+        return launch_tc(grad_tc_kernel<W, OP, false, true>, C::THREADS, smem, C::TMEM_COLS, num_sms, s, &a);
     return launch_tc(grad_tc_kernel<W, OP>, C::THREADS, smem, C::TMEM_COLS, num_sms, s, &a);
 }
 
