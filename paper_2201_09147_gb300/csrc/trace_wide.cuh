@@ -140,8 +140,10 @@ __device__ __forceinline__ bool mbar_wait_spin(uint32_t bar, uint32_t parity, in
 
 // refill_ray, without the work counter once this CTA has seen it run out
 // (*dry): an atomic's round trip would delay every step in which a ray ends.
+// Other warps set *dry meanwhile and refill_ray is a collective of the warp, so
+// the warp decides as one: by what any of its lanes has read.
 __device__ __forceinline__ void wide_refill(const LevelArgs& a, Ray& r, long long n_work, volatile int* dry) {
-    if (*dry) {
+    if (__any_sync(0xffffffffu, *dry != 0)) {
         if (r.state == kSlotEmpty) r.state = kSlotDone;
         return;
     }
@@ -310,8 +312,9 @@ __global__ void __launch_bounds__(WideCfg<W, OP, SPLIT, TILES>::THREADS, 1) trac
                 if (lane == 0) act[slot >> 5] = any ? 1 : 0;
             }
             if (!bar_or(1, C::NRT, owner && ray.state == kSlotActive)) break;
-            if (C::ST == 2) {
-                // *dry and *left change before that barrier only: the same decision in every thread
+            if (C::ST == 2 && a.cap > 0) {
+                // *dry and *left change before that barrier only (another one follows this read): the same decision
+                // in every thread.  A level without steps has one barrier per turn and nothing to regroup.
                 if (regroup == 1 && tid == 0) *left = 0;
                 regroup = *dry == 0 ? 0 : regroup <= 1 ? kWideRegroup + (regroup == 0 ? 0 : 1) : regroup - 1;
             }
@@ -453,7 +456,8 @@ __global__ void __launch_bounds__(WideCfg<W, OP, SPLIT, TILES>::THREADS, 1) trac
                     }
                 }
                 const float f = ((acc01.x + acc01.y) + (acc23.x + acc23.y)) + net.bout;
-                if (good && *abort_flag == 0)
+                // step_ray is a collective of the warp, and another warp may set the flag between two lanes' reads
+                if (!__any_sync(0xffffffffu, !good || *abort_flag != 0))
                     step_ray(a, ray, f);
                 else
                     ray.state = kSlotDone;
