@@ -222,8 +222,10 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
         }
     } else if (warp == C::MMA_WARP) {
         if (lane == 0) {
-            constexpr uint32_t idesc_l = idesc_f32acc(128, C::HROWS, true) | kIdescMajorMnB;
-            constexpr uint32_t idesc_h = idesc_f32acc(128, 2 * C::HROWS, true) | kIdescMajorMnB;
+            // One accumulator and one shape per chain of MMAs: only such instructions are ordered among themselves.
+            // (Heads times both planes as one instruction of N = 256 over both accumulators would overlap the
+            // remainders' N = 128 with nothing between them.)
+            constexpr uint32_t idesc = idesc_f32acc(128, C::HROWS, true) | kIdescMajorMnB;
             uint32_t g = 0;
             for (int k = 0; k < n_groups && ok; ++k)
                 for (int h = 0; h < C::NH && ok; ++h) {
@@ -244,12 +246,14 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
                         for (int kk = 0; kk < 4; ++kk) {
                             const uint64_t wd = desc_add(wd0, kk * 32u);
                             const uint64_t xd = desc_add(xd0, static_cast<uint32_t>(kb * 8 + kk * 2) * 1024u);
-                            // the heads of W times both planes of X (h h' and h l', N = 256: the planes are
-                            // adjacent, as are the accumulators); the remainders of W times the heads of X
-                            if (!rem)
-                                mma_f16kind(d, wd, xd, idesc_h, (kb | kk) != 0);
-                            else
-                                mma_f16kind(d + 128u, wd, xd, idesc_l, 1u);
+                            // the heads of W times both planes of X (h h' and h l'); the remainders of W times
+                            // the heads of X
+                            if (!rem) {
+                                mma_f16kind(d, wd, xd, idesc, (kb | kk) != 0);
+                                mma_f16kind(d + 128u, wd, desc_add(xd, C::PLANE), idesc, (kb | kk) != 0);
+                            } else {
+                                mma_f16kind(d + 128u, wd, xd, idesc, 1u);
+                            }
                         }
                         mma_commit(bar_empty + 8u * stage);
                     }

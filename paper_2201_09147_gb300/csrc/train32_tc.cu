@@ -229,8 +229,8 @@ struct B32 {
     static_assert(TOTAL + 1024u <= 227u * 1024u, "shared memory");
 };
 
-// The warp roles and tiles of grad32_tc_kernel, run from the top layer down.  Bound by the MMAs (five
-// instructions per K step and TMEM tile, 384 clocks) and the reads of the saved (A, H), which are loaded a
+// The warp roles and tiles of grad32_tc_kernel, run from the top layer down.  Bound by the MMAs (six
+// instructions per K step and TMEM tile, 384 clocks at least) and the reads of the saved (A, H), which are loaded a
 // chunk of four points ahead.  Sums over the batch (biases, W_0, w_out) stay in registers of the thread that
 // owns the feature until the end.
 template <int W>
@@ -298,8 +298,8 @@ __global__ void __launch_bounds__(B32<W>::THREADS, 1) train32_bwd_kernel(const T
         }
     } else if (warp == C::MMA_WARP) {
         if (lane == 0) {
-            constexpr uint32_t idesc1 = idesc_f32acc(128, C::HROWS, false) | kIdescMajorMnB;
-            constexpr uint32_t idesc2 = idesc_f32acc(128, 2 * C::HROWS, false) | kIdescMajorMnB;
+            // (one accumulator and one shape per chain of MMAs, as in grad32_tc_kernel)
+            constexpr uint32_t idesc = idesc_f32acc(128, C::HROWS, false) | kIdescMajorMnB;
             uint32_t g = 0;
             for (int k = 0; k < n_groups && ok; ++k)
                 for (int h = 0; h < C::NH && ok; ++h) {
@@ -321,12 +321,13 @@ __global__ void __launch_bounds__(B32<W>::THREADS, 1) train32_bwd_kernel(const T
                                     const uint64_t wd = desc_add(wd0, kk * 32u);
                                     const uint64_t x0 = desc_add(xd0, static_cast<uint32_t>(kb * 8 + kk * 2) * 1024u);
                                     if (p == 0) {
-                                        // w0 d0 | w0 d1 (adjacent planes and accumulators), w0 d2
-                                        mma_f16kind(d, wd, x0, idesc2, (kb | kk) != 0);
-                                        mma_f16kind(d + 128u, wd, desc_add(x0, 2 * C::PLANE), idesc1, 1u);
+                                        // w0 d0; w0 d1, w0 d2
+                                        mma_f16kind(d, wd, x0, idesc, (kb | kk) != 0);
+                                        mma_f16kind(d + 128u, wd, desc_add(x0, C::PLANE), idesc, (kb | kk) != 0);
+                                        mma_f16kind(d + 128u, wd, desc_add(x0, 2 * C::PLANE), idesc, 1u);
                                     } else {
-                                        mma_f16kind(d + 128u, wd, x0, idesc1, 1u);  // w1 d0, w2 d0
-                                        if (p == 1) mma_f16kind(d + 128u, wd, desc_add(x0, C::PLANE), idesc1, 1u);
+                                        mma_f16kind(d + 128u, wd, x0, idesc, 1u);  // w1 d0, w2 d0
+                                        if (p == 1) mma_f16kind(d + 128u, wd, desc_add(x0, C::PLANE), idesc, 1u);
                                     }
                                 }
                                 mma_commit(bar_empty + 8u * stage);
@@ -586,7 +587,7 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
     // job and its last one.
     if (hi > lo && warp == C::BUILDERS / 32) {
         if (lane == 0) {
-            constexpr uint32_t idesc1 = idesc_f32acc(128, C::NB, false), idesc2 = idesc_f32acc(128, 2 * C::NB, false);
+            constexpr uint32_t idesc = idesc_f32acc(128, C::NB, false);
             uint32_t g = 0, flushes = 0;
             int in_acc = 0;
             for (int64_t t = lo; t < hi && ok; ++t, ++g) {
@@ -603,11 +604,12 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
                     const uint64_t a0 = desc_add(ad0, kk * 32u), x0 = desc_add(xd0, kk * 32u);
                     const uint64_t a1 = desc_add(a0, C::A_PLANE), a2 = desc_add(a0, 2 * C::A_PLANE);
                     const uint64_t x1 = desc_add(x0, C::X_PLANE), x2 = desc_add(x0, 2 * C::X_PLANE);
-                    mma_f16kind(tmem, a0, x0, idesc2, (in_acc | kk) != 0);  // a0 x0 | a0 x1 (adjacent planes)
-                    mma_f16kind(tmem + C::NB, a0, x2, idesc1, 1u);
-                    mma_f16kind(tmem + C::NB, a1, x0, idesc1, 1u);
-                    mma_f16kind(tmem + C::NB, a1, x1, idesc1, 1u);
-                    mma_f16kind(tmem + C::NB, a2, x0, idesc1, 1u);
+                    mma_f16kind(tmem, a0, x0, idesc, (in_acc | kk) != 0);
+                    mma_f16kind(tmem + C::NB, a0, x1, idesc, (in_acc | kk) != 0);
+                    mma_f16kind(tmem + C::NB, a0, x2, idesc, 1u);
+                    mma_f16kind(tmem + C::NB, a1, x0, idesc, 1u);
+                    mma_f16kind(tmem + C::NB, a1, x1, idesc, 1u);
+                    mma_f16kind(tmem + C::NB, a2, x0, idesc, 1u);
                 }
                 mma_commit(bar_empty + 8u * stage);
                 if (++in_acc == kFlush || t + 1 == hi || (t + 1) % nkb == 0) {

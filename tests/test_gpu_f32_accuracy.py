@@ -1,0 +1,72 @@
+"""FP32 gradients and training on the tensor cores against the same networks' FMA chains
+(sdf_fit_forward), on networks whose layers are far from those of an untrained SIREN.
+
+Tolerance.  Both paths share the layers' sines (their error) and the networks; the split operands miss a
+float by half a unit at most and their products are summed with fewer roundings than the chain's.  So the
+root mean square error against FP64 is at most 1.5 times the chain's (one and a half: two samples of errors
+of a size), plus u = 2^-24 of the gradients' root mean square for the roundings after the last layer.
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2201_09147_gb300 import inputs, sdfnn
+from test_gpu_f32_tc import reference_training
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -24
+
+
+def rms(x):
+    return float(np.sqrt(np.mean(np.square(x, dtype=np.float64))))
+
+
+def points(n, seed=5):
+    return (2.0 * inputs.uniform01(seed, 3 * n).reshape(3, n) - 1.0).astype(np.float32)
+
+
+def layers(shape, theta):
+    """Views of theta: the hidden layers' (W, b), and the weights that read each (the next layer's, or w_out)."""
+    d, w, k = shape
+    o, ws, bs = w * d + w, [], []
+    for _ in range(k):
+        ws.append(theta[o:o + w * w].reshape(w, w))
+        bs.append(theta[o + w * w:o + w * w + w])
+        o += w * w + w
+    return ws, bs, theta[o:o + w]
+
+
+def unbalanced(width, hidden, s):
+    """A SIREN in which one unit of every hidden layer has its weights times s and the weights that read it over s."""
+    shape, theta = sdfnn.theta_from_sdfn(inputs.net_to_bytes(inputs.siren_init(11, width, hidden)))
+    theta = theta.copy()
+    ws, _, out = layers(shape, theta)
+    for l in range(hidden):
+        j = (37 * l + 5) % width
+        ws[l][j] *= np.float32(s)
+        if l + 1 < hidden:
+            ws[l + 1][:, j] /= np.float32(s)
+        else:
+            out[j] /= np.float32(s)
+    return shape, theta
+
+
+@pytest.mark.parametrize("width,hidden", [(64, 3), (128, 2), (256, 2)])
+def test_repeated_calls_give_the_same_bits(sdf, width, hidden):
+    """The chains of products meet in a fixed order: nothing may depend on how instructions overlap.  (16 points: one
+    CTA adds to each entry of dL/dtheta.)"""
+    shape, theta = unbalanced(width, hidden, 1.0)
+    th, net = torch.from_numpy(theta).cuda(), sdf.Net(sdfnn.sdfn_from_theta(shape, theta), sdf.SDF_FP32)
+    for n in (16, 20011):
+        x = torch.from_numpy(points(n)).cuda()
+        c = torch.from_numpy((2.0 * inputs.uniform01(8, 4 * n) - 1.0).astype(np.float32)).cuda()
+        first = None
+        for _ in range(20):
+            f, g, ws = sdf.train_forward(shape, th, x)
+            out = [sdf.normals(net, x), f, g]
+            if n == 16:
+                out.append(sdf.train_backward(shape, th, x, c[:n].contiguous(), c[n:].reshape(3, n).contiguous(), ws))
+            first = first or out
+            assert all(torch.equal(a, b) for a, b in zip(out, first))
+    sdf.sync_status()
