@@ -271,6 +271,14 @@ __global__ void __launch_bounds__(WideCfg<W, OP, SPLIT, TILES>::THREADS, 1) trac
         bool issue_ok = true;  // the issuer: every weight unit so far arrived in time
         int regroup = 0;  // 0: the work lasts; else the steps to the next regrouping, + 1
         Ray ray;
+        // Few rays: in the first turn one warp of owners per CTA takes them, or two, ..., as far as the work needs: a
+        // CTA's step is shorter with fewer.  If work is left then (not every CTA has an SM yet), the others take part.
+        // With layer 0 below, the (64,1) coarse trace of 49 x 38 rays takes 79 us (first come, first served: 97;
+        // trace_level_tc_kernel: 93), of 64 x 64 78.5 (97; 109), the Lipschitz-stepped one of 32 x 32 64 (79; 95).
+        bool holds = static_cast<long long>(slot >> 5) * 32 * gridDim.x >= n_work;
+        // Layer 0 of a row is computed by warps of all four schedulers.  (TMEM lanes go by the warp's number, so the
+        // warps that read a row's accumulators share one, and late in a level few rows have a ray.)
+        const int row0 = (row + 32 * part) & 127, slot0 = tile * 128 + row0;
         // Stop decisions go through the ray threads' barrier: a timed-out wait drops the rays (the status
         // word reports it) instead of leaving the loop.
         while (true) {
@@ -305,7 +313,8 @@ __global__ void __launch_bounds__(WideCfg<W, OP, SPLIT, TILES>::THREADS, 1) trac
                 }
             }
             if (owner) {
-                wide_refill(a, ray, n_work, dry);
+                if (!holds) wide_refill(a, ray, n_work, dry);
+                holds = false;
                 const bool on = ray.state == kSlotActive;
                 pos[slot] = make_float4(ray.px, ray.py, ray.pz, timed && on ? __ldg(a.ray_time + ray.idx) : 0.0f);
                 const bool any = __any_sync(0xffffffffu, on);
@@ -323,8 +332,8 @@ __global__ void __launch_bounds__(WideCfg<W, OP, SPLIT, TILES>::THREADS, 1) trac
                 continue;
             }
             const bool wact = act[slot >> 5] != 0;  // rows of 32 slots without a ray are skipped (warp-uniform)
-            if (wact) {
-                const float4 p = pos[slot];
+            if (act[slot0 >> 5] != 0) {
+                const float4 p = pos[slot0];
                 const float2 px = make_float2(p.x, p.x), py = make_float2(p.y, p.y), pz = make_float2(p.z, p.z),
                              pt = make_float2(p.w, p.w);
 #pragma unroll 1
@@ -343,7 +352,7 @@ __global__ void __launch_bounds__(WideCfg<W, OP, SPLIT, TILES>::THREADS, 1) trac
                         v[2 * q] = sin_fast(z.x);
                         v[2 * q + 1] = sin_fast(z.y);
                     }
-                    wide_store16<C>(x_s, row, u0 + j * 16, v);
+                    wide_store16<C>(x_s, row0, u0 + j * 16, v);
                 }
             }
             fence_proxy_async_smem();

@@ -46,3 +46,24 @@ def test_levels_without_a_step_change_nothing(sdf, width, hidden, in_dim, precis
     after = trace([9, 0])
     assert not after[2].any()
     sdf.sync_status()
+
+
+@pytest.mark.parametrize("per_sm", [1, 31, 33, 64, 97])
+@pytest.mark.parametrize("width,hidden,in_dim,precision", CASES)
+def test_calls_of_few_rays_match_a_larger_call(sdf, width, hidden, in_dim, precision, per_sm):
+    """The fewer warps of a CTA take rays, at the edges of one, two, ... warps per CTA: the same bits as the same rays
+    among more.  (Rays of the first call that miss the box leave work for the warps that held back.)"""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n, whole = per_sm * sms + 3, 128 * sms
+    b = inputs.net_to_bytes(inputs.siren_init(5, width, hidden, in_dim=in_dim, out_scale=30.0, out_shift=0.1))
+    net = sdf.Net(b, getattr(sdf, precision))
+    orig, d, time = rays(whole, in_dim)
+
+    def trace(k):
+        return sdf.trace_multiscale([net], [0.0], [25], 1e-2, orig[:, :k].contiguous(), d[:, :k].contiguous(),
+                                    step_scale=[0.3], ray_time=None if time is None else time[:k].contiguous())
+
+    few, all_ = trace(n), trace(whole)
+    for x, y in zip(few, all_):
+        assert torch.equal(x, y[..., :n])
+    sdf.sync_status()
