@@ -351,7 +351,7 @@ void sdf_frame_queue_free(sdf_frame_queue_t queue);
  * sdf_train_shape_info: the length of theta and the workspace bytes the
  *   forward / backward pair needs for n points at that precision (either
  *   pointer may be NULL).  FP32: (1 + 8k) w floats per point plus copies of the hidden
- *   weights (14 bytes each); 16-bit: (1 + 5k) w floats per point
+ *   weights (16 bytes each); 16-bit: (1 + 5k) w floats per point
  *   plus two.
  * sdf_train_forward: f (n) and the unnormalised grad f (3, n) at pts (3, n)
  *   (pt_time (n) for 4-input networks, else NULL); saves the layers'

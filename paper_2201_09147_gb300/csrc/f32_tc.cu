@@ -6,8 +6,8 @@ namespace sdfnn {
 
 template <int W>
 static cudaError_t launch_grad32(const GradArgs& a, int num_sms, cudaStream_t s) {
-    return launch_tc(grad32_tc_kernel<W>, G32<W>::THREADS, g32_layout<W>().total + 1024, G32<W>::TMEM_COLS, num_sms, s,
-                     &a);
+    using C = G32<W, 2>;
+    return launch_tc(grad32_tc_kernel<W>, C::THREADS, g32_layout<C>().total + 1024, C::TMEM_COLS, num_sms, s, &a);
 }
 
 cudaError_t launch_grad32_tc(const GradArgs& a, int num_sms, cudaStream_t s) {

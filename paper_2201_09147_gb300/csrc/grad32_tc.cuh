@@ -1,23 +1,28 @@
 // Analytic-gradient kernel (Alg. 2) of the FP32 path on the tensor cores,
 // shared by normal mapping and the FP32 training forward.
 //
-// Every FP32 operand is held as two half-precision values, the rounding h and
-// the rounding l of the remainder x - h: 2 x 11 significand bits and the
-// remainder's sign, so the pair misses x by at most 2^-24 of its binade, the
-// half unit of a float.  A product is h h' + l h' + h l' (l l' is below
-// 2^-24), accumulated in FP32 by three tcgen05.mma per K step.
+// Normal mapping holds every FP32 operand as two half-precision values, the
+// rounding h and the rounding l of the remainder x - h: 2 x 11 significand bits
+// and the remainder's sign, so the pair misses x by at most 2^-24 of its binade,
+// the half unit of a float, while l stays a normal half.  A product is h h' +
+// l h' + h l' (l l' is below 2^-24), three tcgen05.mma per K step.
+//
+// The training forward, whose parameters only the device knows, holds them as
+// three bfloat16 values x0 + x1 + x2 instead (24 significand bits, a float's
+// exponents, no scales) and keeps the six products x_i y_j with i + j <= 2;
+// what is left out is below 2^-24 of the product.
 //
 // What decides the accuracy is the accumulation: the tensor core truncates
 // the running sum to 24 bits once per K step of 16 (measured with random
-// operands: the mean error has the sign opposite to the sum).  So h h' has its own accumulator (the
-// two small products would otherwise truncate the large sum two more times
-// per step), and the known mean of the truncation is multiplied back in
-// (kAccComp: the sums stay rounded by less than the FMA chain they replace).
-// Contractions of 128 x K sines with K x 64 uniform weights on GB300, root
-// mean square error against FP64 in units of 1e-7, for K = 64 / 128 / 256: a
-// chain of FP32 FMAs 1.8 / 3.7 / 7.2, one accumulator for all three products
-// 3.9 / 9.7 / 24.9, two accumulators 1.6 / 3.5 / 8.7, with kAccComp 1.4 / 2.4 /
-// 5.2.
+// operands: the mean error has the sign opposite to the sum).  So h h' (x0 y0)
+// has its own accumulator (the small products would otherwise truncate the
+// large sum two to five more times per step), and the known mean of the
+// truncation is multiplied back in (kAccComp: the sums stay rounded by less than
+// the FMA chain they replace).  Contractions of 128 x K sines with K x 64
+// uniform weights on GB300, halves, root mean square error against FP64 in units
+// of 1e-7, for K = 64 / 128 / 256: a chain of FP32 FMAs 1.8 / 3.7 / 7.2, one
+// accumulator for all three products 3.9 / 9.7 / 24.9, two accumulators 1.6 /
+// 3.5 / 8.7, with kAccComp 1.4 / 2.4 / 5.2.
 #pragma once
 
 #include "tc_common.cuh"
@@ -25,8 +30,11 @@
 namespace sdfnn {
 namespace {
 
-template <int W>
+// P operand planes: 2 halves (head, remainder) or 3 bfloat16 values.
+template <int W, int P>
 struct G32 {
+    static constexpr int PLANES = P;
+    static constexpr bool F16 = P == 2;
     static constexpr int MT = (W + 127) / 128;      // TMEM tiles of 128 feature rows
     static constexpr int KB = W / 64;               // 64-wide K blocks of the contraction
     static constexpr int ROWS_PAD = MT * 128;
@@ -35,31 +43,30 @@ struct G32 {
     static constexpr int HPTS = 32;
     static constexpr int CPTS = HPTS / CS;
     static constexpr int HROWS = 4 * HPTS;          // point-streams of a half = MMA N
-    static constexpr uint32_t PLANE = W * 256u;     // bytes of one operand plane of a half (h or l)
+    static constexpr uint32_t PLANE = W * 256u;     // bytes of one operand plane of a half
     // A ring unit is one plane of a K block for one TMEM tile (16 KB, consecutive in the weight image).
     static constexpr uint32_t UNIT = 16384u;
-    static constexpr int UNITS = KB * 2 * MT;       // units per layer
-    static constexpr int NS = 6;
+    static constexpr int UNITS = KB * P * MT;       // units per layer
+    static constexpr int NS = P == 2 || W == 64 ? 6 : 2;  // (three planes of 64 KB leave room for two units)
     static constexpr int GROUP_WARPS = 4 * MT * CS;
     static constexpr int GROUP_THREADS = GROUP_WARPS * 32;
     static constexpr int EPI_WARPS = NH * GROUP_WARPS;
     static constexpr int PRODUCER_WARP = EPI_WARPS;
     static constexpr int MMA_WARP = EPI_WARPS + 1;
     static constexpr int THREADS = (EPI_WARPS + 2) * 32;
-    static constexpr int TMEM_COLS = 512;           // (half or TMEM tile) * 256 + {0: h h', 128: l h' + h l'}
+    static constexpr int TMEM_COLS = 512;           // (half or TMEM tile) * 256 + {0: h h' or x0 y0, 128: the small products}
 };
 
 struct G32Layout {
     uint32_t x, ring, pts, bars, misc, total;
 };
 
-template <int W>
+template <class C>
 __host__ __device__ inline G32Layout g32_layout() {
-    using C = G32<W>;
     G32Layout L;
     uint32_t o = 0;
     L.x = o;
-    o += C::NH * 2u * C::PLANE;
+    o += C::NH * C::PLANES * C::PLANE;
     L.ring = o;
     o += C::NS * C::UNIT;
     L.pts = o;
@@ -73,13 +80,34 @@ __host__ __device__ inline G32Layout g32_layout() {
     return L;
 }
 
-// Two points (four streams each) of one feature as 16-byte chunks of the two planes.
-__device__ __forceinline__ void store_split8(uint32_t x_s, uint32_t plane, uint32_t off, const float (&v)[8]) {
-    uint32_t h[4], l[4];
+// Three bfloat16 planes of a pair of floats: the rounding of x, of x minus
+// that, and of what is left (the subtractions are exact).
+__device__ __forceinline__ void split3x2(float a, float b, uint32_t (&p)[3]) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) pack_split<true>(v[2 * e], v[2 * e + 1], h[e], l[e]);
-    st_shared_v4(x_s + off, h[0], h[1], h[2], h[3]);
-    st_shared_v4(x_s + plane + off, l[0], l[1], l[2], l[3]);
+    for (int i = 0; i < 3; ++i) {
+        p[i] = pack_bf16x2(a, b);
+        if (i < 2) {
+            const float2 r = __ffma2_rn(make_float2(__uint_as_float(p[i] << 16), __uint_as_float(p[i] & 0xFFFF0000u)),
+                                        make_float2(-1.0f, -1.0f), make_float2(a, b));
+            a = r.x;
+            b = r.y;
+        }
+    }
+}
+
+// Two points (four streams each) of one feature as 16-byte chunks of the P planes.
+template <int P>
+__device__ __forceinline__ void store_split(uint32_t x_s, uint32_t plane, uint32_t off, const float (&v)[8]) {
+    uint32_t q[4][P];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if constexpr (P == 2)
+            pack_split<true>(v[2 * e], v[2 * e + 1], q[e][0], q[e][1]);
+        else
+            split3x2(v[2 * e], v[2 * e + 1], q[e]);
+    }
+#pragma unroll
+    for (int i = 0; i < P; ++i) st_shared_v4(x_s + i * plane + off, q[0][i], q[1][i], q[2][i], q[3][i]);
 }
 
 // Byte offset in a half's MN-major plane of the chunk holding points 2c, 2c + 1 for feature m.
@@ -129,10 +157,44 @@ __device__ __forceinline__ void g32_point_async(uint32_t dst, const GradArgs& a,
         st_shared_u32(dst + 12u, 0u);
 }
 
+// The MMAs of one layer for one half: Y = W X in the ring's order of units (per K block the planes of W, per plane
+// the TMEM tiles).  d holds x0 y0, d + 128 the small products.  One accumulator and one shape per chain of MMAs:
+// only such instructions are ordered among themselves.  (The first plane times two planes of X as one instruction of
+// N = 256 over both accumulators would overlap the other products' N = 128 with nothing between them.)
+template <class C>
+__device__ __forceinline__ bool mma_layer32(uint32_t tmem, int h, uint64_t xd0, uint32_t ring_s, uint32_t bar_full,
+                                            uint32_t bar_empty, uint32_t& g, int* status, volatile int* abort_flag) {
+    constexpr uint32_t idesc = idesc_f32acc(128, C::HROWS, C::F16) | kIdescMajorMnB;
+    for (int kb = 0; kb < C::KB; ++kb)
+        for (int p = 0; p < C::PLANES; ++p)
+            for (int mt = 0; mt < C::MT; ++mt, ++g) {
+                const uint32_t stage = g % C::NS, use = g / C::NS;
+                if (!mbar_wait_bounded(bar_full + 8u * stage, use & 1u, status, abort_flag)) return false;
+                tc_fence_after();
+                const uint64_t wd0 = desc_kmajor_sw128(ring_s + stage * C::UNIT);
+                const uint32_t d = tmem + (mt + h) * 256u;
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const uint64_t wd = desc_add(wd0, kk * 32u);
+                    const uint64_t xd = desc_add(xd0, static_cast<uint32_t>(kb * 8 + kk * 2) * 1024u);
+                    if (p == 0) {
+                        mma_f16kind(d, wd, xd, idesc, (kb | kk) != 0);
+                        mma_f16kind(d + 128u, wd, desc_add(xd, C::PLANE), idesc, (kb | kk) != 0);
+                        if (C::PLANES == 3) mma_f16kind(d + 128u, wd, desc_add(xd, 2 * C::PLANE), idesc, 1u);
+                    } else {
+                        mma_f16kind(d + 128u, wd, xd, idesc, 1u);
+                        if (C::PLANES == 3 && p == 1) mma_f16kind(d + 128u, wd, desc_add(xd, C::PLANE), idesc, 1u);
+                    }
+                }
+                mma_commit(bar_empty + 8u * stage);
+            }
+    return true;
+}
+
 // Same skeleton as grad_tc_kernel (features as MMA rows, N = 32 points x 4
 // streams, a producer warp streaming the weights, an MMA warp, epilogue groups
-// that own a feature per thread), with these differences: operands in two
-// planes and two accumulators; at width 256 the two planes of one half fill
+// that own a feature per thread), with these differences: operands in
+// planes and two accumulators; at width 256 the planes of one half fill
 // the activation memory, so the CTA runs one half of 32 points (its MMAs, 6.1 k
 // clocks a layer, and epilogue, ~2 k, take turns; two halves of 16 points
 // would stream the weights twice and read them at N = 64, where shared-memory
@@ -151,15 +213,15 @@ __device__ __forceinline__ void g32_point_async(uint32_t dst, const GradArgs& a,
 // H_l^z) ([k][n][W] float4: a warp's store is 512 consecutive bytes) and also
 // writes f (no list, no normalisation).
 template <int W, bool TRAIN = false>
-__global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const GradArgs a) {
-    using C = G32<W>;
+__global__ void __launch_bounds__(G32<W, TRAIN ? 3 : 2>::THREADS, 1) grad32_tc_kernel(const GradArgs a) {
+    using C = G32<W, TRAIN ? 3 : 2>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t raw_s = smem_u32(smem_raw);
     const uint32_t base_s = (raw_s + 1023u) & ~1023u;
     uint8_t* base = smem_raw + (base_s - raw_s);
     const NetView& net = a.net;
     const int KH = net.n_hidden;
-    const G32Layout L = g32_layout<W>();
+    const G32Layout L = g32_layout<C>();
     const float4* pts = reinterpret_cast<const float4*>(base + L.pts);
     const uint32_t bar_full = base_s + L.bars;
     const uint32_t bar_empty = bar_full + 8u * C::NS;
@@ -222,41 +284,14 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
         }
     } else if (warp == C::MMA_WARP) {
         if (lane == 0) {
-            // One accumulator and one shape per chain of MMAs: only such instructions are ordered among themselves.
-            // (Heads times both planes as one instruction of N = 256 over both accumulators would overlap the
-            // remainders' N = 128 with nothing between them.)
-            constexpr uint32_t idesc = idesc_f32acc(128, C::HROWS, true) | kIdescMajorMnB;
             uint32_t g = 0;
             for (int k = 0; k < n_groups && ok; ++k)
                 for (int h = 0; h < C::NH && ok; ++h) {
                     ok = mbar_wait_bounded(bar_xready + 8u * h, k & 1, a.status, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t xd0 = desc_mnmajor_sw128(x_s + h * 2u * C::PLANE, W * 128u);
-                    for (int u = 0; u < C::UNITS && ok; ++u, ++g) {
-                        const uint32_t stage = g % C::NS, use = g / C::NS;
-                        ok = mbar_wait_bounded(bar_full + 8u * stage, use & 1u, a.status, abort_flag);
-                        if (!ok) break;
-                        tc_fence_after();
-                        const int mt = C::MT == 2 ? u & 1 : 0, kb = u / (2 * C::MT);
-                        const bool rem = ((u / C::MT) & 1) != 0;
-                        const uint64_t wd0 = desc_kmajor_sw128(ring_s + stage * C::UNIT);
-                        const uint32_t d = tmem + (mt + h) * 256u;
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            const uint64_t wd = desc_add(wd0, kk * 32u);
-                            const uint64_t xd = desc_add(xd0, static_cast<uint32_t>(kb * 8 + kk * 2) * 1024u);
-                            // the heads of W times both planes of X (h h' and h l'); the remainders of W times
-                            // the heads of X
-                            if (!rem) {
-                                mma_f16kind(d, wd, xd, idesc, (kb | kk) != 0);
-                                mma_f16kind(d + 128u, wd, desc_add(xd, C::PLANE), idesc, (kb | kk) != 0);
-                            } else {
-                                mma_f16kind(d + 128u, wd, xd, idesc, 1u);
-                            }
-                        }
-                        mma_commit(bar_empty + 8u * stage);
-                    }
+                    const uint64_t xd0 = desc_mnmajor_sw128(x_s + h * C::PLANES * C::PLANE, W * 128u);
+                    ok = mma_layer32<C>(tmem, h, xd0, ring_s, bar_full, bar_empty, g, a.status, abort_flag);
                     if (ok) mma_commit(bar_dfull + 8u * h);
                 }
         }
@@ -268,11 +303,11 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
         const bool live = mt * 128 + quad * 32 < W;  // warp-uniform
         const int gt = ge * 32 + lane;
         const uint32_t d_s = tmem + (static_cast<uint32_t>(quad * 32) << 16) + (mt + h) * 256u + cs * (C::CPTS * 4u);
-        const uint32_t xh = x_s + h * 2u * C::PLANE;
+        const uint32_t xh = x_s + h * C::PLANES * C::PLANE;
         const int p0 = h * C::HPTS, q0 = p0 + cs * C::CPTS;
         // output sums of the half: one row of HROWS floats per 32 features, in the half's activation
         // memory (free between the last MMA of a tile and the next tile's input layer)
-        float* red = reinterpret_cast<float*>(base + L.x + h * 2u * C::PLANE);
+        float* red = reinterpret_cast<float*>(base + L.x + h * C::PLANES * C::PLANE);
         const bool timed = a.pt_time != nullptr && net.in_dim == 4;
         float4 u0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         float ut = 0.0f, wo = 0.0f;
@@ -286,7 +321,7 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
                 u0.w = fmaf(wt, a.time, u0.w);
             wo = __ldg(net.wout + m);
         }
-        const float g0 = __ldg(net.s32 + 4 * kMaxHidden);
+        const float g0 = TRAIN ? 1.0f : __ldg(net.s32 + 4 * kMaxHidden);
         // Thread gt < HPTS holds the index of point gt; the next tile's index is loaded a tile ahead and its
         // coordinates are copied during this tile's layers, so no global load sits between two tiles.
         int idx = -1, nidx = -1;
@@ -323,7 +358,7 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
                         v[4 * e + 2] = u0.y * cn;
                         v[4 * e + 3] = u0.z * cn;
                     }
-                    store_split8(xh, C::PLANE, xoff32<W>(m, cs * (C::CPTS / 2) + c), v);
+                    store_split<C::PLANES>(xh, C::PLANE, xoff32<W>(m, cs * (C::CPTS / 2) + c), v);
                 }
             }
             fence_proxy_async_smem();
@@ -344,10 +379,11 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
                     continue;
                 }
                 const bool last = l + 1 == KH;
-                const float bb = __ldg(net.bh[l] + m), mf = __ldg(net.s32 + 4 * l);
+                constexpr float comp = static_cast<float>(1.0 + kAccComp * (W / 16));
+                const float bb = __ldg(net.bh[l] + m), mf = TRAIN ? comp : __ldg(net.s32 + 4 * l);
                 // the tangents' multiplier: to the scale of the next operand, or to values times w_out
-                const float mo = __ldg(net.s32 + 4 * l + 2);
-                const float mg = last ? wo * mo : __ldg(net.s32 + 4 * l + 1);
+                const float mo = TRAIN ? comp : __ldg(net.s32 + 4 * l + 2);
+                const float mg = last ? wo * mo : TRAIN ? comp : __ldg(net.s32 + 4 * l + 1);
                 float4* save = TRAIN ? reinterpret_cast<float4*>(a.save_a) + (static_cast<size_t>(l) * a.n + pb) * W + m : nullptr;
 #pragma unroll 1
                 for (int q = 0; q < C::CPTS / 4; ++q) {
@@ -377,8 +413,8 @@ __global__ void __launch_bounds__(G32<W>::THREADS, 1) grad32_tc_kernel(const Gra
                     } else {
                         const float(&lo8)[8] = *reinterpret_cast<const float(*)[8]>(&v[0]);
                         const float(&hi8)[8] = *reinterpret_cast<const float(*)[8]>(&v[8]);
-                        store_split8(xh, C::PLANE, xoff32<W>(m, cs * (C::CPTS / 2) + 2 * q), lo8);
-                        store_split8(xh, C::PLANE, xoff32<W>(m, cs * (C::CPTS / 2) + 2 * q + 1), hi8);
+                        store_split<C::PLANES>(xh, C::PLANE, xoff32<W>(m, cs * (C::CPTS / 2) + 2 * q), lo8);
+                        store_split<C::PLANES>(xh, C::PLANE, xoff32<W>(m, cs * (C::CPTS / 2) + 2 * q + 1), hi8);
                     }
                 }
                 fence_proxy_async_smem();

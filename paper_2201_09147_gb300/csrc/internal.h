@@ -153,12 +153,11 @@ struct TrainWork {
     // both paths
     float* z0;                     // [n][w] layer-0 pre-activations A_0
     uint8_t* wbf;                  // [k] W_l images (K-major, 128-byte swizzle, rows padded to 128): 16-bit, or FP32
-                                   // as two half planes per K block
-    uint8_t* wbft;                 // [k] W_l^T images, same layout: 16-bit, or FP32 as three bfloat16 planes per K block
+                                   // as three bfloat16 planes per K block
+    uint8_t* wbft;                 // [k] W_l^T images, same layout
     unsigned long long* counters;  // [4] tile counters
     // FP32 path
     float* wt;                     // [k][w][w] transposed hidden weights (fitting forward)
-    float* s32;                    // the scales of NetView::s32, and at + 64 the norms they come from
     float* z;                      // [k][n][w][4] per hidden layer: A_i and the tangent pre-images W_i G_{i-1}
     float* d;                      // [k][n][w][4] their adjoints (backward)
     // 16-bit path

@@ -1,18 +1,18 @@
 // FP32 training path on the tensor cores (SDF_FP32): the three kernels of
 // train_tc.cu with operands split so that the products keep FP32 accuracy.
 //
-//   forward:  grad32_tc_kernel<W, true> (half heads and remainders, scales from
-//             the parameters on the device); saves A_0 and (A_l, H_l) in FP32;
+//   forward:  grad32_tc_kernel<W, true>; saves A_0 and (A_l, H_l) in FP32;
 //   backward: train32_bwd_kernel, D_l = (dA_l, dH_l) from Y_l and the saved
 //             (A_l, H_l), then Y_{l-1} = W_l^T D_l;
 //   weights:  train32_wgrad_kernel, dW_l = sum over point-streams of D_l X_{l-1}^T.
 //
-// The adjoints span many binades (1 / n of the loss, growing and shrinking from
-// layer to layer and point to point), beyond a half's exponents.  So backward
-// and weight gradients split every FP32 operand into three bfloat16 values
-// x0 + x1 + x2 (24 significand bits, a float's exponent range) and keep the six
-// products x_i y_j with i + j <= 2; what is left out is below 2^-24 of the
-// product.  x0 y0 has an accumulator of its own (grad32_tc.cuh says why).
+// The parameters change from step to step and the adjoints span many binades
+// (1 / n of the loss, growing and shrinking from layer to layer and point to
+// point), beyond a half's exponents.  So all three split every FP32 operand into
+// three bfloat16 values x0 + x1 + x2 (24 significand bits, a float's exponent
+// range) and keep the six products x_i y_j with i + j <= 2; what is left out is
+// below 2^-24 of the product.  x0 y0 has an accumulator of its own
+// (grad32_tc.cuh says why).
 //
 // A fitting step takes its forward from train.cu (launch_fit_forward): its
 // objective is reported in double and shows the last bits of f.
@@ -39,23 +39,21 @@ size_t rows_pad_of(size_t W) { return W < 128 ? 128 : W; }
 
 }  // namespace
 
-// Scales, raw norms and counters, then the W_l images (two half planes), the
-// W_l^T images (three bfloat16 planes) and W_l^T in FP32, A_0, (A_l, H_l) and
-// (dA_l, dH_l).
+// Counters, then the W_l and W_l^T images (three bfloat16 planes each) and W_l^T
+// in FP32, A_0, (A_l, H_l) and (dA_l, dH_l).
 size_t train_workspace_bytes(const TrainShape& sh, int64_t n) {
     const size_t W = sh.width, k = sh.n_hidden, N = static_cast<size_t>(n), img = rows_pad_of(W) * W * 2;
-    return align256(2 * k * img) + align256(3 * k * img) + align256(k * W * W * 4) + align256(N * W * 4) + 2 * align256(k * N * 4 * W * 4) + 512;
+    return 2 * align256(3 * k * img) + align256(k * W * W * 4) + align256(N * W * 4) + 2 * align256(k * N * 4 * W * 4) + 256;
 }
 
 TrainWork train_work(const TrainShape& sh, int64_t n, void* ws) {
     const size_t W = sh.width, k = sh.n_hidden, N = static_cast<size_t>(n), img = rows_pad_of(W) * W * 2;
     uint8_t* p = static_cast<uint8_t*>(ws);
     TrainWork w{};
-    w.s32 = reinterpret_cast<float*>(p);
-    w.counters = reinterpret_cast<unsigned long long*>(p + 384);
-    p += 512;
+    w.counters = reinterpret_cast<unsigned long long*>(p);
+    p += 256;
     w.wbf = p;
-    p += align256(2 * k * img);
+    p += align256(3 * k * img);
     w.wbft = p;
     p += align256(3 * k * img);
     w.wt = reinterpret_cast<float*>(p);
@@ -70,21 +68,6 @@ TrainWork train_work(const TrainShape& sh, int64_t n, void* ws) {
 
 namespace {
 
-// Three bfloat16 planes of a pair of floats: the rounding of x, of x minus
-// that, and of what is left (the subtractions are exact).
-__device__ __forceinline__ void split3x2(float a, float b, uint32_t (&p)[3]) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        p[i] = pack_bf16x2(a, b);
-        if (i < 2) {
-            const float2 r = __ffma2_rn(make_float2(__uint_as_float(p[i] << 16), __uint_as_float(p[i] & 0xFFFF0000u)),
-                                        make_float2(-1.0f, -1.0f), make_float2(a, b));
-            a = r.x;
-            b = r.y;
-        }
-    }
-}
-
 // Two points (four streams each) of one feature as 16-byte chunks of the three planes.
 __device__ __forceinline__ void store_split3(uint32_t x_s, uint32_t plane, uint32_t off, const float4& a,
                                              const float4& b) {
@@ -98,96 +81,29 @@ __device__ __forceinline__ void store_split3(uint32_t x_s, uint32_t plane, uint3
 }
 
 // ---------------------------------------------------------------------------
-// weight images and scales
+// weight images
 // ---------------------------------------------------------------------------
-// norms[2 l] = max |W_l|, norms[2 l + 1] = max_r sum_k |W_l[r][k]| for the
-// hidden layers (one block each); norms[2 k] = max |W_0[:, 0..2]| (block k).
-__global__ void __launch_bounds__(1024) train32_norms_kernel(const float* __restrict__ theta, TrainShape sh,
-                                                             float* norms) {
-    __shared__ float red[2][32];
-    const int l = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = sh.width;
-    float amax = 0.0f, rmax = 0.0f;
-    if (l < sh.n_hidden) {
-        const float* Wl = theta + sh.off_w[l];
-        for (int r = warp; r < W; r += 32) {
-            float sum = 0.0f;
-            for (int k = lane; k < W; k += 32) {
-                const float x = fabsf(Wl[r * W + k]);
-                amax = fmaxf(amax, x);
-                sum += x;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            rmax = fmaxf(rmax, sum);
-        }
-    } else {
-        for (int i = tid; i < W * 3; i += blockDim.x) amax = fmaxf(amax, fabsf(theta[sh.off_w0 + (i / 3) * sh.in_dim + i % 3]));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    if (lane == 0) {
-        red[0][warp] = amax;
-        red[1][warp] = rmax;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        for (int w = 1; w < 32; ++w) {
-            amax = fmaxf(amax, red[0][w]);
-            rmax = fmaxf(rmax, red[1][w]);
-        }
-        norms[2 * l] = amax;
-        norms[2 * l + 1] = rmax;
-    }
-}
-
-// 14 - e for x < 2^e (14 for 0), kept to +-60: the exponent that scales x into [2^13, 2^14).
-__device__ __forceinline__ int scale_exponent(float x) {
-    const int e = static_cast<int>((__float_as_uint(x) >> 23) & 0xFFu) - 126;
-    return x > 0.0f ? min(max(14 - e, -60), 60) : 14;
-}
-
-__device__ __forceinline__ float exp2i(int e) { return __uint_as_float(static_cast<uint32_t>(e + 127) << 23); }
-
-// The scales of NetView::s32 (as the loader computes them for a network file),
-// and the images: W_l in two half planes per K block (rows = output units),
-// W_l^T in three bfloat16 planes (rows = inputs).  wimg NULL: the W_l^T images
-// only (norms and s32 are not used).
-__global__ void train32_pack_kernel(const float* __restrict__ theta, TrainShape sh, int rows_pad,
-                                    const float* __restrict__ norms, float comp, float* s32, uint8_t* wimg,
+// W_l (rows = output units) and W_l^T (rows = inputs) in three bfloat16 planes per K block.  wimg NULL: the W_l^T
+// images only.
+__global__ void train32_pack_kernel(const float* __restrict__ theta, TrainShape sh, int rows_pad, uint8_t* wimg,
                                     uint8_t* wtimg) {
-    const int W = sh.width, KH = sh.n_hidden;
-    if (wimg != nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
-        float bound = norms[2 * KH];
-        int ge = scale_exponent(bound);
-        s32[4 * kMaxHidden] = exp2i(ge);
-        for (int l = 0; l < KH; ++l) {
-            bound *= norms[2 * l + 1];
-            const int we = scale_exponent(norms[2 * l]), gn = scale_exponent(bound);
-            s32[4 * l] = comp * exp2i(-we);
-            s32[4 * l + 1] = comp * exp2i(min(max(gn - we - ge, -126), 126));
-            s32[4 * l + 2] = comp * exp2i(min(max(-we - ge, -126), 126));
-            ge = gn;
-        }
-    }
-    const int per = rows_pad * W, total = per * KH;
+    const int W = sh.width;
+    const int per = rows_pad * W, total = per * sh.n_hidden;
     const size_t block = static_cast<size_t>(rows_pad) * 128u;  // one plane of a K block
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const int l = i / per, r = (i % per) / W, k = i % W;
         const float* Wl = theta + sh.off_w[l];
-        uint32_t h = 0, hl = 0, t[3] = {0u, 0u, 0u};
+        uint32_t w[3] = {0u, 0u, 0u}, t[3] = {0u, 0u, 0u};
         if (r < W) {
-            if (wimg != nullptr) pack_split<true>(Wl[r * W + k] * exp2i(scale_exponent(norms[2 * l])), 0.0f, h, hl);
+            if (wimg != nullptr) split3x2(Wl[r * W + k], 0.0f, w);
             split3x2(Wl[k * W + r], 0.0f, t);
         }
-        const uint32_t off = sw128_offset(r, k & 63, rows_pad);
-        uint8_t* b = wtimg + (static_cast<size_t>(l) * (W / 64) + k / 64) * 3 * block + off;
-        if (wimg != nullptr) {
-            uint8_t* a = wimg + (static_cast<size_t>(l) * (W / 64) + k / 64) * 2 * block + off;
-            *reinterpret_cast<uint16_t*>(a) = static_cast<uint16_t>(h);
-            *reinterpret_cast<uint16_t*>(a + block) = static_cast<uint16_t>(hl);
-        }
+        const size_t at = (static_cast<size_t>(l) * (W / 64) + k / 64) * 3 * block + sw128_offset(r, k & 63, rows_pad);
 #pragma unroll
-        for (int p = 0; p < 3; ++p) *reinterpret_cast<uint16_t*>(b + p * block) = static_cast<uint16_t>(t[p]);
+        for (int p = 0; p < 3; ++p) {
+            if (wimg != nullptr) *reinterpret_cast<uint16_t*>(wimg + at + p * block) = static_cast<uint16_t>(w[p]);
+            *reinterpret_cast<uint16_t*>(wtimg + at + p * block) = static_cast<uint16_t>(t[p]);
+        }
     }
 }
 
@@ -212,19 +128,10 @@ struct Train32Args {
 // backward through the hidden layers and the input layer
 // ---------------------------------------------------------------------------
 template <int W>
-struct B32 {
-    using G = G32<W>;
-    static constexpr int MT = G::MT, KB = G::KB, NH = G::NH, HPTS = G::HPTS, CPTS = G::CPTS;
-    static constexpr int HROWS = G::HROWS;
-    static constexpr uint32_t PLANE = G::PLANE;     // one of the three planes of D of a half
-    static constexpr uint32_t UNIT = 16384u;        // one plane of a K block for one TMEM tile
-    static constexpr int UNITS = KB * 3 * MT;
-    static constexpr int NS = W == 64 ? 6 : 2;
-    static constexpr int GROUP_THREADS = G::GROUP_THREADS, GROUP_WARPS = G::GROUP_WARPS;
-    static constexpr int PRODUCER_WARP = G::PRODUCER_WARP, MMA_WARP = G::MMA_WARP, THREADS = G::THREADS;
-    static constexpr uint32_t X = NH * 3u * PLANE;
-    static constexpr uint32_t RING = X, ADJ = RING + NS * UNIT;
-    static constexpr uint32_t BARS = ADJ + NH * HPTS * 16u, MISC = BARS + (2 * NS + 2 * NH) * 8u;
+struct B32 : G32<W, 3> {
+    using G = G32<W, 3>;
+    static constexpr uint32_t RING = G::NH * 3u * G::PLANE, ADJ = RING + G::NS * G::UNIT;
+    static constexpr uint32_t BARS = ADJ + G::NH * G::HPTS * 16u, MISC = BARS + (2 * G::NS + 2 * G::NH) * 8u;
     static constexpr uint32_t TOTAL = MISC + 32u;
     static_assert(TOTAL + 1024u <= 227u * 1024u, "shared memory");
 };
@@ -298,8 +205,6 @@ __global__ void __launch_bounds__(B32<W>::THREADS, 1) train32_bwd_kernel(const T
         }
     } else if (warp == C::MMA_WARP) {
         if (lane == 0) {
-            // (one accumulator and one shape per chain of MMAs, as in grad32_tc_kernel)
-            constexpr uint32_t idesc = idesc_f32acc(128, C::HROWS, false) | kIdescMajorMnB;
             uint32_t g = 0;
             for (int k = 0; k < n_groups && ok; ++k)
                 for (int h = 0; h < C::NH && ok; ++h) {
@@ -307,31 +212,7 @@ __global__ void __launch_bounds__(B32<W>::THREADS, 1) train32_bwd_kernel(const T
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t xd0 = desc_mnmajor_sw128(base_s + h * 3u * C::PLANE, W * 128u);
-                    for (int kb = 0; kb < C::KB && ok; ++kb)
-                        for (int p = 0; p < 3 && ok; ++p)
-                            for (int mt = 0; mt < C::MT && ok; ++mt, ++g) {
-                                const uint32_t stage = g % C::NS, use = g / C::NS;
-                                ok = mbar_wait_bounded(bar_full + 8u * stage, use & 1u, a.status, abort_flag);
-                                if (!ok) break;
-                                tc_fence_after();
-                                const uint64_t wd0 = desc_kmajor_sw128(ring_s + stage * C::UNIT);
-                                const uint32_t d = tmem + (mt + h) * 256u;
-#pragma unroll
-                                for (int kk = 0; kk < 4; ++kk) {
-                                    const uint64_t wd = desc_add(wd0, kk * 32u);
-                                    const uint64_t x0 = desc_add(xd0, static_cast<uint32_t>(kb * 8 + kk * 2) * 1024u);
-                                    if (p == 0) {
-                                        // w0 d0; w0 d1, w0 d2
-                                        mma_f16kind(d, wd, x0, idesc, (kb | kk) != 0);
-                                        mma_f16kind(d + 128u, wd, desc_add(x0, C::PLANE), idesc, (kb | kk) != 0);
-                                        mma_f16kind(d + 128u, wd, desc_add(x0, 2 * C::PLANE), idesc, 1u);
-                                    } else {
-                                        mma_f16kind(d + 128u, wd, x0, idesc, 1u);  // w1 d0, w2 d0
-                                        if (p == 1) mma_f16kind(d + 128u, wd, desc_add(x0, C::PLANE), idesc, 1u);
-                                    }
-                                }
-                                mma_commit(bar_empty + 8u * stage);
-                            }
+                    ok = mma_layer32<C>(tmem, h, xd0, ring_s, bar_full, bar_empty, g, a.status, abort_flag);
                     if (ok) mma_commit(bar_dfull + 8u * h);
                 }
         }
@@ -726,11 +607,10 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
 
 float accumulation_comp(int W) { return static_cast<float>(1.0 + kAccComp * (W / 16)); }
 
-cudaError_t pack32(const TrainArgs& a, const float* norms, uint8_t* wimg, int num_sms, cudaStream_t s) {
+cudaError_t pack32(const TrainArgs& a, uint8_t* wimg, int num_sms, cudaStream_t s) {
     const int W = a.sh.width, rows_pad = static_cast<int>(rows_pad_of(W));
     const int blocks = std::min((rows_pad * W * a.sh.n_hidden + 255) / 256, 8 * num_sms);
-    train32_pack_kernel<<<blocks, 256, 0, s>>>(a.theta, a.sh, rows_pad, norms, accumulation_comp(W), a.w.s32, wimg,
-                                               a.w.wbft);
+    train32_pack_kernel<<<blocks, 256, 0, s>>>(a.theta, a.sh, rows_pad, wimg, a.w.wbft);
     return cudaGetLastError();
 }
 
@@ -738,9 +618,7 @@ template <int W>
 cudaError_t forward32_w(const TrainArgs& a, int num_sms, cudaStream_t s) {
     const TrainShape& sh = a.sh;
     const int rows_pad = static_cast<int>(rows_pad_of(W));
-    float* norms = a.w.s32 + 64;
-    train32_norms_kernel<<<sh.n_hidden + 1, 1024, 0, s>>>(a.theta, sh, norms);
-    cudaError_t e = pack32(a, norms, a.w.wbf, num_sms, s);
+    cudaError_t e = pack32(a, a.w.wbf, num_sms, s);
     if (e != cudaSuccess) return e;
     GradArgs ga{};
     ga.net.in_dim = sh.in_dim;
@@ -751,9 +629,8 @@ cudaError_t forward32_w(const TrainArgs& a, int num_sms, cudaStream_t s) {
     for (int l = 0; l < sh.n_hidden; ++l) ga.net.bh[l] = a.theta + sh.off_b[l];
     ga.net.wout = a.theta + sh.off_wout;
     ga.net.wbf = a.w.wbf;
-    ga.net.wbf_layer_bytes = static_cast<uint32_t>(rows_pad) * W * 4u;
+    ga.net.wbf_layer_bytes = static_cast<uint32_t>(rows_pad) * W * 6u;
     ga.net.rows_pad = rows_pad;
-    ga.net.s32 = a.w.s32;
     ga.pt_time = a.pt_time;
     ga.pts = a.pts;
     ga.n = a.n;
@@ -763,8 +640,8 @@ cudaError_t forward32_w(const TrainArgs& a, int num_sms, cudaStream_t s) {
     ga.save_a = a.w.z;
     ga.out_f = a.out_f;
     ga.out_bias = a.theta + sh.off_bout;
-    return launch_tc(grad32_tc_kernel<W, true>, G32<W>::THREADS, g32_layout<W>().total + 1024, G32<W>::TMEM_COLS, num_sms,
-                     s, &ga);
+    using C = G32<W, 3>;
+    return launch_tc(grad32_tc_kernel<W, true>, C::THREADS, g32_layout<C>().total + 1024, C::TMEM_COLS, num_sms, s, &ga);
 }
 
 template <int W>
@@ -792,7 +669,7 @@ cudaError_t backward32_w(const TrainArgs& a, int num_sms, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_pack32_backward(const TrainArgs& a, int num_sms, cudaStream_t s) {
-    return pack32(a, nullptr, nullptr, num_sms, s);
+    return pack32(a, nullptr, num_sms, s);
 }
 
 cudaError_t launch_train_forward(const TrainArgs& a, int num_sms, cudaStream_t s) {

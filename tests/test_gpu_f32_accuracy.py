@@ -52,6 +52,53 @@ def unbalanced(width, hidden, s):
     return shape, theta
 
 
+def small_layers(width, hidden, exponents):
+    """A SIREN with hidden layer l's weights and biases times 2^exponents[l]."""
+    shape, theta = sdfnn.theta_from_sdfn(inputs.net_to_bytes(inputs.siren_init(11, width, hidden)))
+    theta = theta.copy()
+    ws, bs, _ = layers(shape, theta)
+    for w, b, e in zip(ws, bs, exponents):
+        w *= np.float32(2.0 ** e)
+        b *= np.float32(2.0 ** e)
+    return shape, theta
+
+
+def compare_training(shape, theta, n=3001):
+    """f, grad f and dL/dtheta of sdf_train_forward / _backward are as near to FP64 as those of the FMA chains'
+    forward and the same backward."""
+    pts = points(n)
+    z = (2.0 * inputs.uniform01(8, 4 * n) - 1.0).astype(np.float32) / n
+    d_f, d_g = z[:n].copy(), z[n:].reshape(3, n).copy()
+    dev = lambda a: torch.from_numpy(a).cuda()
+    th, x = dev(theta), dev(pts)
+
+    def run(entry):
+        f, g, ws = sdfnn._forward(entry, shape, th, x, None, None, None, sdfnn.SDF_FP32)
+        d = sdfnn.train_backward(shape, th, x, dev(d_f), dev(d_g), ws)
+        return [t.cpu().numpy().astype(np.float64) for t in (f, g, d)]
+
+    tc, fma = run(sdfnn.lib().sdf_train_forward), run(sdfnn.lib().sdf_fit_forward)
+    sdfnn.sync_status()
+    ref = [t.cpu().numpy() for t in reference_training(shape, theta, pts, None, d_f, d_g)]
+    # (b_out, the last entry, is a plain sum of d_f in the order of atomics on both sides)
+    tc[2], fma[2], ref[2] = tc[2][:-1], fma[2][:-1], ref[2][:-1]
+    for name, a, b, r in zip(("f", "grad f", "dL/dtheta"), tc, fma, ref):
+        assert np.isfinite(a).all(), name
+        assert rms(a - r) <= 1.5 * rms(b - r) + U * rms(r), name
+
+
+@pytest.mark.parametrize("s", [1.0, 16.0, 32.0, 1024.0])
+@pytest.mark.parametrize("width,hidden", [(64, 2), (128, 3), (256, 4)])
+def test_training_of_unbalanced_networks(sdf, width, hidden, s):
+    compare_training(*unbalanced(width, hidden, s))
+
+
+# a layer at 2^-70 alone, and layers whose product is (beyond a half's exponents, or a scale of 2^60)
+@pytest.mark.parametrize("exponents", [(0, -70), (-40, -40), (-25, -25), (20, -50)])
+def test_training_of_small_layers(sdf, exponents):
+    compare_training(*small_layers(128, 2, exponents))
+
+
 @pytest.mark.parametrize("width,hidden", [(64, 3), (128, 2), (256, 2)])
 def test_repeated_calls_give_the_same_bits(sdf, width, hidden):
     """The chains of products meet in a fixed order: nothing may depend on how instructions overlap.  (16 points: one
