@@ -304,63 +304,108 @@ struct ParsedImage {
     float bout = 0.0f;
 };
 
-// FP32 operands as half-precision heads and remainders (grad32_tc.cuh), per
-// hidden layer and K block the heads and then the remainders, and the scales
-// of NetView::s32.  All scales are powers of two, so that only the operands'
-// own rounding remains: a layer's weights are scaled to a largest magnitude in
-// [2^13, 2^14); the tangents after layer l are scaled so that their bound
-// max|W_0| * prod ||W_i||_inf lies there too (the bound exceeds the tangents of
-// real networks by a few bits per layer, of the 28 that a half has below 2^14).
-// Returns false (nothing usable) when a scale would leave the range of a float:
-// such a network runs on the SIMT kernels.
+// FP32 operands as half-precision heads and remainders (grad32_tc.cuh): per
+// hidden layer and K block the heads and then the remainders, and the scales of
+// NetView::s32.  All scales are powers of two, so that only the operands' own
+// rounding remains.  Unit k of layer l has a bound b on its tangents, b_0[k] =
+// max_c |W_0[k][c]| and b_l[r] = sum_k |W_l[r][k]| b_{l-1}[k], below 2^e:
+//
+//   tangents  G[k] 2^(14 - e[k])                    below 2^14, never beyond a half;
+//   sines     P[k] 2^(14 + e_min - e[k])            the same weights serve both, so
+//   weights   W[r][k] 2^(e[k] + w[r])               the sines share the units' scales;
+//             w[r] puts the largest of the row into [2^13, 2^14).
+//
+// A power of two moved from a unit's input weights to its output weights
+// changes e[k] and nothing else.  The pair of halves keeps a float's accuracy
+// while a tangent is within 26 bits of its bound.  The bound exceeds the root of
+// the sum of squares by log2(sqrt(W)) = 4 bits per layer at most (Cauchy and
+// Schwarz), 16 for four layers of 256, which leaves 10 bits to cosines near zero.
+// The spread of e within a layer is taken from the sines (scale 2^14 down to
+// 2^(14 - spread)) and the weights: up to kSpread32 they too keep a float's accuracy.
+// Returns false (nothing usable) beyond that, or when a scale would leave the
+// range of a float: such a network runs on the SIMT kernels.
+constexpr int kSpread32 = 16;
+
 bool split_image32(const std::vector<std::vector<double>>& Wl, int IN, int W, int KH, int rows_pad,
-                   std::vector<uint8_t>* img, float* s32) {
+                   std::vector<uint8_t>* img, std::vector<float>* s32) {
     auto exponent = [](double x) {  // x < 2^e
         int e = 0;
         if (x > 0.0) std::frexp(x, &e);
         return e;
     };
-    double bound = 0.0;
-    for (int i = 0; i < W; ++i)
+    std::vector<double> b(W), bn(W);
+    std::vector<int> e(W);
+    int emin = 0;
+    bool ok = true;
+    // the exponents of the bounds b (a unit without tangents: the layer's largest), within what a scale can be
+    auto exponents = [&]() {
+        int emax = -1000;
+        emin = 1000;
+        for (int k = 0; k < W; ++k) {
+            ok = ok && std::isfinite(b[k]);
+            if (b[k] > 0.0) emax = std::max(emax, exponent(b[k]));
+        }
+        if (emax == -1000) emax = 0;
+        for (int k = 0; ok && k < W; ++k) {
+            e[k] = b[k] > 0.0 ? exponent(b[k]) : emax;
+            emin = std::min(emin, e[k]);
+        }
+        ok = ok && emax - emin <= kSpread32 && std::abs(14 - emax) <= 60 && std::abs(14 - emin) <= 60;
+    };
+    auto pow2 = [&](double c, int x) {
+        ok = ok && std::abs(x) <= 120;
+        return static_cast<float>(std::ldexp(c, x));
+    };
+    for (int k = 0; k < W; ++k) {
+        b[k] = 0.0;
         for (int c = 0; c < 3; ++c)
-            bound = std::max(bound, std::fabs(static_cast<double>(static_cast<float>(Wl[0][static_cast<size_t>(i) * IN + c]))));
-    int ge = 14 - exponent(bound);
-    bool ok = std::abs(ge) <= 60;
-    s32[4 * kMaxHidden] = std::ldexp(1.0f, ge);
+            b[k] = std::max(b[k], std::fabs(static_cast<double>(static_cast<float>(Wl[0][static_cast<size_t>(k) * IN + c]))));
+    }
+    exponents();
+    if (!ok) return false;
+    s32->assign(static_cast<size_t>(KH + 1) * W * 4, 0.0f);
+    for (int k = 0; k < W; ++k) {
+        (*s32)[4 * k] = pow2(1.0, 14 + emin - e[k]);
+        (*s32)[4 * k + 1] = pow2(1.0, 14 - e[k]);
+    }
     const size_t plane = static_cast<size_t>(rows_pad) * 128u, layer = 2 * plane * (W / 64);
     img->assign(KH * layer, 0);
     const double comp = 1.0 + kAccComp * (W / 16);
+    std::vector<int> w(W);
     for (int l = 1; l <= KH; ++l) {
-        double amax = 0.0, rmax = 0.0;
+        uint8_t* dst = img->data() + static_cast<size_t>(l - 1) * layer;
         for (int r = 0; r < W; ++r) {
-            double sum = 0.0;
+            double amax = 0.0;
+            bn[r] = 0.0;
             for (int k = 0; k < W; ++k) {
                 const double x = std::fabs(static_cast<double>(static_cast<float>(Wl[l][static_cast<size_t>(r) * W + k])));
-                amax = std::max(amax, x);
-                sum += x;
+                amax = std::max(amax, std::ldexp(x, e[k]));
+                bn[r] += x * b[k];
             }
-            rmax = std::max(rmax, sum);
-        }
-        const int we = 14 - exponent(amax);
-        bound *= rmax;
-        const int gn = 14 - exponent(bound);
-        ok = ok && std::isfinite(bound) && std::abs(we) <= 60 && std::abs(gn) <= 60;
-        if (!ok) return false;
-        s32[4 * (l - 1)] = static_cast<float>(std::ldexp(comp, -we));
-        s32[4 * (l - 1) + 1] = static_cast<float>(std::ldexp(comp, gn - we - ge));
-        s32[4 * (l - 1) + 2] = static_cast<float>(std::ldexp(comp, -we - ge));
-        s32[4 * (l - 1) + 3] = 0.0f;
-        ge = gn;
-        uint8_t* dst = img->data() + static_cast<size_t>(l - 1) * layer;
-        for (int r = 0; r < W; ++r)
+            ok = ok && std::isfinite(amax);
+            w[r] = amax > 0.0 ? 14 - exponent(amax) : 0;
+            ok = ok && std::abs(w[r]) <= 60;
+            if (!ok) return false;
             for (int k = 0; k < W; ++k) {
-                const float x = std::ldexp(static_cast<float>(Wl[l][static_cast<size_t>(r) * W + k]), we);
-                const __half hi = __float2half_rn(x), lo = __float2half_rn(x - __half2float(hi));
+                const float x = static_cast<float>(
+                    std::ldexp(static_cast<double>(static_cast<float>(Wl[l][static_cast<size_t>(r) * W + k])), e[k] + w[r]));
+                const __half hi = __float2half_rn(x), lo = __float2half_rn((x - __half2float(hi)) * 2048.0f);
                 const uint16_t hb = __half_as_ushort(hi), lb = __half_as_ushort(lo);
                 uint8_t* at = dst + static_cast<size_t>(k / 64) * 2 * plane + sw128_offset(r, k & 63, rows_pad);
                 std::memcpy(at, &hb, 2);
                 std::memcpy(at + plane, &lb, 2);
             }
+        }
+        const int sines = 14 + emin;
+        b.swap(bn);
+        if (l < KH) exponents();  // (the last layer's outputs are no operands)
+        if (!ok) return false;
+        for (int r = 0; r < W; ++r) {
+            float* q = s32->data() + (static_cast<size_t>(l) * W + r) * 4;
+            q[0] = pow2(comp, -w[r] - sines);
+            q[1] = pow2(comp, -w[r] - (l < KH ? e[r] : 14));
+            q[2] = l < KH ? pow2(1.0, 14 + emin - e[r]) : 1.0f;
+        }
     }
     return ok;
 }
@@ -523,12 +568,12 @@ int load_from_memory(const uint8_t* buf, size_t len, int precision, int device, 
         for (int l = 0; l <= KH; ++l) n->q_g[l] = static_cast<float>(gmax[l] > 0.0 ? 64.0 / gmax[l] : 1.0);
     }
 
-    float s32[kScales32] = {};
+    std::vector<float> s32;
     bool tc32 = false;
     if (precision == SDF_FP32) {
         n->rows_pad = W < 128 ? 128 : W;
         n->bf16_layer_bytes = static_cast<uint32_t>(n->rows_pad) * W * 4u;
-        tc32 = split_image32(Wl, IN, W, KH, n->rows_pad, &bf, s32);
+        tc32 = split_image32(Wl, IN, W, KH, n->rows_pad, &bf, &s32);
         if (!tc32) bf.clear();
     }
 
@@ -551,8 +596,8 @@ int load_from_memory(const uint8_t* buf, size_t len, int precision, int device, 
         if (e == cudaSuccess) e = cudaMemcpy(n->d_bf16, bf.data(), bf.size(), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess && tc32) {
-        e = cudaMalloc(&n->d_s32, sizeof(s32));
-        if (e == cudaSuccess) e = cudaMemcpy(n->d_s32, s32, sizeof(s32), cudaMemcpyHostToDevice);
+        e = cudaMalloc(&n->d_s32, s32.size() * sizeof(float));
+        if (e == cudaSuccess) e = cudaMemcpy(n->d_s32, s32.data(), s32.size() * sizeof(float), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
         free_net(n);

@@ -2,10 +2,12 @@
 // shared by normal mapping and the FP32 training forward.
 //
 // Normal mapping holds every FP32 operand as two half-precision values, the
-// rounding h and the rounding l of the remainder x - h: 2 x 11 significand bits
-// and the remainder's sign, so the pair misses x by at most 2^-24 of its binade,
-// the half unit of a float, while l stays a normal half.  A product is h h' +
-// l h' + h l' (l l' is below 2^-24), three tcgen05.mma per K step.
+// rounding h and the rounding l of 2^11 (x - h): 2 x 11 significand bits and the
+// remainder's sign, so the pair misses x by at most 2^-24 of its binade, the half
+// unit of a float, down to |x| = 2^-12 (below, by 2^-36).  A product is h h' +
+// 2^-11 (l h' + h l') (l l' is below 2^-24), three tcgen05.mma per K step.  The
+// operands are scaled by powers of two for it, unit by unit (split_image32 in
+// api.cu, which also says how far a unit's tangents may stay below their bound).
 //
 // The training forward, whose parameters only the device knows, holds them as
 // three bfloat16 values x0 + x1 + x2 instead (24 significand bits, a float's
@@ -80,6 +82,18 @@ __host__ __device__ inline G32Layout g32_layout() {
     return L;
 }
 
+// A remainder is held times 2^11: as large as its head, it is no smaller a half than the head is.
+constexpr float kRemScale = 2048.0f;
+
+// Two half planes of a pair of floats: the rounding of x and of 2^11 times what is left (exact, an FMA).
+__device__ __forceinline__ void split2x2(float a, float b, uint32_t (&p)[2]) {
+    p[0] = pack16x2<true>(a, b);
+    const float2 h = make_float2(from16<true>(static_cast<uint16_t>(p[0] & 0xFFFFu)),
+                                 from16<true>(static_cast<uint16_t>(p[0] >> 16)));
+    const float2 r = __ffma2_rn(h, make_float2(-kRemScale, -kRemScale), make_float2(a * kRemScale, b * kRemScale));
+    p[1] = pack16x2<true>(r.x, r.y);
+}
+
 // Three bfloat16 planes of a pair of floats: the rounding of x, of x minus
 // that, and of what is left (the subtractions are exact).
 __device__ __forceinline__ void split3x2(float a, float b, uint32_t (&p)[3]) {
@@ -102,7 +116,7 @@ __device__ __forceinline__ void store_split(uint32_t x_s, uint32_t plane, uint32
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         if constexpr (P == 2)
-            pack_split<true>(v[2 * e], v[2 * e + 1], q[e][0], q[e][1]);
+            split2x2(v[2 * e], v[2 * e + 1], q[e]);
         else
             split3x2(v[2 * e], v[2 * e + 1], q[e]);
     }
@@ -321,7 +335,11 @@ __global__ void __launch_bounds__(G32<W, TRAIN ? 3 : 2>::THREADS, 1) grad32_tc_k
                 u0.w = fmaf(wt, a.time, u0.w);
             wo = __ldg(net.wout + m);
         }
-        const float g0 = TRAIN ? 1.0f : __ldg(net.s32 + 4 * kMaxHidden);
+        // normal mapping: this feature's scales (split_image32 in api.cu), entry 0 for the input layer
+        const float4* scales = reinterpret_cast<const float4*>(net.s32) + m;
+        float4 sc = make_float4(1.0f, 1.0f, 1.0f, 0.0f);
+        if (!TRAIN && live) sc = __ldg(scales);
+        const float p_in = sc.x, g_in = sc.y;
         // Thread gt < HPTS holds the index of point gt; the next tile's index is loaded a tile ahead and its
         // coordinates are copied during this tile's layers, so no global load sits between two tiles.
         int idx = -1, nidx = -1;
@@ -340,7 +358,7 @@ __global__ void __launch_bounds__(G32<W, TRAIN ? 3 : 2>::THREADS, 1) grad32_tc_k
             // TRAIN: this thread's first point, and how many of its points are in the batch
             const long long pb = ((static_cast<long long>(i) * G + blockIdx.x) * C::NH + h) * C::HPTS + cs * C::CPTS;
             const int nv = TRAIN ? static_cast<int>(min(max(a.n - pb, 0ll), static_cast<long long>(C::CPTS))) : 0;
-            // input layer: P_0 = sin(A_0), G_0^c = W_0[:, c] (.) cos(A_0), the tangents at scale g0
+            // input layer: P_0 = sin(A_0), G_0^c = W_0[:, c] (.) cos(A_0), at the feature's scales
             if (live) {
 #pragma unroll 2
                 for (int c = 0; c < C::CPTS / 2; ++c) {
@@ -352,8 +370,8 @@ __global__ void __launch_bounds__(G32<W, TRAIN ? 3 : 2>::THREADS, 1) grad32_tc_k
                         if (TRAIN && 2 * c + e < nv) a.save_a0[(pb + 2 * c + e) * W + m] = z;
                         float sn, cn;
                         sincos_r(z, &sn, &cn);
-                        cn *= g0;
-                        v[4 * e] = sn;
+                        cn *= g_in;
+                        v[4 * e] = TRAIN ? sn : sn * p_in;
                         v[4 * e + 1] = u0.x * cn;
                         v[4 * e + 2] = u0.y * cn;
                         v[4 * e + 3] = u0.z * cn;
@@ -380,10 +398,11 @@ __global__ void __launch_bounds__(G32<W, TRAIN ? 3 : 2>::THREADS, 1) grad32_tc_k
                 }
                 const bool last = l + 1 == KH;
                 constexpr float comp = static_cast<float>(1.0 + kAccComp * (W / 16));
-                const float bb = __ldg(net.bh[l] + m), mf = TRAIN ? comp : __ldg(net.s32 + 4 * l);
-                // the tangents' multiplier: to the scale of the next operand, or to values times w_out
-                const float mo = TRAIN ? comp : __ldg(net.s32 + 4 * l + 2);
-                const float mg = last ? wo * mo : TRAIN ? comp : __ldg(net.s32 + 4 * l + 1);
+                // from the accumulators to A, from the tangents' to the next operand (the last layer: to values
+                // times w_out), and the next operand's scale of the sines
+                sc = TRAIN ? make_float4(comp, comp, 1.0f, 0.0f) : __ldg(scales + (l + 1) * W);
+                const float bb = __ldg(net.bh[l] + m), mg = last ? wo * sc.y : sc.y;
+                constexpr float lo = TRAIN ? 1.0f : 1.0f / kRemScale;
                 float4* save = TRAIN ? reinterpret_cast<float4*>(a.save_a) + (static_cast<size_t>(l) * a.n + pb) * W + m : nullptr;
 #pragma unroll 1
                 for (int q = 0; q < C::CPTS / 4; ++q) {
@@ -395,15 +414,15 @@ __global__ void __launch_bounds__(G32<W, TRAIN ? 3 : 2>::THREADS, 1) grad32_tc_k
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const int j = 4 * e;
-                        const float A = fmaf(v[j] + c[j], mf, bb);
 #pragma unroll
-                        for (int s = 1; s < 4; ++s) v[j + s] += c[j + s];
+                        for (int s = 0; s < 4; ++s) v[j + s] = fmaf(c[j + s], lo, v[j + s]);
+                        const float A = fmaf(v[j], sc.x, bb);
                         if (TRAIN && 4 * q + e < nv)
-                            save[(4 * q + e) * W] = make_float4(A, v[j + 1] * mo, v[j + 2] * mo, v[j + 3] * mo);
+                            save[(4 * q + e) * W] = make_float4(A, v[j + 1] * sc.y, v[j + 2] * sc.y, v[j + 3] * sc.y);
                         float sn, cn;
                         sincos_r(A, &sn, &cn);
                         cn *= mg;
-                        v[j] = TRAIN && last ? wo * sn : sn;
+                        v[j] = TRAIN ? (last ? wo * sn : sn) : sn * sc.z;
 #pragma unroll
                         for (int s = 1; s < 4; ++s) v[j + s] *= cn;
                     }

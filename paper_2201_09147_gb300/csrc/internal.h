@@ -8,7 +8,6 @@ namespace sdfnn {
 
 constexpr int kMaxHidden = 4;
 constexpr int kMaxLevels = 8;
-constexpr int kScales32 = 4 * kMaxHidden + 1;  // floats at NetView::s32
 
 // Mean relative truncation of the tensor core's FP32 accumulation (see
 // grad32_tc.cuh): each K step of 16 takes about kAccComp of the final sum.
@@ -37,10 +36,10 @@ struct NetView {
     float q_g[kMaxHidden + 1];
     float q_o;
     // FP32 networks on the tensor cores (s32 != NULL): wbf holds, per hidden layer and 64-wide K block, the
-    // half-precision heads and then the remainders of W_l * 2^w_l (each rows_pad x 128 bytes, 128-byte
-    // swizzle).  s32, device memory: [4 l] the multiplier from a layer-l accumulator to A, [4 l + 1] from a
-    // tangent accumulator to the tangent operand of layer l + 1, [4 l + 2] to W_l G_{l-1}; [4 kMaxHidden] the
-    // scale of the input layer's tangents.
+    // half-precision heads and then the remainders (times 2^11) of the scaled W_l (each rows_pad x 128 bytes,
+    // 128-byte swizzle).  s32, device memory: a float4 per layer and unit.  Input layer: (scale of the sine operand,
+    // of the tangent operands, -, -); hidden layers: (from the accumulator to A, from the tangents' accumulators to
+    // the next operand, at the last layer to W G; scale of the sine operand, -).
     // One slot for both, each read for its own precision only: eight more bytes of launch
     // parameters cost a 1080p trace 2.1 us of 495 (0.4 %).
     union {

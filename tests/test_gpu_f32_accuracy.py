@@ -117,3 +117,19 @@ def test_repeated_calls_give_the_same_bits(sdf, width, hidden):
             first = first or out
             assert all(torch.equal(a, b) for a, b in zip(out, first))
     sdf.sync_status()
+
+
+@pytest.mark.parametrize("s", [1.0, 16.0, 32.0, 1024.0, 2.0 ** 18])
+@pytest.mark.parametrize("width,hidden", [(64, 2), (128, 3), (256, 4)])
+def test_normals_of_unbalanced_networks(sdf, width, hidden, s):
+    """The last factor is beyond the scales of the split operands: the network runs on the FMA units."""
+    shape, theta = unbalanced(width, hidden, s)
+    pts = points(3001)
+    x = torch.from_numpy(pts).cuda()
+    g = sdf.normals(sdf.Net(sdfnn.sdfn_from_theta(shape, theta), sdf.SDF_FP32), x).cpu().numpy().astype(np.float64)
+    fma = sdfnn._forward(sdfnn.lib().sdf_fit_forward, shape, torch.from_numpy(theta).cuda(), x, None, None, None,
+                         sdfnn.SDF_FP32)[1].cpu().numpy().astype(np.float64)
+    sdf.sync_status()
+    zero = np.zeros(3001, np.float32)
+    ref = reference_training(shape, theta, pts, None, zero, np.zeros((3, 3001), np.float32))[1].cpu().numpy()
+    assert rms(g - ref) <= 1.5 * rms(fma - ref) + U * rms(ref)
