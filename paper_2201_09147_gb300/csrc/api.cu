@@ -370,8 +370,19 @@ bool split_image32(const std::vector<std::vector<double>>& Wl, int IN, int W, in
     }
     const size_t plane = static_cast<size_t>(rows_pad) * 128u, layer = 2 * plane * (W / 64);
     img->assign(KH * layer, 0);
-    const double comp = 1.0 + kAccComp * (W / 16);
     std::vector<int> w(W);
+    std::vector<double> sq(W), gain_p(W), gain_g(W);
+    // the correction of a row's sums (grad32_tc.cuh), from the squares of its terms' magnitudes
+    auto gain = [&]() {
+        double sum = 0.0, shares = 0.0;
+        for (int s = 0; s < W; s += 16) {
+            double step = 0.0;
+            for (int k = s; k < s + 16; ++k) step += sq[k];
+            sum += step;
+            if (step > 0.0) shares += sum;
+        }
+        return sum > 0.0 ? 1.0 + kStepLoss * (shares / sum) : 1.0;
+    };
     for (int l = 1; l <= KH; ++l) {
         uint8_t* dst = img->data() + static_cast<size_t>(l - 1) * layer;
         for (int r = 0; r < W; ++r) {
@@ -386,6 +397,13 @@ bool split_image32(const std::vector<std::vector<double>>& Wl, int IN, int W, in
             w[r] = amax > 0.0 ? 14 - exponent(amax) : 0;
             ok = ok && std::abs(w[r]) <= 60;
             if (!ok) return false;
+            // (squares of the scaled weights: no overflow, and what underflows does not matter)
+            for (int k = 0; k < W; ++k)
+                sq[k] = std::pow(std::ldexp(Wl[l][static_cast<size_t>(r) * W + k], emin + w[r]), 2);
+            gain_p[r] = gain();
+            for (int k = 0; k < W; ++k)
+                sq[k] = std::pow(std::ldexp(Wl[l][static_cast<size_t>(r) * W + k] * b[k], w[r]), 2);
+            gain_g[r] = gain();
             for (int k = 0; k < W; ++k) {
                 const float x = static_cast<float>(
                     std::ldexp(static_cast<double>(static_cast<float>(Wl[l][static_cast<size_t>(r) * W + k])), e[k] + w[r]));
@@ -402,8 +420,8 @@ bool split_image32(const std::vector<std::vector<double>>& Wl, int IN, int W, in
         if (!ok) return false;
         for (int r = 0; r < W; ++r) {
             float* q = s32->data() + (static_cast<size_t>(l) * W + r) * 4;
-            q[0] = pow2(comp, -w[r] - sines);
-            q[1] = pow2(comp, -w[r] - (l < KH ? e[r] : 14));
+            q[0] = pow2(gain_p[r], -w[r] - sines);
+            q[1] = pow2(gain_g[r], -w[r] - (l < KH ? e[r] : 14));
             q[2] = l < KH ? pow2(1.0, 14 + emin - e[r]) : 1.0f;
         }
     }

@@ -18,13 +18,20 @@
 // the running sum to 24 bits once per K step of 16 (measured with random
 // operands: the mean error has the sign opposite to the sum).  So h h' (x0 y0)
 // has its own accumulator (the small products would otherwise truncate the
-// large sum two to five more times per step), and the known mean of the
-// truncation is multiplied back in (kAccComp: the sums stay rounded by less than
-// the FMA chain they replace).  Contractions of 128 x K sines with K x 64
-// uniform weights on GB300, halves, root mean square error against FP64 in units
-// of 1e-7, for K = 64 / 128 / 256: a chain of FP32 FMAs 1.8 / 3.7 / 7.2, one
-// accumulator for all three products 3.9 / 9.7 / 24.9, two accumulators 1.6 /
-// 3.5 / 8.7, with kAccComp 1.4 / 2.4 / 5.2.
+// large sum two to five more times per step), and the mean of the truncation is
+// multiplied back in: a step takes about kStepLoss of the sum that it leaves, and
+// after step s of a row w that sum is, in the mean, sum_{k <= s} w_k^2 / sum w_k^2
+// of the whole.  So a row's gain is 1 + kStepLoss times the sum of these shares
+// over the steps in which it has weights: 8.5 kStepLoss = 2.7e-7 for a dense row
+// of 256, next to nothing for a row of a few weights, whose sums lose little.  (One
+// gain for all rows would be an error of its own there.)  Contractions of 128 x K
+// sines with K x 64 uniform weights on GB300, halves, root mean square error
+// against FP64 in units of 1e-7, for K = 64 / 128 / 256: a chain of FP32 FMAs 1.8 /
+// 3.7 / 7.2, one accumulator for all three products 3.9 / 9.7 / 24.9, two
+// accumulators 1.6 / 3.5 / 8.7, with the gain 1.4 / 2.4 / 5.2.  (h h' of the upper
+// half of K added to the complete small products instead, without a gain: 8
+// truncations per accumulator, gradients of the (256,3) up to 18 % further off and 6 %
+// slower.)
 #pragma once
 
 #include "tc_common.cuh"
@@ -397,10 +404,10 @@ __global__ void __launch_bounds__(G32<W, TRAIN ? 3 : 2>::THREADS, 1) grad32_tc_k
                     continue;
                 }
                 const bool last = l + 1 == KH;
-                constexpr float comp = static_cast<float>(1.0 + kAccComp * (W / 16));
+                const float gain = TRAIN ? __ldg(net.s32 + l * W + m) : 1.0f;
                 // from the accumulators to A, from the tangents' to the next operand (the last layer: to values
                 // times w_out), and the next operand's scale of the sines
-                sc = TRAIN ? make_float4(comp, comp, 1.0f, 0.0f) : __ldg(scales + (l + 1) * W);
+                sc = TRAIN ? make_float4(gain, gain, 1.0f, 0.0f) : __ldg(scales + (l + 1) * W);
                 const float bb = __ldg(net.bh[l] + m), mg = last ? wo * sc.y : sc.y;
                 constexpr float lo = TRAIN ? 1.0f : 1.0f / kRemScale;
                 float4* save = TRAIN ? reinterpret_cast<float4*>(a.save_a) + (static_cast<size_t>(l) * a.n + pb) * W + m : nullptr;

@@ -9,9 +9,9 @@ namespace sdfnn {
 constexpr int kMaxHidden = 4;
 constexpr int kMaxLevels = 8;
 
-// Mean relative truncation of the tensor core's FP32 accumulation (see
-// grad32_tc.cuh): each K step of 16 takes about kAccComp of the final sum.
-constexpr double kAccComp = 0.14 * 0x1p-23;
+// Mean relative truncation of the tensor core's FP32 accumulation: a K step of 16 takes this part of the sum that
+// it leaves (grad32_tc.cuh).
+constexpr double kStepLoss = 0.264 * 0x1p-23;
 
 // Device view of one prepared network (all pointers are device memory).
 struct NetView {
@@ -39,7 +39,8 @@ struct NetView {
     // half-precision heads and then the remainders (times 2^11) of the scaled W_l (each rows_pad x 128 bytes,
     // 128-byte swizzle).  s32, device memory: a float4 per layer and unit.  Input layer: (scale of the sine operand,
     // of the tangent operands, -, -); hidden layers: (from the accumulator to A, from the tangents' accumulators to
-    // the next operand, at the last layer to W G; scale of the sine operand, -).
+    // the next operand, at the last layer to W G; scale of the sine operand, -).  Training forward: s32 holds a
+    // float per hidden layer and unit, the correction of its sums (TrainWork::gain).
     // One slot for both, each read for its own precision only: eight more bytes of launch
     // parameters cost a 1080p trace 2.1 us of 495 (0.4 %).
     union {
@@ -157,6 +158,7 @@ struct TrainWork {
     unsigned long long* counters;  // [4] tile counters
     // FP32 path
     float* wt;                     // [k][w][w] transposed hidden weights (fitting forward)
+    float* gain;                   // [2][k][w] the truncation's correction per row of the W_l, then of the W_l^T
     float* z;                      // [k][n][w][4] per hidden layer: A_i and the tangent pre-images W_i G_{i-1}
     float* d;                      // [k][n][w][4] their adjoints (backward)
     // 16-bit path

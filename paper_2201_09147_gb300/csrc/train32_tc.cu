@@ -39,11 +39,11 @@ size_t rows_pad_of(size_t W) { return W < 128 ? 128 : W; }
 
 }  // namespace
 
-// Counters, then the W_l and W_l^T images (three bfloat16 planes each) and W_l^T
-// in FP32, A_0, (A_l, H_l) and (dA_l, dH_l).
+// Counters, then the W_l and W_l^T images (three bfloat16 planes each), their rows'
+// gains, W_l^T in FP32, A_0, (A_l, H_l) and (dA_l, dH_l).
 size_t train_workspace_bytes(const TrainShape& sh, int64_t n) {
     const size_t W = sh.width, k = sh.n_hidden, N = static_cast<size_t>(n), img = rows_pad_of(W) * W * 2;
-    return 2 * align256(3 * k * img) + align256(k * W * W * 4) + align256(N * W * 4) + 2 * align256(k * N * 4 * W * 4) + 256;
+    return 2 * align256(3 * k * img) + align256(2 * k * W * 4) + align256(k * W * W * 4) + align256(N * W * 4) + 2 * align256(k * N * 4 * W * 4) + 256;
 }
 
 TrainWork train_work(const TrainShape& sh, int64_t n, void* ws) {
@@ -56,6 +56,8 @@ TrainWork train_work(const TrainShape& sh, int64_t n, void* ws) {
     p += align256(3 * k * img);
     w.wbft = p;
     p += align256(3 * k * img);
+    w.gain = reinterpret_cast<float*>(p);
+    p += align256(2 * k * W * 4);
     w.wt = reinterpret_cast<float*>(p);
     p += align256(k * W * W * 4);
     w.z0 = reinterpret_cast<float*>(p);
@@ -83,20 +85,25 @@ __device__ __forceinline__ void store_split3(uint32_t x_s, uint32_t plane, uint3
 // ---------------------------------------------------------------------------
 // weight images
 // ---------------------------------------------------------------------------
-// W_l (rows = output units) and W_l^T (rows = inputs) in three bfloat16 planes per K block.  wimg NULL: the W_l^T
-// images only.
-__global__ void train32_pack_kernel(const float* __restrict__ theta, TrainShape sh, int rows_pad, uint8_t* wimg,
-                                    uint8_t* wtimg) {
-    const int W = sh.width;
+// W_l (rows = output units) and W_l^T (rows = inputs) in three bfloat16 planes per K block, and the correction of
+// each row's sums (grad32_tc.cuh).  wimg NULL: without the W_l images.  256 threads: a block's elements are whole
+// rows.
+__global__ void __launch_bounds__(256) train32_pack_kernel(const float* __restrict__ theta, TrainShape sh, int rows_pad,
+                                                           uint8_t* wimg, uint8_t* wtimg, float* gain) {
+    __shared__ float sq[2][16];  // sums of squares over 16 elements: W_l, W_l^T
+    const int W = sh.width, tid = threadIdx.x;
     const int per = rows_pad * W, total = per * sh.n_hidden;
     const size_t block = static_cast<size_t>(rows_pad) * 128u;  // one plane of a K block
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int l = i / per, r = (i % per) / W, k = i % W;
+    for (int i0 = blockIdx.x * 256; i0 < total; i0 += gridDim.x * 256) {
+        const int i = i0 + tid, l = i / per, r = (i % per) / W, k = i % W;
         const float* Wl = theta + sh.off_w[l];
         uint32_t w[3] = {0u, 0u, 0u}, t[3] = {0u, 0u, 0u};
+        float x = 0.0f, y = 0.0f;
         if (r < W) {
-            if (wimg != nullptr) split3x2(Wl[r * W + k], 0.0f, w);
-            split3x2(Wl[k * W + r], 0.0f, t);
+            x = Wl[r * W + k];
+            y = Wl[k * W + r];
+            split3x2(x, 0.0f, w);
+            split3x2(y, 0.0f, t);
         }
         const size_t at = (static_cast<size_t>(l) * (W / 64) + k / 64) * 3 * block + sw128_offset(r, k & 63, rows_pad);
 #pragma unroll
@@ -104,6 +111,45 @@ __global__ void train32_pack_kernel(const float* __restrict__ theta, TrainShape 
             if (wimg != nullptr) *reinterpret_cast<uint16_t*>(wimg + at + p * block) = static_cast<uint16_t>(w[p]);
             *reinterpret_cast<uint16_t*>(wtimg + at + p * block) = static_cast<uint16_t>(t[p]);
         }
+        // scaled by the row's largest, so that no square leaves a float's range
+        float mx = fabsf(x), my = fabsf(y);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, o));
+        }
+        if ((tid & 15) == 0) {
+            sq[0][tid >> 4] = mx;
+            sq[1][tid >> 4] = my;
+        }
+        __syncthreads();
+        const int s0 = tid / W * (W / 16);  // the row's first step in sq
+        for (int s = s0; s < s0 + W / 16; ++s) {
+            mx = fmaxf(mx, sq[0][s]);
+            my = fmaxf(my, sq[1][s]);
+        }
+        __syncthreads();
+        float vx = mx > 0.0f ? (x / mx) * (x / mx) : 0.0f, vy = my > 0.0f ? (y / my) * (y / my) : 0.0f;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            vx += __shfl_xor_sync(0xffffffffu, vx, o);
+            vy += __shfl_xor_sync(0xffffffffu, vy, o);
+        }
+        if ((tid & 15) == 0) {
+            sq[0][tid >> 4] = vx;
+            sq[1][tid >> 4] = vy;
+        }
+        __syncthreads();
+        if (k < 2 && r < W) {
+            float sum = 0.0f, shares = 0.0f;
+            for (int s = s0; s < s0 + W / 16; ++s) {
+                sum += sq[k][s];
+                if (sq[k][s] > 0.0f) shares += sum;
+            }
+            gain[(static_cast<size_t>(k) * sh.n_hidden + l) * W + r] =
+                sum > 0.0f ? 1.0f + static_cast<float>(kStepLoss) * (shares / sum) : 1.0f;
+        }
+        __syncthreads();
     }
 }
 
@@ -119,7 +165,7 @@ struct Train32Args {
     const float* a0;       // [n][W] A_0
     const float4* z;       // [k][n][W] (A_l, H_l^x, H_l^y, H_l^z)
     float4* d;             // [k][n][W] (dA_l, dH_l^x, dH_l^y, dH_l^z)
-    float comp;            // 1 + the mean relative truncation of a contraction over W
+    const float* gain;     // [k][W] the correction of a row's sums, W_l^T
     float* d_theta;
     int* status;
 };
@@ -265,6 +311,7 @@ __global__ void __launch_bounds__(B32<W>::THREADS, 1) train32_bwd_kernel(const T
                     tc_fence_after();
                 }
                 float sb = 0.0f, so = 0.0f;
+                const float gain = !top && live ? __ldg(a.gain + (l + 1) * W + m) : 1.0f;
 #pragma unroll 1
                 for (int q = 0; live && q < C::CPTS / 4; ++q) {
                     // Y of four points (16 columns); at the top w_out times the adjoints
@@ -284,7 +331,7 @@ __global__ void __launch_bounds__(B32<W>::THREADS, 1) train32_bwd_kernel(const T
                         tmem_ld16(d_s + 128u + q * 16u, c);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] = (v[j] + c[j]) * a.comp;
+                        for (int j = 0; j < 16; ++j) v[j] = (v[j] + c[j]) * gain;
                     }
                     float4 Z[4];
                     zp += 4 * W;
@@ -330,6 +377,7 @@ __global__ void __launch_bounds__(B32<W>::THREADS, 1) train32_bwd_kernel(const T
                 const float* ap = a.a0 + pb * W + m;
                 const float* xp = a.pts + pb;  // the points: the same address for the whole warp
                 float sb = 0.0f, sw[4] = {};   // sums over the tile first: shorter chains of roundings
+                const float gain = __ldg(a.gain + m);
 #pragma unroll 1
                 for (int q = 0; q < C::CPTS / 4; ++q) {
                     float A0[4];
@@ -341,7 +389,7 @@ __global__ void __launch_bounds__(B32<W>::THREADS, 1) train32_bwd_kernel(const T
                     tmem_ld16(d_s + 128u + q * 16u, c);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] = (v[j] + c[j]) * a.comp;
+                    for (int j = 0; j < 16; ++j) v[j] = (v[j] + c[j]) * gain;
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         if (4 * q + e >= nv) continue;  // Y is zero past the batch
@@ -417,7 +465,10 @@ struct Wg32 {
     static constexpr uint32_t BARS = NS * STAGE, MISC = BARS + (2 * NS + 2) * 8u, TOTAL = MISC + 32u;
 };
 constexpr int kFlush = 4;
-constexpr float kFlushComp = static_cast<float>(1.0 + kAccComp * (4 * kFlush));
+// The correction of a flush's sums over `steps` K steps of points (grad32_tc.cuh: terms of one size).
+__device__ __forceinline__ float flush_gain(int steps) {
+    return 1.0f + static_cast<float>(0.5 * kStepLoss) * static_cast<float>(steps + 1);
+}
 
 template <int W>
 __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(const Train32Args a) {
@@ -509,9 +560,11 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
         float acc[FC];
 #pragma unroll
         for (int j = 0; j < FC; ++j) acc[j] = 0.0f;
-        // the flush of the blocks multiplied so far; `job` >= 0 also adds the registers to dL/dtheta
+        // the flush of the blocks multiplied so far (`steps` K steps of points); `job` >= 0 also adds the registers
+        // to dL/dtheta
         uint32_t flushes = 0;
-        auto flush = [&](int64_t job) {
+        auto flush = [&](int64_t job, int steps) {
+            const float gain = flush_gain(steps);
             ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_done, flushes & 1u, a.status, abort_flag)) && ok;
             ++flushes;
             if (!ok) return;
@@ -523,7 +576,7 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
                 tmem_ld16(d_s + C::NB + j, c);
                 tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 16; ++e) acc[j + e] = fmaf(v[e] + c[e], kFlushComp, acc[j + e]);
+                for (int e = 0; e < 16; ++e) acc[j + e] = fmaf(v[e] + c[e], gain, acc[j + e]);
             }
             tc_fence_before();
             mbar_arrive(bar_flushed);
@@ -542,7 +595,7 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
             }
         };
         uint32_t g = 0;
-        int in_acc = 0;
+        int in_acc = 0, steps = 0, pending_steps = 0;
         int64_t pending = -2;  // the flush to run after the next build: -2 none, -1 to registers, >= 0 to that job
         for (int64_t t = lo; t < hi && ok; ++t, ++g) {
             const int64_t job = t / nkb, pbase = (t % nkb) * 16 + p_off;
@@ -585,16 +638,18 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
             fence_proxy_async_smem();
             mbar_arrive(bar_full + 8u * stage);
             if (pending != -2) {
-                flush(pending);
+                flush(pending, pending_steps);
                 pending = -2;
             }
             const bool job_end = t + 1 == hi || (t + 1) % nkb == 0;
+            steps += static_cast<int>(min(a.n - (t % nkb) * 16 + 3, static_cast<int64_t>(16)) / 4);
             if (++in_acc == kFlush || job_end) {
                 pending = job_end ? job : -1;
-                in_acc = 0;
+                pending_steps = steps;
+                in_acc = steps = 0;
             }
         }
-        if (ok && pending != -2) flush(pending);
+        if (ok && pending != -2) flush(pending, pending_steps);
     }
 
     tc_fence_before();
@@ -605,12 +660,10 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
     }
 }
 
-float accumulation_comp(int W) { return static_cast<float>(1.0 + kAccComp * (W / 16)); }
-
 cudaError_t pack32(const TrainArgs& a, uint8_t* wimg, int num_sms, cudaStream_t s) {
     const int W = a.sh.width, rows_pad = static_cast<int>(rows_pad_of(W));
     const int blocks = std::min((rows_pad * W * a.sh.n_hidden + 255) / 256, 8 * num_sms);
-    train32_pack_kernel<<<blocks, 256, 0, s>>>(a.theta, a.sh, rows_pad, wimg, a.w.wbft);
+    train32_pack_kernel<<<blocks, 256, 0, s>>>(a.theta, a.sh, rows_pad, wimg, a.w.wbft, a.w.gain);
     return cudaGetLastError();
 }
 
@@ -631,6 +684,7 @@ cudaError_t forward32_w(const TrainArgs& a, int num_sms, cudaStream_t s) {
     ga.net.wbf = a.w.wbf;
     ga.net.wbf_layer_bytes = static_cast<uint32_t>(rows_pad) * W * 6u;
     ga.net.rows_pad = rows_pad;
+    ga.net.s32 = a.w.gain;
     ga.pt_time = a.pt_time;
     ga.pts = a.pts;
     ga.n = a.n;
@@ -658,7 +712,7 @@ cudaError_t backward32_w(const TrainArgs& a, int num_sms, cudaStream_t s) {
     t.a0 = a.w.z0;
     t.z = reinterpret_cast<const float4*>(a.w.z);
     t.d = reinterpret_cast<float4*>(a.w.d);
-    t.comp = accumulation_comp(W);
+    t.gain = a.w.gain + static_cast<size_t>(a.sh.n_hidden) * W;
     t.d_theta = a.d_theta;
     t.status = a.status;
     cudaError_t e = launch_tc(train32_bwd_kernel<W>, B32<W>::THREADS, B32<W>::TOTAL + 1024, 512, num_sms, s, &t);

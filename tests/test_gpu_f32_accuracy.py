@@ -133,3 +133,86 @@ def test_normals_of_unbalanced_networks(sdf, width, hidden, s):
     zero = np.zeros(3001, np.float32)
     ref = reference_training(shape, theta, pts, None, zero, np.zeros((3, 3001), np.float32))[1].cpu().numpy()
     assert rms(g - ref) <= 1.5 * rms(fma - ref) + U * rms(ref)
+
+
+def permuted(width, hidden):
+    """Hidden layers that pass one unit on to one unit: contractions of a single product, where a correction of the
+    mean error of long sums would show as a gain."""
+    shape, theta = sdfnn.theta_from_sdfn(inputs.net_to_bytes(inputs.siren_init(11, width, hidden)))
+    theta = theta.copy()
+    for l, w in enumerate(layers(shape, theta)[0]):
+        w[:] = 0.0
+        w[np.arange(width), (5 * np.arange(width) + 3 * l) % width] = 0.75
+    return shape, theta
+
+
+# A product alone is rounded to within u of itself and a sum of such products in either direction: over k + 1 layers
+# the gain stays within u (k + 1) of the FMA chains' (the sines' error is common to both), with the backward's and
+# the weight gradients' contractions within 3 u (k + 1) of it.
+@pytest.mark.parametrize("width,hidden", [(64, 3), (128, 4), (256, 4)])
+def test_single_products_have_no_gain(sdf, width, hidden):
+    shape, theta = permuted(width, hidden)
+    n = 4096
+    pts = points(n)
+    z = (2.0 * inputs.uniform01(8, 4 * n) - 1.0).astype(np.float32) / n
+    d_f, d_g = z[:n].copy(), z[n:].reshape(3, n).copy()
+    dev = lambda a: torch.from_numpy(a).cuda()
+    th, x = dev(theta), dev(pts)
+    host = lambda t: t.cpu().numpy().astype(np.float64)
+    normals = host(sdf.normals(sdf.Net(sdfnn.sdfn_from_theta(shape, theta), sdf.SDF_FP32), x))
+    f, g, ws = sdf.train_forward(shape, th, x)
+    d = host(sdf.train_backward(shape, th, x, dev(d_f), dev(d_g), ws))
+    _, fma, _ = sdfnn._forward(sdfnn.lib().sdf_fit_forward, shape, th, x, None, None, None, sdfnn.SDF_FP32)
+    sdf.sync_status()
+    _, rg, rd = (t.cpu().numpy() for t in reference_training(shape, theta, pts, None, d_f, d_g))
+    gain = lambda a, r: float((a * r).sum() / (r * r).sum()) - 1.0
+    base, tol = gain(host(fma), rg), U * (hidden + 1)
+    assert abs(gain(normals, rg) - base) <= tol
+    assert abs(gain(host(g), rg) - base) <= tol
+    assert abs(gain(d, rd) - base) <= 3 * tol
+
+
+def test_accuracy_of_the_split_products(sdf):
+    """On untrained SIRENs of every width: gradients and training against the FMA chains, and every block of
+    dL/dtheta against a plain FP32 evaluation.  That one has the sines of the math library; the kernels' sines are
+    off by up to 8 u each, so a block may be off by 8 u (k + 1) of its root mean square more than twice its error."""
+    for width, hidden in [(64, 1), (128, 2), (256, 1), (256, 3)]:
+        shape, theta = unbalanced(width, hidden, 1.0)
+        compare_training(shape, theta, n=6001)
+        n = 6001
+        pts = points(n)
+        z = (2.0 * inputs.uniform01(8, 4 * n) - 1.0).astype(np.float32) / n
+        d_f, d_g = z[:n].copy(), z[n:].reshape(3, n).copy()
+        dev = lambda a: torch.from_numpy(a).cuda()
+        th, x = dev(theta), dev(pts)
+        _, _, ws = sdf.train_forward(shape, th, x)
+        d = sdf.train_backward(shape, th, x, dev(d_f), dev(d_g), ws).cpu().numpy().astype(np.float64)
+        plain = plain_training(shape, theta, pts, d_f, d_g).cpu().numpy().astype(np.float64)
+        ref = reference_training(shape, theta, pts, None, d_f, d_g)[2].cpu().numpy()
+        o, bounds = 0, []
+        for fan in [3] + [width] * hidden:
+            bounds += [(o, o + width * fan), (o + width * fan, o + width * fan + width)]
+            o += width * fan + width
+        bounds += [(o, o + width), (o + width, o + width + 1)]
+        for lo, hi in bounds[:-1]:  # (b_out is a plain sum of d_f)
+            r = ref[lo:hi]
+            assert rms(d[lo:hi] - r) <= 2.0 * rms(plain[lo:hi] - r) + 8 * U * (hidden + 1) * rms(r), (width, hidden, lo)
+
+
+def plain_training(shape, theta, pts, d_f, d_g):
+    """dL/dtheta in FP32 by torch's own operations."""
+    d, w, k = shape
+    torch.backends.cuda.matmul.allow_tf32 = False
+    th = torch.from_numpy(theta).cuda().requires_grad_(True)
+    o, h, g = 0, torch.from_numpy(pts).cuda(), None
+    for layer in range(k + 1):
+        fan = d if layer == 0 else w
+        W, b = th[o:o + w * fan].reshape(w, fan), th[o + w * fan:o + w * fan + w]
+        o += w * fan + w
+        z = W @ h + b[:, None]
+        c, h = torch.cos(z), torch.sin(z)
+        g = [W[:, i:i + 1] * c for i in range(3)] if layer == 0 else [(W @ t) * c for t in g]
+    f = th[o:o + w] @ h + th[o + w]
+    grad = torch.stack([th[o:o + w] @ t for t in g])
+    loss = (f * torch.from_numpy(d_f).cuda()).sum() + (grad * torch.from_numpy(d_g).cuda()).sum()
+    return torch.autograd.grad(loss, th)[0]
