@@ -725,10 +725,12 @@ void fill_trace_consts(const sdf_net* n, LevelArgs& la) {
 // Zeroes the 2 * kMaxLevels counters and launches the levels of Alg. 1 on
 // `s` (the validated parameters' device current); list0 / list1 hold n
 // entries each (unused with one level).  tiles: per-level tile counts for
-// the tensor-core kernel, or NULL.
+// the tensor-core kernel, or NULL.  overlapped: frames beside this one, on
+// another stream.
 int launch_levels_at(const sdf_trace_params* P, const float* orig, const float* dir, int64_t n, float* out_pos,
                      float* out_t, uint8_t* out_hit, uint16_t* out_iters, unsigned long long* counters,
-                     int32_t* list0, int32_t* list1, int* status, int num_sms, const int* tiles, cudaStream_t s) {
+                     int32_t* list0, int32_t* list1, int* status, int num_sms, const int* tiles, cudaStream_t s,
+                     bool overlapped = false) {
     const int m = P->n_levels;
     cudaError_t e = cudaMemsetAsync(counters, 0, 2 * kMaxLevels * sizeof(unsigned long long), s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(counters)");
@@ -762,7 +764,7 @@ int launch_levels_at(const sdf_trace_params* P, const float* orig, const float* 
         la.grab = &counters[j];
         la.status = status;
         if (net->width == kConstWidth) fill_trace_consts(net, la);
-        e = (net->precision != SDF_FP32) ? launch_trace_level_tc(la, num_sms, s)
+        e = (net->precision != SDF_FP32) ? launch_trace_level_tc(la, num_sms, s, overlapped)
                                          : launch_trace_level_simt(la, num_sms, s);
         if (e != cudaSuccess) return cuda_fail(e, "launching trace level");
     }
@@ -773,11 +775,11 @@ int launch_levels_at(const sdf_trace_params* P, const float* orig, const float* 
 // trace_scratch_bytes(m, n) bytes.
 int launch_levels(const sdf_trace_params* P, const float* orig, const float* dir, int64_t n, float* out_pos,
                   float* out_t, uint8_t* out_hit, uint16_t* out_iters, void* scratch, int* status, int num_sms,
-                  const int* tiles, cudaStream_t s) {
+                  const int* tiles, cudaStream_t s, bool overlapped = false) {
     auto* counters = static_cast<unsigned long long*>(scratch);
     int32_t* l0 = reinterpret_cast<int32_t*>(counters + 2 * kMaxLevels);
     return launch_levels_at(P, orig, dir, n, out_pos, out_t, out_hit, out_iters, counters, l0, l0 + n, status,
-                            num_sms, tiles, s);
+                            num_sms, tiles, s, overlapped);
 }
 
 int trace_impl(const sdf_trace_params* P, const float* orig, const float* dir, int64_t n, float* out_pos,
@@ -970,6 +972,7 @@ struct sdf_plan {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     size_t n_nodes = 0;
+    bool overlapped = false;    // a queue of several frames in flight launches it
 };
 
 namespace {
@@ -987,7 +990,7 @@ void free_plan(sdf_plan* p) {
 int plan_enqueue(sdf_plan* p, const int* tiles, int* status, int num_sms, cudaStream_t s) {
     const sdf_frame_batch& b = p->batch;
     int rc = launch_levels(&p->params, b.orig, b.dir, b.n, b.out_pos, b.out_t, b.out_hit, b.out_iters, p->scratch,
-                           status, num_sms, tiles, s);
+                           status, num_sms, tiles, s, p->overlapped);
     if (rc || !p->fine) return rc;
     return launch_gradients(p->fine, b.out_pos, b.ray_time, b.out_hit, b.n, b.out_normal, 1,
                             static_cast<uint8_t*>(p->scratch) + p->trace_bytes, status, num_sms, s);
@@ -1022,7 +1025,7 @@ int plan_autotune(sdf_plan* p, int* status, int num_sms, cudaStream_t s) {
             for (int rep = 0; rep < 3 && rc == SDF_OK; ++rep) {
                 cudaEventRecord(e0, s);
                 rc = launch_levels(&p->params, b.orig, b.dir, b.n, b.out_pos, b.out_t, b.out_hit, b.out_iters,
-                                   p->scratch, status, num_sms, p->tiles, s);
+                                   p->scratch, status, num_sms, p->tiles, s, p->overlapped);
                 cudaEventRecord(e1, s);
                 if ((e = cudaEventSynchronize(e1)) != cudaSuccess) rc = cuda_fail(e, "autotune run");
                 float ms = 0.0f;
@@ -1042,7 +1045,7 @@ int plan_autotune(sdf_plan* p, int* status, int num_sms, cudaStream_t s) {
 }
 
 int plan_create(const sdf_trace_params* P, sdf_net_t fine, const sdf_frame_batch* B, int autotune,
-                cudaStream_t s, sdf_plan_t* out) {
+                cudaStream_t s, sdf_plan_t* out, bool overlapped = false) {
     if (!out) return fail(SDF_ERR_ARG, "out is NULL");
     *out = nullptr;
     if (!B) return fail(SDF_ERR_ARG, "batch is NULL");
@@ -1083,6 +1086,7 @@ int plan_create(const sdf_trace_params* P, sdf_net_t fine, const sdf_frame_batch
     p->params.step_scale = Q.step_scale ? p->step_scale : nullptr;
     p->fine = fine;
     p->batch = *B;
+    p->overlapped = overlapped;
     if (B->n == 0) {
         *out = p;
         return SDF_OK;
@@ -1341,7 +1345,7 @@ int queue_create(const sdf_trace_params* P, sdf_net_t fine, int64_t n, int depth
         fb.out_t = sl.t;
         fb.out_hit = sl.hit;
         fb.out_normal = sl.nrm;
-        rc = plan_create(P, fine, &fb, 0, q->cmp[0], &sl.plan);
+        rc = plan_create(P, fine, &fb, 0, q->cmp[0], &sl.plan, depth > 1);
     }
     if (rc == SDF_OK && e != cudaSuccess) rc = cuda_fail(e, "creating the frame queue");
     if (rc) {

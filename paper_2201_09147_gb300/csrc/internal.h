@@ -122,7 +122,8 @@ struct GradArgs {
 // Kernel launchers (return cudaError_t of the launch).
 cudaError_t launch_trace_level_simt(const LevelArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_grad_simt(const GradArgs& a, int num_sms, cudaStream_t s);
-cudaError_t launch_trace_level_tc(const LevelArgs& a, int num_sms, cudaStream_t s);
+// overlapped: other frames run beside this one on another stream (the choice of a kernel, not its results).
+cudaError_t launch_trace_level_tc(const LevelArgs& a, int num_sms, cudaStream_t s, bool overlapped);
 cudaError_t launch_trace_wide(const LevelArgs& a, int num_sms, cudaStream_t s);  // trace_wide.cuh
 cudaError_t launch_grad_tc(const GradArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_grad32_tc(const GradArgs& a, int num_sms, cudaStream_t s);  // FP32 networks with s32

@@ -16,7 +16,8 @@
 //   TMEM, so the step t = f - d is never rounded to 16 bits.  Once the work
 //   list is empty the CTA regroups its remaining rays into its first tiles
 //   every few iterations.  Widths 128 (head + remainder) and 256, and small
-//   calls of width 64, run trace_wide_kernel (trace_wide.cuh).
+//   calls of width 64, run trace_wide_kernel (trace_wide.cuh); large calls of
+//   the (256,1) trace_single_tc_kernel.
 //
 // grad_tc : analytic gradients (Alg. 2).  Tiles of 64 points in two halves;
 //   the MMA runs with the features as rows (M = 128 per TMEM tile,
@@ -92,6 +93,11 @@ constexpr int kMaxTraceTiles = 6;
 // on 152 SMs, in us: (64,1) Lipschitz steps 82 / 156 / 227 against 196 / 211 /
 // 211, (64,1) coarse trace 99 / 120 / 139 against 119 / 122 / 124.
 constexpr int kWideRays = 256;
+// Queues keep several frames in flight on two streams, which share the SMs: there the kernels that keep fewer SMs
+// busy win earlier.  Four three-level host frames of 160^2 rays: 469 us with kWideRays, 421 with this line; of 140^2
+// (below both) 409, with the old kernels 417.
+constexpr int kWideRaysOverlapped = 128;
+static int wide_line(bool overlapped) { return overlapped ? kWideRaysOverlapped : kWideRays; }
 constexpr int kTraceMaxThreads = 128 * kMaxTraceTiles;
 
 // The trace kernel's tensor pipe is mostly idle (its time goes to the sines),
@@ -145,16 +151,18 @@ __device__ __forceinline__ void trace_layer0(const LevelArgs& a, const float4* w
 // Output layer of one ray row from N of its TMEM accumulator columns:
 // acc += w_out . sin(D + b), the bias additions and the products on unit
 // pairs (two packed accumulators, for units 4j, 4j+1 and 4j+2, 4j+3).
-template <int N>
+// E4M3: the accumulator holds mf times the value.
+template <int N, bool FP8 = false>
 __device__ __forceinline__ void output_dot(const float (&v)[N], const float* bl, const float* wo, float2& acc01,
-                                           float2& acc23) {
+                                           float2& acc23, float mf = 1.0f) {
+    const float2 mf2 = make_float2(mf, mf);
 #pragma unroll
     for (int j4 = 0; j4 < N / 4; ++j4) {
         const float4 b4 = reinterpret_cast<const float4*>(bl)[j4];
         const float4 w4 = reinterpret_cast<const float4*>(wo)[j4];
         const float2 v01 = make_float2(v[4 * j4 + 0], v[4 * j4 + 1]), v23 = make_float2(v[4 * j4 + 2], v[4 * j4 + 3]);
-        const float2 x01 = __fadd2_rn(v01, make_float2(b4.x, b4.y));
-        const float2 x23 = __fadd2_rn(v23, make_float2(b4.z, b4.w));
+        const float2 x01 = FP8 ? __ffma2_rn(v01, mf2, make_float2(b4.x, b4.y)) : __fadd2_rn(v01, make_float2(b4.x, b4.y));
+        const float2 x23 = FP8 ? __ffma2_rn(v23, mf2, make_float2(b4.z, b4.w)) : __fadd2_rn(v23, make_float2(b4.z, b4.w));
         acc01 = __ffma2_rn(make_float2(w4.x, w4.y), make_float2(sin_fast(x01.x), sin_fast(x01.y)), acc01);
         acc23 = __ffma2_rn(make_float2(w4.z, w4.w), make_float2(sin_fast(x23.x), sin_fast(x23.y)), acc23);
     }
@@ -437,6 +445,274 @@ __global__ void __launch_bounds__(kTraceMaxThreads, 1) trace_level_tc_kernel(con
     }
 }
 
+// Layer 0 of one ray row as E4M3 bytes of 256 sin(W_0 (p, t) + b_0): K-major
+// rows of 128-element blocks with the 128-byte swizzle, one 16-byte chunk
+// (16 units) per vector store; the units in pairs as in trace_layer0.
+template <int W, bool TIMED>
+__device__ __forceinline__ void trace_layer0_e4m3(const LevelArgs& a, const float* w0s, const float* wts,
+                                                  const Ray& ray, int row, uint32_t x_s) {
+    const float tm = (TIMED && ray.state == kSlotActive) ? __ldg(a.ray_time + ray.idx) : 0.0f;
+    const float2 px = make_float2(ray.px, ray.px), py = make_float2(ray.py, ray.py), pz = make_float2(ray.pz, ray.pz);
+    const float2 t2 = make_float2(tm, tm);
+    for (int j16 = 0; j16 < W / 16; ++j16) {
+        float sv[16];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int pr = j16 * 8 + q;
+            const float4 A = reinterpret_cast<const float4*>(w0s)[2 * pr];
+            const float4 B = reinterpret_cast<const float4*>(w0s)[2 * pr + 1];
+            float2 c = make_float2(B.z, B.w);
+            if (TIMED) c = __ffma2_rn(reinterpret_cast<const float2*>(wts)[pr], t2, c);
+            const float2 z = __ffma2_rn(make_float2(A.x, A.y), px,
+                                        __ffma2_rn(make_float2(A.z, A.w), py, __ffma2_rn(make_float2(B.x, B.y), pz, c)));
+            sv[2 * q] = kFp8ActScale * sin_fast(z.x);
+            sv[2 * q + 1] = kFp8ActScale * sin_fast(z.y);
+        }
+        st_shared_v4(x_s + sw128_chunk_offset(row, j16, 128), pack_e4m3x4(sv[0], sv[1], sv[2], sv[3]),
+                     pack_e4m3x4(sv[4], sv[5], sv[6], sv[7]), pack_e4m3x4(sv[8], sv[9], sv[10], sv[11]),
+                     pack_e4m3x4(sv[12], sv[13], sv[14], sv[15]));
+    }
+}
+
+// ---------------------------------------------------------------------------
+// trace kernel, one hidden layer of width 256
+// ---------------------------------------------------------------------------
+// One thread per ray as in trace_level_tc_kernel, the layer's weights (128 KB
+// beside 128 KB of activations, half of both in E4M3) streamed as in
+// trace_wide_kernel: a producer warp sends the K blocks of 128 bytes (256 rows = 32
+// KB) from L2 through a ring of two, cyclically for as long as rays remain, and
+// thread 0 issues the MMAs as they arrive.  Two tiles of 128 rays (TMEM columns
+// [t*256, (t+1)*256)) share every unit.
+//
+// For large calls, first of all as a later level of a multiscale trace: rays that
+// a coarser level has brought to its shell take about one step each, with a single
+// epilogue to share between more threads.  And for its registers: 288 threads of
+// 128 leave an SM 28 K registers for another stream's kernels, trace_wide_kernel's
+// 544 of 96 13 K (this kernel with 168: 17 K, and two overlapped host frames of 828
+// x 574 took 955 us instead of 897).  trace_wide_kernel -> this one, us: (64,1) >
+// (256,1) frames of 512^2 356 -> 344, 1900 x 1000 1,121 -> 1,083, overlapped host
+// frames, two of 828 x 574 967 -> 897, four of 200^2 469 -> 445 (one frame of 200^2
+// alone 163 -> 176: the line is where overlapped frames are even); the (256,1) traced
+// alone, 512 x 400 rays 573 -> 618, 720 x 600 997 -> 991, 1900 x 1000 2,543 -> 2,354,
+// in E4M3 300^2 336 -> 352, 400^2 464 -> 457, 1280 x 720 1,217 -> 1,075.
+constexpr int kSingleW = 256;
+// Rays per SM above which it runs: a level that continues another's rays (the lines of width 64, see kWideRays), and
+// a network traced alone, whose rays take many steps.
+constexpr int kSingleFirst = 2700, kSingleFirstFp8 = 1000;
+constexpr int kSingleRayThreads = 256;
+constexpr int kSingleThreads = kSingleRayThreads + 32;  // ray threads + producer warp
+constexpr int kSingleStages = 2;
+constexpr uint32_t kSingleUnit = kSingleW * 128u;
+
+struct SingleLayout {
+    uint32_t ring, w0, wt, bh, wout, bars, misc, total;
+};
+
+template <int OP>
+__host__ __device__ inline SingleLayout single_layout() {
+    SingleLayout L;
+    uint32_t o = 2u * 128u * kSingleW * (OP == kOpE4M3 ? 1u : 2u);
+    L.ring = o;
+    o += kSingleStages * kSingleUnit;
+    L.w0 = o;
+    o += kSingleW * 16u;
+    L.wt = o;
+    o += kSingleW * 4u;
+    L.bh = o;
+    o += kSingleW * 4u;
+    L.wout = o;
+    o += kSingleW * 4u;
+    L.bars = o;
+    o += (2 * kSingleStages + 1) * 8u;
+    o = (o + 15u) & ~15u;
+    L.misc = o;
+    o += 32u;
+    L.total = o;
+    return L;
+}
+
+template <int OP>
+__global__ void __maxnreg__(128) trace_single_tc_kernel(const LevelArgs a) {
+    constexpr bool F16 = OP == kOpF16, FP8 = OP == kOpE4M3;
+    constexpr int EB = FP8 ? 1 : 2;  // operand bytes per element
+    constexpr int W = kSingleW, KB = W * EB / 128, NS = kSingleStages, NRAY = kSingleRayThreads;
+    constexpr uint32_t kSingleX = 128u * W * EB;  // a tile's activations
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t raw_s = smem_u32(smem_raw);
+    const uint32_t base_s = (raw_s + 1023u) & ~1023u;
+    uint8_t* base = smem_raw + (base_s - raw_s);
+    const NetView& net = a.net;
+    const SingleLayout L = single_layout<OP>();
+    float* w0s = reinterpret_cast<float*>(base + L.w0);
+    float* wts = reinterpret_cast<float*>(base + L.wt);
+    float* bhs = reinterpret_cast<float*>(base + L.bh);
+    float* wos = reinterpret_cast<float*>(base + L.wout);
+    const uint32_t bar_full = base_s + L.bars, bar_empty = bar_full + 8u * NS, bar_mma = bar_empty + 8u * NS;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + L.misc);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(base + L.misc + 4);
+    volatile int* done_flag = reinterpret_cast<volatile int*>(base + L.misc + 8);
+    volatile uint32_t* consumed = reinterpret_cast<volatile uint32_t*>(base + L.misc + 12);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tile = tid >> 7, ttid = tid & 127;
+    const uint32_t x_s = base_s + static_cast<uint32_t>(tile < 2 ? tile : 0) * kSingleX;
+    const uint32_t ring_s = base_s + L.ring;
+
+    if (tid == 0) {
+        for (int s = 0; s < NS; ++s) {
+            mbar_init(bar_full + 8u * s, 1);
+            mbar_init(bar_empty + 8u * s, 1);
+        }
+        mbar_init(bar_mma, 1);
+        *abort_flag = 0;
+        *done_flag = 0;
+        *consumed = 0;
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        tmem_alloc(smem_u32(tmem_slot), 2 * W);
+        tmem_relinquish();
+    }
+    const bool timed = a.ray_time != nullptr && net.in_dim == 4;
+    for (int i = tid; i < W; i += kSingleThreads) {
+        stage_layer0_pairs(net, a.time, timed, i, w0s, wts);
+        wos[i] = net.wout[i];
+        bhs[i] = net.bh[0][i];
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem0 = *tmem_slot;
+
+    if (warp == NRAY / 32) {
+        if (lane == 0) {
+            uint32_t g = 0;
+            while (true) {
+                const uint32_t stage = g % NS, use = g / NS;
+                if (use > 0) {
+                    const uint32_t bar = bar_empty + 8u * stage, par = (use - 1) & 1u;
+                    const uint64_t t0 = globaltimer_ns();
+                    bool got = false;
+                    while (!(got = mbar_try_wait(bar, par))) {
+                        if (*done_flag || *abort_flag) break;
+                        if (globaltimer_ns() - t0 > kWaitBudgetNs) {
+                            raise_status(a.status, kStatusTimeout);
+                            *abort_flag = 1;
+                            break;
+                        }
+                    }
+                    if (!got) break;
+                }
+                mbar_arrive_expect_tx(bar_full + 8u * stage, kSingleUnit);
+                bulk_g2s(ring_s + stage * kSingleUnit,
+                         net.wbf + static_cast<size_t>(g % KB) * net.rows_pad * 128u, kSingleUnit, bar_full + 8u * stage);
+                ++g;
+            }
+            // every copy issued must land before the block exits
+            for (uint32_t gg = *consumed; gg < g; ++gg) mbar_drain(bar_full + 8u * (gg % NS), (gg / NS) & 1u);
+        }
+    } else {
+        const long long n_work = a.in_list ? static_cast<long long>(*a.in_count) : a.n;
+        const uint32_t tmem = tmem0 + static_cast<uint32_t>(tile * W) + (static_cast<uint32_t>((ttid >> 5) * 32) << 16);
+        // E4M3: the format fields 0 of this descriptor select E4M3 under kind::f8f6f4
+        constexpr uint32_t idesc = idesc_f32acc(128, W, F16 || FP8);
+        // E4M3: accumulator -> value (the operand scales q_w and 256 divided out)
+        const float mf = FP8 ? 1.0f / (net.q_w[0] * kFp8ActScale) : 1.0f;
+        const uint64_t rd0 = desc_kmajor_sw128(ring_s);
+        uint32_t mma_phase = 0, g = 0;
+        bool issue_ok = true;  // thread 0: every weight unit so far arrived in time
+        Ray ray;
+        // Stop decisions go through the ray threads' barrier: a timed-out wait drops the ray (the status word
+        // reports it) instead of leaving the loop.
+        while (true) {
+            refill_ray(a, ray, n_work);
+            if (a.cap <= 0) {
+                if (!bar_or(1, NRAY, ray.state == kSlotActive)) break;
+                pass_ray(a, ray);
+                continue;
+            }
+            // a warp with no active slot skips its rows (as in trace_level_tc_kernel)
+            const bool wact = __any_sync(0xffffffffu, ray.state == kSlotActive);
+            if (wact) {
+                if (FP8) {
+                    if (timed)
+                        trace_layer0_e4m3<W, true>(a, w0s, wts, ray, ttid, x_s);
+                    else
+                        trace_layer0_e4m3<W, false>(a, w0s, wts, ray, ttid, x_s);
+                } else if (timed)
+                    trace_layer0<W, F16, false, true>(a, reinterpret_cast<const float4*>(w0s), wts, ray, ttid, x_s, x_s);
+                else
+                    trace_layer0<W, F16, false, false>(a, reinterpret_cast<const float4*>(w0s), wts, ray, ttid, x_s, x_s);
+            }
+            fence_proxy_async_smem();
+            tc_fence_before();
+            if (!bar_or(1, NRAY, ray.state == kSlotActive)) break;
+
+            if (tid == 0) {
+                tc_fence_after();
+                for (int kb = 0; kb < KB && issue_ok; ++kb, ++g) {
+                    const uint32_t stage = g % NS;
+                    issue_ok = mbar_wait_bounded(bar_full + 8u * stage, (g / NS) & 1u, a.status, abort_flag);
+                    if (!issue_ok) break;
+                    tc_fence_after();
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const uint64_t xd0 = desc_kmajor_sw128(base_s + t * kSingleX);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            const uint64_t xd = desc_add(xd0, kb * 128u * 128u + kk * 32u);
+                            const uint64_t wd = desc_add(rd0, stage * kSingleUnit + kk * 32u);
+                            if (FP8)
+                                mma_f8kind(tmem0 + t * W, xd, wd, idesc, (kb | kk) != 0);
+                            else
+                                mma_f16kind(tmem0 + t * W, xd, wd, idesc, (kb | kk) != 0);
+                        }
+                    }
+                    mma_commit(bar_empty + 8u * stage);
+                }
+                if (issue_ok) mma_commit(bar_mma);
+            }
+            // a warp either reads the accumulator whole or not at all
+            const bool good = __all_sync(0xffffffffu, mbar_wait_bounded(bar_mma, mma_phase, a.status, abort_flag));
+            mma_phase ^= 1u;
+            tc_fence_after();
+            float2 acc01 = make_float2(0.0f, 0.0f), acc23 = make_float2(0.0f, 0.0f);
+            if (good && wact) {
+                // 32-column chunks, the next one loading from TMEM while the current one is processed
+                float va[32], vb[32];
+                tmem_ld32(tmem, va);
+                tmem_wait_ld();
+#pragma unroll
+                for (int q = 0; q < W / 32; ++q) {
+                    float(&v)[32] = (q & 1) ? vb : va;
+                    float(&vn)[32] = (q & 1) ? va : vb;
+                    if (q + 1 < W / 32) tmem_ld32(tmem + (q + 1) * 32u, vn);
+                    output_dot<32, FP8>(v, bhs + q * 32, wos + q * 32, acc01, acc23, mf);
+                    tmem_wait_ld();
+                }
+            }
+            const float f = ((acc01.x + acc01.y) + (acc23.x + acc23.y)) + net.bout;
+            tc_fence_before();
+            if (good)
+                step_ray(a, ray, f);
+            else
+                ray.state = kSlotDone;
+        }
+        if (tid == 0) *consumed = g;
+        bar_named(1, NRAY);
+        if (tid == 0) {
+            __threadfence_block();
+            *done_flag = 1;
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc(tmem0, 2 * W);
+    }
+}
+
 }  // namespace
 
 bool tc_trace_supported(int width, int n_hidden) {
@@ -502,16 +778,29 @@ int trace_tiles_max(const NetView& net) {
     return 1;  // trace_wide_kernel: one launch shape
 }
 
-cudaError_t launch_trace_level_tc(const LevelArgs& a, int num_sms, cudaStream_t s) {
+template <int OP>
+static cudaError_t launch_single(const LevelArgs& a, int num_sms, cudaStream_t s) {
+    return launch_tc(trace_single_tc_kernel<OP>, kSingleThreads, single_layout<OP>().total + 1024, 2 * kSingleW, num_sms,
+                     s, &a);
+}
+
+cudaError_t launch_trace_level_tc(const LevelArgs& a, int num_sms, cudaStream_t s, bool overlapped) {
     const bool f16 = a.net.op_f16 != 0;
     if (a.net.width == 64) {
-        if (a.n <= static_cast<int64_t>(num_sms) * kWideRays) return launch_trace_wide(a, num_sms, s);
+        if (a.n <= static_cast<int64_t>(num_sms) * wide_line(overlapped)) return launch_trace_wide(a, num_sms, s);
         return f16 ? launch_trace_resident<64, true, true>(a, num_sms, s)
                    : launch_trace_resident<64, false, true>(a, num_sms, s);
     }
     if (a.net.width == 128 && !split_of(a.net))
         return f16 ? launch_trace_resident<128, true, false>(a, num_sms, s)
                    : launch_trace_resident<128, false, false>(a, num_sms, s);
+    if (a.net.width == kSingleW && a.net.n_hidden == 1) {
+        const int line = a.in_list != nullptr ? wide_line(overlapped) : a.net.op_fp8 ? kSingleFirstFp8 : kSingleFirst;
+        if (a.n > static_cast<int64_t>(num_sms) * line) {
+            if (a.net.op_fp8) return launch_single<kOpE4M3>(a, num_sms, s);
+            return f16 ? launch_single<kOpF16>(a, num_sms, s) : launch_single<kOpBF16>(a, num_sms, s);
+        }
+    }
     return launch_trace_wide(a, num_sms, s);
 }
 

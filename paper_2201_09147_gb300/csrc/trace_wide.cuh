@@ -19,7 +19,8 @@ namespace {
 //   width 128, head + remainder operands (resident, one tile, CS = 4): the
 //     weights leave room for one tile of activations per SM, which had 128
 //     threads.
-//   width 256 (weights streamed through a ring): two tiles that share every
+//   width 256 (weights streamed through a ring; large calls of a single layer
+//     run trace_single_tc_kernel): two tiles that share every
 //     weight unit, CS = 2; for calls of at most 128 rays per SM one tile, CS = 4
 //     and a third ring stage (a lone tile's MMAs consume a unit faster than two
 //     outstanding copies bring them).

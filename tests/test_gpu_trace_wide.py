@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2201_09147_gb300 import inputs
+from paper_2201_09147_gb300 import inputs, workloads
 
 pytestmark = pytest.mark.gpu
 
@@ -67,3 +67,52 @@ def test_calls_of_few_rays_match_a_larger_call(sdf, width, hidden, in_dim, preci
     for x, y in zip(few, all_):
         assert torch.equal(x, y[..., :n])
     sdf.sync_status()
+
+
+@pytest.mark.parametrize("in_dim,precision,line", [(3, "SDF_BF16", 2700), (4, "SDF_FP16", 256), (4, "SDF_FP8", 1000)])
+def test_one_hidden_layer_of_256_in_large_calls(sdf, in_dim, precision, line):
+    """Later levels of calls of more than 256 rays per SM, and first levels of more than 2,700 (E4M3: 1,000), run on a
+    kernel of their own: the same bits as in calls of fewer, with and without levels that do no step."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = line * sms + 33
+    b = inputs.net_to_bytes(inputs.siren_init(5, 256, 1, in_dim=in_dim, out_scale=30.0, out_shift=0.1))
+    net = sdf.Net(b, getattr(sdf, precision))
+    orig, d, time = rays(n, in_dim)
+
+    def trace(lo, hi, caps):
+        k = len(caps)
+        return sdf.trace_multiscale([net] * k, [0.01] * (k - 1) + [0.0], caps, 1e-2, orig[:, lo:hi].contiguous(),
+                                    d[:, lo:hi].contiguous(), step_scale=[0.3] * k,
+                                    ray_time=None if time is None else time[lo:hi].contiguous())
+
+    for caps in ([25], [3, 25], [0, 25], [25, 0], [2, 3, 4]):
+        whole = trace(0, n, caps)
+        for lo, hi in ((0, line * sms), (line * sms, n)):
+            assert all(torch.equal(x[..., lo:hi], y) for x, y in zip(whole, trace(lo, hi, caps)))
+    assert 0 < int(trace(0, n, [25])[2].sum()) < n
+    sdf.sync_status()
+
+
+@pytest.mark.parametrize("width,height", [(150, 129), (180, 170), (200, 195)])
+def test_queued_frames_match_direct_calls(sdf, width, height):
+    """Frames overlapped on two streams take other kernels from 128 rays per SM on: the same bits as direct calls."""
+    wl = workloads.get("three_level_512", width, height)
+    nets = [sdf.Net((workloads.SCENES / x).read_bytes(), sdf.SDF_BF16) for x in wl.levels]
+    fine = sdf.Net((workloads.SCENES / wl.fine).read_bytes(), sdf.SDF_BF16)
+    n = width * height
+    orig, d, _ = rays(n, 3)
+    host = [x.cpu().pin_memory() for x in (orig, d)]
+    out = [(torch.empty(3, n).pin_memory(), torch.empty(n, dtype=torch.uint8).pin_memory(), torch.empty(3, n).pin_memory())
+           for _ in range(4)]
+    queue = sdf.FrameQueue(nets, wl.delta, wl.caps, wl.eps, fine, n, depth=3, step_scale=wl.step_scale,
+                           final_mode=wl.final_mode)
+    for o in out:
+        queue.submit(*host, *o)
+    queue.wait()
+    pos, _, hit, _ = sdf.trace_multiscale(nets, wl.delta, wl.caps, wl.eps, orig, d, step_scale=wl.step_scale,
+                                          final_mode=wl.final_mode)
+    normal = sdf.normal_map(fine, pos, hit)
+    sdf.sync_status()
+    assert hit.any()
+    for o in out:
+        assert all(torch.equal(a, b.cpu()) for a, b in zip(o, (pos, hit, normal)))
