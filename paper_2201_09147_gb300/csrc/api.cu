@@ -1012,7 +1012,7 @@ int plan_autotune(sdf_plan* p, int* status, int num_sms, cudaStream_t s) {
     const sdf_frame_batch& b = p->batch;
     for (int j = 0; j < p->n_levels && rc == SDF_OK; ++j) {
         const sdf_net* net = p->nets[j];
-        const int tmax = net->precision == SDF_FP32 ? 0 : trace_tiles_max(view_of(net));
+        const int tmax = net->precision == SDF_FP32 ? 0 : trace_tiles_max(view_of(net), b.n, num_sms, p->overlapped);
         if (tmax <= 1) {
             p->tiles[j] = tmax;  // one launch shape (0: FP32)
             continue;

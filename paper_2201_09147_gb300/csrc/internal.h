@@ -127,7 +127,8 @@ cudaError_t launch_trace_level_tc(const LevelArgs& a, int num_sms, cudaStream_t 
 cudaError_t launch_trace_wide(const LevelArgs& a, int num_sms, cudaStream_t s);  // trace_wide.cuh
 cudaError_t launch_grad_tc(const GradArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_grad32_tc(const GradArgs& a, int num_sms, cudaStream_t s);  // FP32 networks with s32
-int trace_tiles_max(const NetView& net);  // largest `tiles` the tensor-core trace kernel accepts for net
+// Largest `tiles` that changes the launch of a level of n rays (1: the kernel that it takes has one launch shape).
+int trace_tiles_max(const NetView& net, int64_t n, int num_sms, bool overlapped);
 bool tc_trace_supported(int width, int n_hidden);
 // Measured throughput of the tensor-core kernels' sine on all SMs (sines per second).
 cudaError_t measure_sine_rate(int num_sms, cudaStream_t s, double* sines_per_s);

@@ -766,10 +766,10 @@ static cudaError_t launch_trace_resident(const LevelArgs& a, int num_sms, cudaSt
 // Networks of width 64 always fit with head and remainder operands; width 128 does up to k = 2.
 static bool split_of(const NetView& net) { return net.wbf_lo != nullptr && trace_split(net.width, net.n_hidden); }
 
-int trace_tiles_max(const NetView& net) {
+int trace_tiles_max(const NetView& net, int64_t n, int num_sms, bool overlapped) {
     if (!tc_trace_supported(net.width, net.n_hidden)) return 0;
     const int KH = net.n_hidden;
-    if (net.width == 64)
+    if (net.width == 64 && n > static_cast<int64_t>(num_sms) * wide_line(overlapped))
         return net.op_f16 ? trace_tiles(trace_level_tc_kernel<64, true, true>, 64, KH, true)
                           : trace_tiles(trace_level_tc_kernel<64, false, true>, 64, KH, true);
     if (net.width == 128 && !split_of(net))

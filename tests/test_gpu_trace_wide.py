@@ -116,3 +116,20 @@ def test_queued_frames_match_direct_calls(sdf, width, height):
     assert hit.any()
     for o in out:
         assert all(torch.equal(a, b.cpu()) for a, b in zip(o, (pos, hit, normal)))
+
+
+@pytest.mark.parametrize("per_sm,most", [(3, 1), (256, 1), (257, 6)])
+def test_autotuned_plans_report_what_they_run(sdf, per_sm, most):
+    """The tile count of a plan is a count that its launches use: one for the calls of few rays, whose kernel has
+    one launch shape."""
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    net = sdf.Net(inputs.net_to_bytes(inputs.siren_init(5, 64, 1, out_scale=30.0, out_shift=0.1)), sdf.SDF_BF16)
+    orig, d, _ = rays(n, 3)
+    plan = sdf.Plan([net], [0.0], [9], 1e-2, orig, d, step_scale=[0.3], autotune=True)
+    tiles, _ = plan.info()
+    assert 1 <= tiles[0] <= most
+    plan.launch()
+    direct = sdf.trace_multiscale([net], [0.0], [9], 1e-2, orig, d, step_scale=[0.3])
+    assert torch.equal(plan.pos, direct[0]) and torch.equal(plan.hit, direct[2])
+    plan.close()
+    sdf.sync_status()
