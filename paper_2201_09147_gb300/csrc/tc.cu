@@ -15,9 +15,9 @@
 //   output layer is an FP32 dot product of the last sine layer straight from
 //   TMEM, so the step t = f - d is never rounded to 16 bits.  Once the work
 //   list is empty the CTA regroups its remaining rays into its first tiles
-//   every few iterations.  Widths 128 (head + remainder) and 256, and small
-//   calls of width 64, run trace_wide_kernel (trace_wide.cuh); large calls of
-//   the (256,1) trace_single_tc_kernel.
+//   every few iterations.  Width 128 with two hidden layers (head + remainder)
+//   and 256, and small calls of width 64 and the (128,1), run trace_wide_kernel
+//   (trace_wide.cuh); large calls of the (256,1) trace_single_tc_kernel.
 //
 // grad_tc : analytic gradients (Alg. 2).  Tiles of 64 points in two halves;
 //   the MMA runs with the features as rows (M = 128 per TMEM tile,
@@ -97,6 +97,9 @@ constexpr int kWideRays = 256;
 // busy win earlier.  Four three-level host frames of 160^2 rays: 469 us with kWideRays, 421 with this line; of 140^2
 // (below both) 409, with the old kernels 417.
 constexpr int kWideRaysOverlapped = 128;
+// One hidden layer of width 128 leaves shared memory for several tiles: trace_wide_kernel's one is slower in large
+// calls (700 x 500 rays 457 us against 331, 33,000 rays 178 against 173, 60^2 rays 141 against 168).
+constexpr int kWideRays128x1 = 192;
 static int wide_line(bool overlapped) { return overlapped ? kWideRaysOverlapped : kWideRays; }
 constexpr int kTraceMaxThreads = 128 * kMaxTraceTiles;
 
@@ -775,6 +778,9 @@ int trace_tiles_max(const NetView& net, int64_t n, int num_sms, bool overlapped)
     if (net.width == 128 && !split_of(net))
         return net.op_f16 ? trace_tiles(trace_level_tc_kernel<128, true, false>, 128, KH, false)
                           : trace_tiles(trace_level_tc_kernel<128, false, false>, 128, KH, false);
+    if (net.width == 128 && KH == 1 && n > static_cast<int64_t>(num_sms) * kWideRays128x1)
+        return net.op_f16 ? trace_tiles(trace_level_tc_kernel<128, true, true>, 128, KH, true)
+                          : trace_tiles(trace_level_tc_kernel<128, false, true>, 128, KH, true);
     return 1;  // trace_wide_kernel: one launch shape
 }
 
@@ -794,6 +800,9 @@ cudaError_t launch_trace_level_tc(const LevelArgs& a, int num_sms, cudaStream_t 
     if (a.net.width == 128 && !split_of(a.net))
         return f16 ? launch_trace_resident<128, true, false>(a, num_sms, s)
                    : launch_trace_resident<128, false, false>(a, num_sms, s);
+    if (a.net.width == 128 && a.net.n_hidden == 1 && a.n > static_cast<int64_t>(num_sms) * kWideRays128x1)
+        return f16 ? launch_trace_resident<128, true, true>(a, num_sms, s)
+                   : launch_trace_resident<128, false, true>(a, num_sms, s);
     if (a.net.width == kSingleW && a.net.n_hidden == 1) {
         const int line = a.in_list != nullptr ? wide_line(overlapped) : a.net.op_fp8 ? kSingleFirstFp8 : kSingleFirst;
         if (a.n > static_cast<int64_t>(num_sms) * line) {

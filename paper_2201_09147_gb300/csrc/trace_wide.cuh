@@ -17,13 +17,13 @@ namespace {
 //
 //   width 64 (weights resident, one tile, CS = 4): calls of few rays.
 //   width 128, head + remainder operands (resident, one tile, CS = 4): the
-//     weights leave room for one tile of activations per SM, which had 128
-//     threads.
+//     weights of two layers leave room for one tile of activations per SM, which
+//     had 128 threads; with one layer, small calls only.
 //   width 256 (weights streamed through a ring; large calls of a single layer
-//     run trace_single_tc_kernel): two tiles that share every
-//     weight unit, CS = 2; for calls of at most 128 rays per SM one tile, CS = 4
-//     and a third ring stage (a lone tile's MMAs consume a unit faster than two
-//     outstanding copies bring them).
+//     run trace_single_tc_kernel): two tiles that share every weight unit, CS =
+//     2; for calls of at most 128 rays per SM one tile, CS = 4 and a third ring
+//     stage (a lone tile's MMAs consume a unit faster than two outstanding copies
+//     bring them).
 //
 // What it measured (one call, us, before -> after): a 128 x 128 frame of the
 // Lipschitz-stepped (64,1) 183 -> 80; the plain (256,3) trace of 139^2 rays 610
