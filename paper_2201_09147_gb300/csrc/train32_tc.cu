@@ -560,11 +560,9 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
         float acc[FC];
 #pragma unroll
         for (int j = 0; j < FC; ++j) acc[j] = 0.0f;
-        // the flush of the blocks multiplied so far (`steps` K steps of points); `job` >= 0 also adds the registers
-        // to dL/dtheta
+        // the flush of the blocks multiplied so far; `job` >= 0 also adds the registers to dL/dtheta
         uint32_t flushes = 0;
-        auto flush = [&](int64_t job, int steps) {
-            const float gain = flush_gain(steps);
+        auto flush = [&](int job, float gain) {
             ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_done, flushes & 1u, a.status, abort_flag)) && ok;
             ++flushes;
             if (!ok) return;
@@ -581,7 +579,7 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
             tc_fence_before();
             mbar_arrive(bar_flushed);
             if (job >= 0) {
-                const int l = static_cast<int>(job / (C::JB * C::JB)), b = static_cast<int>(job % (C::JB * C::JB));
+                const int l = job / (C::JB * C::JB), b = job % (C::JB * C::JB);
                 const int unit = (b / C::JB) * C::NB + quad * 32 + lane;
                 if (quad * 32 < C::NB) {
                     float4* out = reinterpret_cast<float4*>(a.d_theta + sh.off_w[l] + static_cast<size_t>(unit) * W +
@@ -595,11 +593,13 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
             }
         };
         uint32_t g = 0;
-        int in_acc = 0, steps = 0, pending_steps = 0;
-        int64_t pending = -2;  // the flush to run after the next build: -2 none, -1 to registers, >= 0 to that job
+        int in_acc = 0;
+        float gain = 1.0f;     // of the pending flush
+        int pending = -2;      // the flush to run after the next build: -2 none, -1 to registers, >= 0 to that job
         for (int64_t t = lo; t < hi && ok; ++t, ++g) {
-            const int64_t job = t / nkb, pbase = (t % nkb) * 16 + p_off;
-            const int l = static_cast<int>(job / (C::JB * C::JB)), b = static_cast<int>(job % (C::JB * C::JB));
+            const int job = static_cast<int>(t / nkb);
+            const int64_t pbase = (t % nkb) * 16 + p_off;
+            const int l = job / (C::JB * C::JB), b = job % (C::JB * C::JB);
             const int feat = (is_x ? b % C::JB : b / C::JB) * C::NB + row;
             // this thread's points of the K block: D_l, or the layer below's (A, H) (A_0 and W_0 for layer 0)
             float4 q[C::PPT];
@@ -638,18 +638,18 @@ __global__ void __launch_bounds__(Wg32<W>::THREADS, 1) train32_wgrad_kernel(cons
             fence_proxy_async_smem();
             mbar_arrive(bar_full + 8u * stage);
             if (pending != -2) {
-                flush(pending, pending_steps);
+                flush(pending, gain);
                 pending = -2;
             }
             const bool job_end = t + 1 == hi || (t + 1) % nkb == 0;
-            steps += static_cast<int>(min(a.n - (t % nkb) * 16 + 3, static_cast<int64_t>(16)) / 4);
             if (++in_acc == kFlush || job_end) {
                 pending = job_end ? job : -1;
-                pending_steps = steps;
-                in_acc = steps = 0;
+                // four K steps a block; the batch's last block has one per four points
+                gain = flush_gain(4 * in_acc - (pbase - p_off + 16 > a.n ? static_cast<int>(pbase - p_off + 16 - a.n) / 4 : 0));
+                in_acc = 0;
             }
         }
-        if (ok && pending != -2) flush(pending, pending_steps);
+        if (ok && pending != -2) flush(pending, gain);
     }
 
     tc_fence_before();
