@@ -92,12 +92,12 @@ __host__ __device__ inline G32Layout g32_layout() {
 // A remainder is held times 2^11: as large as its head, it is no smaller a half than the head is.
 constexpr float kRemScale = 2048.0f;
 
-// Two half planes of a pair of floats: the rounding of x and of 2^11 times what is left (exact, an FMA).
+// Two half planes of a pair of floats: the rounding of x and of 2^11 times what is left (exact).
 __device__ __forceinline__ void split2x2(float a, float b, uint32_t (&p)[2]) {
     p[0] = pack16x2<true>(a, b);
     const float2 h = make_float2(from16<true>(static_cast<uint16_t>(p[0] & 0xFFFFu)),
                                  from16<true>(static_cast<uint16_t>(p[0] >> 16)));
-    const float2 r = __ffma2_rn(h, make_float2(-kRemScale, -kRemScale), make_float2(a * kRemScale, b * kRemScale));
+    const float2 r = __fmul2_rn(__ffma2_rn(h, make_float2(-1.0f, -1.0f), make_float2(a, b)), make_float2(kRemScale, kRemScale));
     p[1] = pack16x2<true>(r.x, r.y);
 }
 
@@ -422,16 +422,25 @@ __global__ void __launch_bounds__(G32<W, TRAIN ? 3 : 2>::THREADS, 1) grad32_tc_k
                     for (int e = 0; e < 4; ++e) {
                         const int j = 4 * e;
 #pragma unroll
-                        for (int s = 0; s < 4; ++s) v[j + s] = fmaf(c[j + s], lo, v[j + s]);
+                        for (int s = 0; s < 4; s += 2) {
+                            const float2 r = __ffma2_rn(make_float2(c[j + s], c[j + s + 1]), make_float2(lo, lo),
+                                                        make_float2(v[j + s], v[j + s + 1]));
+                            v[j + s] = r.x;
+                            v[j + s + 1] = r.y;
+                        }
                         const float A = fmaf(v[j], sc.x, bb);
                         if (TRAIN && 4 * q + e < nv)
                             save[(4 * q + e) * W] = make_float4(A, v[j + 1] * sc.y, v[j + 2] * sc.y, v[j + 3] * sc.y);
                         float sn, cn;
                         sincos_r(A, &sn, &cn);
                         cn *= mg;
-                        v[j] = TRAIN ? (last ? wo * sn : sn) : sn * sc.z;
-#pragma unroll
-                        for (int s = 1; s < 4; ++s) v[j + s] *= cn;
+                        const float ps = TRAIN ? (last ? wo : 1.0f) : sc.z;
+                        const float2 r01 = __fmul2_rn(make_float2(sn, v[j + 1]), make_float2(ps, cn));
+                        const float2 r23 = __fmul2_rn(make_float2(v[j + 2], v[j + 3]), make_float2(cn, cn));
+                        v[j] = r01.x;
+                        v[j + 1] = r01.y;
+                        v[j + 2] = r23.x;
+                        v[j + 3] = r23.y;
                     }
                     if (last) {
                         warp_sum16(v, lane);
