@@ -371,7 +371,7 @@ bool split_image32(const std::vector<std::vector<double>>& Wl, int IN, int W, in
     const size_t plane = static_cast<size_t>(rows_pad) * 128u, layer = 2 * plane * (W / 64);
     img->assign(KH * layer, 0);
     std::vector<int> w(W);
-    std::vector<double> sq(W), gain_p(W), gain_g(W);
+    std::vector<double> sq(W), gain_p(W), gain_g(W), col(W);  // col: 2^e (exact products: every factor is a power of two)
     // the correction of a row's sums (grad32_tc.cuh), from the squares of its terms' magnitudes
     auto gain = [&]() {
         double sum = 0.0, shares = 0.0;
@@ -385,12 +385,14 @@ bool split_image32(const std::vector<std::vector<double>>& Wl, int IN, int W, in
     };
     for (int l = 1; l <= KH; ++l) {
         uint8_t* dst = img->data() + static_cast<size_t>(l - 1) * layer;
+        for (int k = 0; k < W; ++k) col[k] = std::ldexp(1.0, e[k]);
         for (int r = 0; r < W; ++r) {
+            const double* row = &Wl[l][static_cast<size_t>(r) * W];
             double amax = 0.0;
             bn[r] = 0.0;
             for (int k = 0; k < W; ++k) {
-                const double x = std::fabs(static_cast<double>(static_cast<float>(Wl[l][static_cast<size_t>(r) * W + k])));
-                amax = std::max(amax, std::ldexp(x, e[k]));
+                const double x = std::fabs(static_cast<double>(static_cast<float>(row[k])));
+                amax = std::max(amax, x * col[k]);
                 bn[r] += x * b[k];
             }
             ok = ok && std::isfinite(amax);
@@ -398,15 +400,13 @@ bool split_image32(const std::vector<std::vector<double>>& Wl, int IN, int W, in
             ok = ok && std::abs(w[r]) <= 60;
             if (!ok) return false;
             // (squares of the scaled weights: no overflow, and what underflows does not matter)
-            for (int k = 0; k < W; ++k)
-                sq[k] = std::pow(std::ldexp(Wl[l][static_cast<size_t>(r) * W + k], emin + w[r]), 2);
+            const double scale = std::ldexp(1.0, w[r]), low = std::ldexp(1.0, emin + w[r]);
+            for (int k = 0; k < W; ++k) sq[k] = (row[k] * low) * (row[k] * low);
             gain_p[r] = gain();
-            for (int k = 0; k < W; ++k)
-                sq[k] = std::pow(std::ldexp(Wl[l][static_cast<size_t>(r) * W + k] * b[k], w[r]), 2);
+            for (int k = 0; k < W; ++k) sq[k] = (row[k] * b[k] * scale) * (row[k] * b[k] * scale);
             gain_g[r] = gain();
             for (int k = 0; k < W; ++k) {
-                const float x = static_cast<float>(
-                    std::ldexp(static_cast<double>(static_cast<float>(Wl[l][static_cast<size_t>(r) * W + k])), e[k] + w[r]));
+                const float x = static_cast<float>(static_cast<double>(static_cast<float>(row[k])) * col[k] * scale);
                 const __half hi = __float2half_rn(x), lo = __float2half_rn((x - __half2float(hi)) * 2048.0f);
                 const uint16_t hb = __half_as_ushort(hi), lb = __half_as_ushort(lo);
                 uint8_t* at = dst + static_cast<size_t>(k / 64) * 2 * plane + sw128_offset(r, k & 63, rows_pad);
