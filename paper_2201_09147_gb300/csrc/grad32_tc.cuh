@@ -216,23 +216,25 @@ __device__ __forceinline__ bool mma_layer32(uint32_t tmem, int h, uint64_t xd0, 
 // streams, a producer warp streaming the weights, an MMA warp, epilogue groups
 // that own a feature per thread), with these differences: operands in
 // planes and two accumulators; at width 256 the planes of one half fill
-// the activation memory, so the CTA runs one half of 32 points (its MMAs, 6.1 k
-// clocks a layer, and epilogue, ~2 k, take turns; two halves of 16 points
-// would stream the weights twice and read them at N = 64, where shared-memory
-// bandwidth and not the tensor pipe bounds the MMAs); two threads share a
+// the activation memory, so the CTA runs one half of 32 points (its MMAs, 96 of
+// about 77 clocks a layer, and epilogue, about as long, take turns; an MMA of N =
+// 64 costs its issuer the same 77, so two halves of 16 points lose: the training
+// forward of the (128,2) 93 -> 113 us); two threads share a
 // feature, so 16 epilogue warps hide the sines' latency; the output layer
 // runs in FP32 on the CUDA cores (w_out times the last tangents, summed over
 // the features by a warp butterfly and, in a fixed order, over the warps).
 // The FP32 FMA units did the same products before (grad_simt_kernel, now for
 // networks beyond the scales only): a call of 20,011 points of a (256,3) 0.73
-// -> 0.14 ms, of a (128,2) 0.168 -> 0.043, of a (64,2) 0.074 -> 0.042 (the
-// last two bound by the host), the error against FP64 5 to 15 % lower on each
-// of six networks.  What bounds the (256,3) now is the alternation of MMAs
-// (6.1 k clocks a layer) and epilogue.
+// -> 0.124 ms, of a (128,2) 0.168 -> 0.040, of a (64,2) 0.074 -> 0.049 (the
+// last two bound by the host), the error against FP64 4 to 14 % lower on each
+// of six networks.  What bounds the (256,3) now is the alternation of MMAs and
+// epilogue (14.7 k clocks a layer and tile).
 //
 // TRAIN: the training forward.  It saves A_0 ([n][W]) and (A_l, H_l^x, H_l^y,
 // H_l^z) ([k][n][W] float4: a warp's store is 512 consecutive bytes) and also
-// writes f (no list, no normalisation).
+// writes f (no list, no normalisation).  Bound by its MMAs, six per K step: 93 us
+// for 50,001 points of the (128,2), where halves under a scale per layer, which
+// some networks exceed, took 68.
 template <int W, bool TRAIN = false>
 __global__ void __launch_bounds__(G32<W, TRAIN ? 3 : 2>::THREADS, 1) grad32_tc_kernel(const GradArgs a) {
     using C = G32<W, TRAIN ? 3 : 2>;
