@@ -25,11 +25,10 @@ namespace {
 //     stage (a lone tile's MMAs consume a unit faster than two outstanding copies
 //     bring them).
 //
-// What it measured (one call, us, before -> after): a 128 x 128 frame of the
-// Lipschitz-stepped (64,1) 183 -> 80; the plain (256,3) trace of 139^2 rays 610
-// -> 459 (one tile, third stage), of 1280 x 720 2,950 -> 2,740; a nested
-// (64,2) > (128,2) > (256,2) frame of 139^2 rays 624 -> 512, of 512^2 1,120 ->
-// 1,060.  At width 256 the two tiles' MMAs and epilogues still take turns, and
+// What it measured (one call, us, before -> after): a 128 x 128 trace of the
+// Lipschitz-stepped (64,1) 159 .. 191 -> 80; the plain (256,3) trace of 100^2 rays
+// 822 -> 461 (one tile, third stage), of 1280 x 720 2,704 -> 2,492; a nested (64,2) > (128,2) > (256,2) frame of 150^2 rays 700 -> 554, of
+// 512^2 1,046 -> 999.  At width 256 the two tiles' MMAs and epilogues still take turns, and
 // a lone tile waits for its weights (9 k clocks a layer with two stages).
 // Handing the rays left at the end of a level to a second, one-tile launch was
 // tried: 3 % faster on the plain 1280 x 720 trace, 6 to 20 % slower on the
